@@ -29,6 +29,8 @@ SOURCES = [
     "kernels_query_grad.cu",
     "kernels_image.cu",
     "kernels_tc.cu",
+    "kernels_tree.cu",
+    "kernels_prune.cu",
     "zoom_noalloc.cu",
     "kernels_backward.cu",
     "zoom_api_backward.cu",
@@ -36,7 +38,8 @@ SOURCES = [
     "zoom_sample.cu",
     "zoom_random.cu",
 ]
-HEADERS = ["zoom_internal.h", "device_common.cuh", "knn_kernels.cuh"]
+HEADERS = ["zoom_internal.h", "device_common.cuh", "knn_kernels.cuh", "tc_ptx.cuh", "warp_select.cuh",
+           "search_tree.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -35,6 +35,8 @@
 #include <type_traits>
 
 #include "device_common.cuh"
+#include "tc_ptx.cuh"
+#include "warp_select.cuh"
 #include "zoom_internal.h"
 
 namespace {
@@ -85,212 +87,6 @@ __host__ __device__ constexpr int tc_stages(int KC, int MC) {
 static_assert(tc_stages(4, 16) == 16 && tc_stages(8, 16) == 10 && tc_stages(8, 32) == 10 &&
                   tc_stages(10, 16) == 7 && tc_stages(20, 16) == 3,
               "ring depths");
-constexpr uint32_t kWaitNs = 2000000000u;   // 2 s bound on any single wait
-
-// ---------------------------------------------------------------------------
-// PTX wrappers
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ uint64_t globaltimer() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
-               "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}\n"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// As mbar_try_wait, but the thread may sleep in hardware until the phase
-// completes or about `hint_ns` pass, instead of re-issuing polls.
-__device__ __forceinline__ bool mbar_try_wait_sleep(uint64_t* bar, uint32_t parity, uint32_t hint_ns) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}\n"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity), "r"(hint_ns)
-      : "memory");
-  return ok != 0;
-}
-
-// Waits for the phase of `parity` to complete.  Gives up after limit_ns
-// (kWaitNs unless the context set another limit; or 2^30 polls), or as soon
-// as another role gave up: then it raises the shared abort flag, records
-// ZOOM_ERR_TIMEOUT in the status word and returns false.
-__device__ __noinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
-                                       unsigned int* status, uint64_t limit_ns) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = globaltimer();
-  for (uint32_t it = 0; it < (1u << 30); ++it) {
-    if (mbar_try_wait_sleep(bar, parity, 1000000u)) return true;
-    if (*abort_flag) return false;
-    if (globaltimer() - t0 > limit_ns) break;
-  }
-  *abort_flag = 1;
-  atomicExch(status, 1u);
-  return false;
-}
-// Non-blocking poll of the phase of `parity`.
-__device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}\n"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// The common case inline: a short spin of non-blocking polls, then the
-// bounded slow path.  A thread suspended in try_wait resumes noticeably later
-// than a polling one sees the phase complete; on the filter's hand-offs
-// (accumulator full / free, a few hundred cycles apart) the spin takes about
-// 15 % off the step.
-constexpr int kSpinPolls = 32;
-__device__ __forceinline__ bool mbar_wait_fast(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
-                                               unsigned int* status, uint64_t limit_ns) {
-  for (int i = 0; i < kSpinPolls; ++i)
-    if (mbar_test_wait(bar, parity)) return true;
-  return mbar_wait(bar, parity, abort_flag, status, limit_ns);
-}
-// Before a CTA exits, also after an abort: waits for an asynchronous
-// operation it started (a bulk copy, or the MMAs a commit tracks) to signal
-// its barrier, whatever the abort flag says, for at most kWaitNs.
-__device__ __noinline__ bool mbar_drain(uint64_t* bar, uint32_t parity, unsigned int* status) {
-  const uint64_t t0 = globaltimer();
-  for (uint32_t it = 0; it < (1u << 30); ++it) {
-    if (mbar_try_wait_sleep(bar, parity, 100000u)) return true;
-    if (globaltimer() - t0 > kWaitNs) break;
-  }
-  atomicExch(status, 1u);
-  return false;
-}
-
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-          smem_u32(dst)),
-      "l"(src), "r"(bytes), "r"(smem_u32(bar))
-      : "memory");
-}
-
-__device__ __forceinline__ void tmem_alloc(uint32_t* slot, uint32_t ncols) {
-  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)),
-               "r"(ncols)
-               : "memory");
-}
-__device__ __forceinline__ void tmem_relinquish() {
-  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
-  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() {
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void tc_fence_after() {
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-}
-
-// D[tmem] (+)= A[smem] * B[smem]^T, M = N = 128, kind::f16 (fp16 or bf16 in,
-// fp32 accumulate).
-__device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                        uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                   smem_u32(bar))
-               : "memory");
-}
-
-// Issues the load of 32 consecutive TMEM columns of this warp's 32 lanes
-// (one lane per thread) into `v`, and `m` receives the minimum of the 32
-// values, reduced in the TMEM load path (tcgen05.ld.red, sm_103a): the
-// threshold test of a chunk costs one comparison instead of a min tree on the
-// 16-lane ALU pipe.  The registers are valid after tmem_ld_wait.
-__device__ __forceinline__ void tmem_ld32_min_issue(uint32_t taddr, float (&v)[32], float& m) {
-  uint32_t* r = reinterpret_cast<uint32_t*>(v);
-  asm volatile(
-      "tcgen05.ld.red.sync.aligned.32x32b.x32.min.f32 "
-      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, %32, [%33];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]),
-        "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]),
-        "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]), "=f"(m)
-      : "r"(taddr)
-      : "memory");
-}
-// Waits for the TMEM loads in flight; `v` and `m` (the destinations of the
-// last one) are in-out operands, so the compiler reads those registers only
-// after the wait and may do other work between the load and the wait.
-__device__ __forceinline__ void tmem_ld_wait(float (&v)[32], float& m) {
-  uint32_t* r = reinterpret_cast<uint32_t*>(v);
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]),
-                 "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]),
-                 "+r"(r[14]), "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]),
-                 "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]),
-                 "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31]), "+f"(m)
-               :
-               : "memory");
-}
-
-// After a tcgen05.wait::ld that covered the load into `v` and `m`: tells the
-// compiler those registers are valid from here on (no instruction).
-__device__ __forceinline__ void tmem_regs_ready(float (&v)[32], float& m) {
-  uint32_t* r = reinterpret_cast<uint32_t*>(v);
-  asm volatile(""
-               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]),
-                 "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]),
-                 "+r"(r[14]), "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]),
-                 "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]),
-                 "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31]), "+f"(m)
-               :
-               : "memory");
-}
-
-// Shared-memory matrix descriptor, K-major, no swizzle: core matrices of
-// 8 rows x 16 bytes stored as 128 contiguous bytes; `lbo` = byte distance
-// between core matrices adjacent along K, `sbo` = along M/N.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
-  d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
-  d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
-  d |= (uint64_t)1 << 46;  // descriptor version of sm_100-family tcgen05
-  return d;                // base offset 0, absolute LBO mode, no swizzle
-}
-
 // Instruction descriptor of kind::f16: D fp32, A and B of the same type
 // (fp16: 0, bf16: 1), both K-major, M = N = 128.
 __host__ __device__ constexpr uint32_t instr_desc(uint32_t ab_type) {
@@ -321,6 +117,14 @@ struct TcArgs {
   // nq_dev != nullptr: only the first min(*nq_dev, nq) queries are searched
   // (a count written by an earlier kernel); nq stays the lists' row stride
   const unsigned long long* nq_dev;
+  // part_d / part_id (with nq_dev): room for 2 * gridDim.x parts of 256
+  // queries' lists.  Where the count is small the dictionary part of a list
+  // is cut into fan_out() equal pieces, each with lists of its own there,
+  // and k_merge_parts joins them: a few hundred queries would otherwise
+  // leave most SMs idle (124 queries, 1M entries, 8 parts: 475 us on 8 SMs,
+  // 55 us so).
+  float* part_d = nullptr;
+  int32_t* part_id = nullptr;
   // bound on every wait (ns), and the testing aid: inject == 1 makes each
   // CTA's epilogue withhold the release of its accumulators from the third
   // tile of its first item on, so the issuing threads' waits run out
@@ -329,6 +133,10 @@ struct TcArgs {
   // packed chunk lists (the BF16 form of the wide-step filter): bits of a
   // list key that hold the chunk number
   int id_bits;
+  // wide-step filter over a step list: pair qp's step t is the dictionary
+  // step step_tiles[qp * nd_tiles + t] (nullptr: step t itself); the chunk
+  // numbers written are then those of the list
+  const int32_t* step_tiles = nullptr;
 };
 
 // Queries searched: nq, or the device count when one is given (read where
@@ -337,6 +145,16 @@ __device__ __forceinline__ int64_t searched_queries(const TcArgs& a) {
   if (!a.nq_dev) return a.nq;
   const int64_t c = (int64_t)*a.nq_dev;
   return c < a.nq ? c : a.nq;
+}
+
+// Pieces per list of a search over a device count of `pairs` query pairs: the
+// largest power of two (at most 16) that still gives every CTA of `grid` two
+// items at most, so that the pieces' lists fit the 2 * grid places of
+// part_d; 1 = no pieces.
+__device__ __forceinline__ int fan_out(int pairs, int nsplit, int grid) {
+  int m = 1;
+  while (m < 16 && pairs * nsplit * 2 * m <= 2 * grid) m *= 2;
+  return m;
 }
 
 // The work items of one CTA, in order; every role walks the same sequence.
@@ -363,16 +181,38 @@ struct WorkIter {
       }
     } else {
       const int item = c + k * G;
-      if (item >= a.nsplit * nq_pairs) return false;
+      const int m = a.part_d ? fan_out(nq_pairs, a.nsplit, G) : 1;
+      if (item >= a.nsplit * m * nq_pairs) return false;
       seg = item / nq_pairs;
       qp = item % nq_pairs;
-      t0 = seg * a.tiles_per_split;
+      const int s = seg / m, j = seg - s * m;   // piece j of list s
+      t0 = s * a.tiles_per_split;
       t1 = min(a.nd_tiles, t0 + a.tiles_per_split);
+      if (m > 1) {
+        const int n = t1 - t0;
+        t1 = t0 + (int)((int64_t)n * (j + 1) / m);
+        t0 += (int)((int64_t)n * j / m);
+      }
     }
     ++k;
     return true;
   }
 };
+
+// Where list `seg` of query q goes.
+__device__ __forceinline__ int64_t list_row(const TcArgs& a, int seg, int64_t q, float*& d, int32_t*& id) {
+  d = a.out_d;
+  id = a.out_id;
+  if (a.part_d) {
+    const int pairs = (int)((searched_queries(a) + 2 * TC_ROWS - 1) / (2 * TC_ROWS));
+    if (fan_out(pairs, a.nsplit, gridDim.x) > 1) {
+      d = a.part_d;
+      id = a.part_id;
+      return (int64_t)seg * pairs * (2 * TC_ROWS) + q;
+    }
+  }
+  return (int64_t)seg * a.nq + q;
+}
 
 // Inserts (v, id) into the ascending list, dropping its last entry; nothing
 // changes when v >= ld[MC-1].  Selects only, no branches: the lanes of a
@@ -391,8 +231,6 @@ __device__ __forceinline__ void list_push(float (&ld)[MC], int (&li)[MC], float 
   ld[0] = first ? v : ld[0];
   li[0] = first ? id : li[0];
 }
-
-constexpr unsigned kFull = 0xffffffffu;
 
 template <int MC>
 __device__ __forceinline__ void flush_appends(float (&ld)[MC], int (&li)[MC], float& thr,
@@ -688,8 +526,11 @@ __global__ void __maxnreg__(tc_max_regs(KC, MC)) k_knn_tc(TcArgs a) {
       if (!ok) break;
       flush();
       if (valid) {
-        float* od = a.out_d + ((int64_t)split * a.nq + q) * MC;
-        int32_t* oi = a.out_id + ((int64_t)split * a.nq + q) * MC;
+        float* od;
+        int32_t* oi;
+        const int64_t lrow = list_row(a, split, q, od, oi);
+        od += lrow * MC;
+        oi += lrow * MC;
 #pragma unroll
         for (int j = 0; j < MC; ++j) {
           const bool real = li[j] >= 0 && (int64_t)li[j] * 32 < a.nd;
@@ -712,6 +553,7 @@ __global__ void __maxnreg__(tc_max_regs(KC, MC)) k_knn_tc(TcArgs a) {
     }
   }
   tc_fence_before();
+  __syncwarp();   // the issuing and producing lanes rejoin their warps before the block's barrier
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
@@ -969,7 +811,8 @@ __global__ void __launch_bounds__(352, 1) k_knn_tw(TcArgs a) {
         for (int t = t0; t < t1; ++t) {
           if (!mbar_wait_fast(b_empty + stage, phase ^ 1u, abort_flag, a.status, a.wait_ns)) break;
           mbar_arrive_expect_tx(b_full + stage, kStep);
-          bulk_g2s(sB + stage * kStep, (const unsigned char*)a.dop + (size_t)t * kStep, kStep, b_full + stage);
+          const size_t step = a.step_tiles ? (size_t)a.step_tiles[(size_t)qp * a.nd_tiles + t] : (size_t)t;
+          bulk_g2s(sB + stage * kStep, (const unsigned char*)a.dop + step * kStep, kStep, b_full + stage);
           ++b_copies;
           if (++stage == kStages) {
             stage = 0;
@@ -1064,7 +907,7 @@ __global__ void __launch_bounds__(352, 1) k_knn_tw(TcArgs a) {
       if (__any_sync(kFull, *abort_flag != 0)) break;   // warp-uniform exit
       const bool withhold = a.inject == 1 && item_no++ == 0;   // testing aid (see TcArgs)
       const int64_t q = ((int64_t)qp * 2 + qt) * TC_ROWS + row;
-      const bool valid = q < a.nq;
+      const bool valid = q < searched_queries(a);
       const float qn = valid ? a.qn[q] : 0.f;
       if constexpr (PACKED) L.qn = qn;
       L.init();
@@ -1116,7 +959,10 @@ __global__ void __launch_bounds__(352, 1) k_knn_tw(TcArgs a) {
       if (!ok) break;
       L.flush();
       if (valid) {
-        L.write(qn, a.nd, a.out_d + ((int64_t)split * a.nq + q) * MC, a.out_id + ((int64_t)split * a.nq + q) * MC);
+        float* od;
+        int32_t* oi;
+        const int64_t lrow = list_row(a, split, q, od, oi);
+        L.write(qn, a.nd, od + lrow * MC, oi + lrow * MC);
         if (a.tail_split > 0 && t0 == 0 && t1 == a.nd_tiles) {
           for (int s2 = 1; s2 < a.tail_split; ++s2) {
             float* od1 = a.out_d + ((int64_t)s2 * a.nq + q) * MC;
@@ -1132,10 +978,44 @@ __global__ void __launch_bounds__(352, 1) k_knn_tw(TcArgs a) {
     }
   }
   tc_fence_before();
+  __syncwarp();   // the issuing and producing lanes rejoin their warps before the block's barrier
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem, 512);
+  }
+}
+
+// The pieces' lists of a search with fan_out() > 1 joined: a warp per query
+// and list keeps the MC smallest (d~, chunk) of its pieces' lists, which is
+// the list one piece would have written (equal d~ keep the lower chunk there
+// too).
+template <int MC>
+__global__ void __launch_bounds__(128) k_merge_parts(const unsigned long long* __restrict__ nq_dev, int64_t nq,
+                                                     int nsplit, int grid, const float* __restrict__ part_d,
+                                                     const int32_t* __restrict__ part_id, float* __restrict__ out_d,
+                                                     int32_t* __restrict__ out_id) {
+  const int64_t n = (int64_t)*nq_dev < nq ? (int64_t)*nq_dev : nq;
+  const int pairs = (int)((n + 2 * TC_ROWS - 1) / (2 * TC_ROWS));
+  const int m = fan_out(pairs, nsplit, grid);
+  if (m == 1) return;
+  const int lane = threadIdx.x & 31;
+  const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t q = w / nsplit;
+  const int s = (int)(w % nsplit);
+  if (q >= n) return;   // warp-uniform
+  float bd = FLT_MAX;
+  int bi = INT_MAX;
+  for (int j = 0; j < m; ++j) {
+    const int64_t o = (((int64_t)s * m + j) * pairs * (2 * TC_ROWS) + q) * MC + lane;
+    const float v = lane < MC ? part_d[o] : FLT_MAX;
+    const int id = v < FLT_MAX ? part_id[o] : INT_MAX;
+    warp_merge_best(bd, bi, v, id, MC, lane);
+  }
+  if (lane < MC) {
+    const int64_t o = ((int64_t)s * nq + q) * MC + lane;
+    out_d[o] = bd;
+    out_id[o] = bi == INT_MAX ? -1 : bi;
   }
 }
 
@@ -1321,78 +1201,6 @@ __global__ void k_operand_f16s(const float* __restrict__ feat, int dpad, int64_t
 // threshold over the splits), so T - delta > D_K proves the result; a query
 // it cannot settle is flagged for the SIMT re-run.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ bool lex_less(float a, int ai, float b, int bi) {
-  return a < b || (a == b && ai < bi);
-}
-
-// Bitonic sort of one (value, ID) pair per lane, ascending across the lanes.
-__device__ __forceinline__ void warp_sort32(float& v, int& id, int lane) {
-#pragma unroll
-  for (int k = 2; k <= 32; k <<= 1) {
-#pragma unroll
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      const float ov = __shfl_xor_sync(kFull, v, j);
-      const int oi = __shfl_xor_sync(kFull, id, j);
-      const bool keep_small = ((lane & j) == 0) == ((lane & k) == 0);
-      if (keep_small == lex_less(ov, oi, v, id)) {
-        v = ov;
-        id = oi;
-      }
-    }
-  }
-}
-
-// Merges 32 ascending candidates (one per lane) into the ascending K best
-// held by lanes 0..K-1: min(A[j], B[31 - j]) is a bitonic sequence holding
-// the 32 smallest of both, which a bitonic merge sorts.
-__device__ __forceinline__ void warp_merge_best(float& bd, int& bi, float v, int id, int K, int lane) {
-  float a = lane < K ? bd : FLT_MAX;
-  int ai = lane < K ? bi : INT_MAX;
-  const float rb = __shfl_sync(kFull, v, 31 - lane);
-  const int rbi = __shfl_sync(kFull, id, 31 - lane);
-  if (lex_less(rb, rbi, a, ai)) {
-    a = rb;
-    ai = rbi;
-  }
-#pragma unroll
-  for (int j = 16; j > 0; j >>= 1) {
-    const float ov = __shfl_xor_sync(kFull, a, j);
-    const int oi = __shfl_xor_sync(kFull, ai, j);
-    if (((lane & j) == 0) == lex_less(ov, oi, a, ai)) {
-      a = ov;
-      ai = oi;
-    }
-  }
-  bd = a;
-  bi = ai;
-}
-
-// t-of-L membership: at least tmin of the entry's L bucket keys equal the
-// query's.  Eight tables at a time (loads issued together); stops at tmin
-// hits.
-__device__ __forceinline__ bool lsh_member(const uint64_t* __restrict__ dk, const uint64_t* qk, int L,
-                                           int tmin) {
-  int hits = 0;
-  for (int l0 = 0; l0 < L && hits < tmin; l0 += 8) {
-    uint64_t kk[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) kk[j] = l0 + j < L ? __ldg(dk + l0 + j) : 0ull;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) hits += (l0 + j < L && kk[j] == qk[l0 + j]) ? 1 : 0;
-  }
-  return hits >= tmin;
-}
-
-__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(smem_dst)), "l"(gmem_src)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
 // queries (warps) per block: the staged rows of wide features (D = 50, two
 // buffers of 32 rows of 52 floats per warp) would exceed 48 KB of static
 // shared memory at four warps.  Seven blocks of four warps fill the shared
@@ -1741,21 +1549,61 @@ static cudaError_t run_tc_kernel(const TcArgs& args, int grid, size_t smem, cuda
   return cudaGetLastError();
 }
 
+struct TcParts {
+  float* d = nullptr;
+  int32_t* id = nullptr;
+};
+static cudaError_t knn_tc(const uint16_t* qop, const float* qn, int64_t nq, const uint16_t* dop, int64_t nd,
+                          int precision, int kc, int MC, int nsplit, int tail_split, int grid, float* out_d,
+                          int32_t* out_id, unsigned int* status, cudaStream_t st, const unsigned long long* nq_dev,
+                          uint64_t wait_ns, int inject, const TcParts& parts);
+
+int64_t tc_part_floats(int grid, int MC) { return (int64_t)2 * grid * 2 * TC_ROWS * MC; }
+
 cudaError_t launch_knn_tc(const uint16_t* qop, const float* qn, int64_t nq, const uint16_t* dop,
                           int64_t nd, int precision, int kc, int MC, int nsplit, int tail_split, int grid,
                           float* out_d, int32_t* out_id, unsigned int* status, cudaStream_t st,
-                          const unsigned long long* nq_dev, uint64_t wait_ns, int inject) {
+                          const unsigned long long* nq_dev, uint64_t wait_ns, int inject, float* part_d,
+                          int32_t* part_id) {
+  if (part_d) {
+    if (!nq_dev || tail_split > 0) return cudaErrorInvalidValue;
+    TcParts parts{part_d, part_id};
+    cudaError_t e = knn_tc(qop, qn, nq, dop, nd, precision, kc, MC, nsplit, 0, grid, out_d, out_id, status, st, nq_dev,
+                           wait_ns, inject, parts);
+    if (e != cudaSuccess) return e;
+    // a grid smaller than the items' count means every item has a CTA; the
+    // kernel's own grid decides the pieces
+    const int64_t pairs = (nq + 2 * TC_ROWS - 1) / (2 * TC_ROWS);
+    const int g = (int)(grid < nsplit * pairs ? grid : nsplit * pairs);
+    // fan_out() > 1 needs pairs * nsplit <= g: at most that many lists to join
+    const int64_t lists = std::min<int64_t>((int64_t)g * 2 * TC_ROWS, nq * nsplit);
+    if (MC == 16)
+      k_merge_parts<16><<<(unsigned)((lists + 3) / 4), 128, 0, st>>>(nq_dev, nq, nsplit, g, part_d, part_id, out_d, out_id);
+    else
+      k_merge_parts<32><<<(unsigned)((lists + 3) / 4), 128, 0, st>>>(nq_dev, nq, nsplit, g, part_d, part_id, out_d, out_id);
+    return cudaGetLastError();
+  }
+  return knn_tc(qop, qn, nq, dop, nd, precision, kc, MC, nsplit, tail_split, grid, out_d, out_id, status, st, nq_dev,
+                wait_ns, inject, TcParts{});
+}
+
+static cudaError_t knn_tc(const uint16_t* qop, const float* qn, int64_t nq, const uint16_t* dop, int64_t nd,
+                          int precision, int kc, int MC, int nsplit, int tail_split, int grid, float* out_d,
+                          int32_t* out_id, unsigned int* status, cudaStream_t st, const unsigned long long* nq_dev,
+                          uint64_t wait_ns, int inject, const TcParts& parts) {
   if (tc_wide_form(precision, kc)) {
     // the wide-step kernel: items of 256 queries x a part of the 256-row steps
-    if (nq_dev || (MC != 16 && MC != 32)) return cudaErrorInvalidValue;
+    if ((nq_dev && tail_split > 0) || (MC != 16 && MC != 32)) return cudaErrorInvalidValue;
     TcArgs a;
+    a.part_d = parts.d;
+    a.part_id = parts.id;
     a.wait_ns = wait_ns > 0 ? wait_ns : kWaitNs;
     a.inject = inject;
     a.qop = qop;
     a.qn = qn;
     a.dop = dop;
     a.nq = nq;
-    a.nq_dev = nullptr;
+    a.nq_dev = nq_dev;
     a.nd = nd;
     a.nq_pairs = (int)((nq + 2 * TC_ROWS - 1) / (2 * TC_ROWS));
     a.nd_tiles = (int)((nd + TW_ROWS - 1) / TW_ROWS);   // 256-row steps
@@ -1789,6 +1637,8 @@ cudaError_t launch_knn_tc(const uint16_t* qop, const float* qn, int64_t nq, cons
     return cudaErrorInvalidValue;
   }
   TcArgs a;
+  a.part_d = parts.d;
+  a.part_id = parts.id;
   a.wait_ns = wait_ns > 0 ? wait_ns : kWaitNs;
   a.inject = inject;
   a.qop = qop;
@@ -1824,6 +1674,37 @@ cudaError_t launch_knn_tc(const uint16_t* qop, const float* qn, int64_t nq, cons
   return cudaErrorInvalidValue;
 }
 
+cudaError_t launch_knn_seeds(const uint16_t* qop, const float* qn, int64_t nq, const uint16_t* dop, int64_t nd,
+                             int precision, int kc, int MC, const int32_t* seeds, int grid, float* out_d,
+                             int32_t* out_id, unsigned int* status, cudaStream_t st, uint64_t wait_ns, int inject) {
+  TcArgs a{};
+  a.wait_ns = wait_ns > 0 ? wait_ns : kWaitNs;
+  a.inject = inject;
+  a.qop = qop;
+  a.qn = qn;
+  a.dop = dop;
+  a.nq = nq;
+  a.nd = nd;
+  a.nq_pairs = (int)((nq + 2 * TC_ROWS - 1) / (2 * TC_ROWS));
+  a.nd_tiles = kPruneSeeds;
+  a.nsplit = 1;
+  a.tiles_per_split = kPruneSeeds;
+  a.out_d = out_d;
+  a.out_id = out_id;
+  a.status = status;
+  a.step_tiles = seeds;
+  grid = grid < a.nq_pairs ? grid : a.nq_pairs;
+#define ZOOM_TW(KC, T) \
+  return MC == 16 ? run_tw_kernel<KC, 16, T, false>(a, grid, st) : run_tw_kernel<KC, 32, T, false>(a, grid, st)
+  if (MC != 16 && MC != 32) return cudaErrorInvalidValue;
+  if (precision == 2 && kc == 4) ZOOM_TW(4, 0);
+  if (precision == 2 && kc == 8) ZOOM_TW(8, 0);
+  if (precision == 1 && kc == 4) ZOOM_TW(4, 1);
+  if (precision == 1 && kc == 8) ZOOM_TW(8, 1);
+#undef ZOOM_TW
+  return cudaErrorInvalidValue;
+}
+
 template <int D, int MC>
 static cudaError_t rerank_k(int K, const float* qfeat, int dpad, const float* qn, const uint64_t* qkeys,
                             int64_t nq, const float* dfeat, const uint64_t* dkeys, int64_t nd, int L,
@@ -1839,6 +1720,31 @@ static cudaError_t rerank_k(int K, const float* qfeat, int dpad, const float* qn
   return cudaGetLastError();
 }
 
+FilterError tc_filter_error(int d, int precision) {
+  // |d~ - d| <= c_qr ||q|| r + c_sq (r^2 + ||q||^2) + c_abs (||q|| + r)
+  // + c_rel d for an entry with ||c|| <= r.  precision 0 (FP16 hi/lo split): the
+  // dropped q_lo.c_lo term and the rounding of the split, within
+  // 6 * 2^-16 ||q|| r, FP32 accumulation of 80 terms and the FP32 rerank
+  // (2^-16 (r^2 + ||q||^2), 4e-6 d).  2 (one FP16 term): q and c each
+  // rounded to 11 significant bits, 2 (2^-10 + 2^-22) ||q|| r for the
+  // product term (Cauchy-Schwarz), 1.05 * 2^-9 with the accumulation of 32
+  // terms.  Both: FP16 subnormals round with an absolute error up to 2^-25
+  // per element, 2 * 2^-25 * sum(|q_i| + |c_i|) <= 2^-23 sqrt(D) (||q|| + r)
+  // with slack.  1 (BF16): each operand rounded to 8 significant bits
+  // (2 * 2^-8 ||q|| r for the product term), 32 FP32 accumulations; used only
+  // to stop examining (no proof).  Twice the operand width (gradient
+  // features of 5 x 5 patches, K = 160 or 64) doubles the accumulation
+  // terms: the coefficients are doubled (the kernel doubles the relative
+  // term of its FP32 rerank for D > 25 too).
+  const float wide = tc_kc(d, precision) > (precision == 0 ? 10 : 4) ? 2.f : 1.f;
+  FilterError fe;
+  fe.c_qr = wide * (precision == 0 ? 6.f / 65536.f : precision == 2 ? 1.05f / 512.f : 1.05f / 128.f);
+  fe.c_sq = wide * (precision == 1 ? 1.f / 262144.f : 1.f / 65536.f);
+  fe.c_abs = 1.1920929e-07f * sqrtf((float)d);   // 2^-23 sqrt(D)
+  fe.c_rel = d > 25 ? 8e-6f : 4e-6f;
+  return fe;
+}
+
 cudaError_t launch_rerank(int d, int MC, int K, const float* qfeat, int dpad, const float* qn,
                           const uint64_t* qkeys, int64_t nq, const float* dfeat, const uint64_t* dkeys,
                           int64_t nd, int L, int tmin, const float* ld, const int32_t* li, int nsplit,
@@ -1847,26 +1753,8 @@ cudaError_t launch_rerank(int d, int MC, int K, const float* qfeat, int dpad, co
   if (nsplit > 8 || K < 1 || K > 16 || dpad != (d + 3) / 4 * 4 || form < 0 || form > 2)
     return cudaErrorInvalidValue;
   if (nq == 0) return cudaSuccess;
-  // |d~ - d| <= c_qr ||q|| r + c_sq (r^2 + ||q||^2) + c_abs (||q|| + r)
-  // + 4e-6 d for an entry with ||c|| <= r.  form 1 (FP16 hi/lo split): the
-  // dropped q_lo.c_lo term and the rounding of the split, within
-  // 6 * 2^-16 ||q|| r, FP32 accumulation of 80 terms and the FP32 rerank
-  // (2^-16 (r^2 + ||q||^2), 4e-6 d).  form 2 (one FP16 term): q and c each
-  // rounded to 11 significant bits, 2 (2^-10 + 2^-22) ||q|| r for the
-  // product term (Cauchy-Schwarz), 1.05 * 2^-9 with the accumulation of 32
-  // terms.  Both: FP16 subnormals round with an absolute error up to 2^-25
-  // per element, 2 * 2^-25 * sum(|q_i| + |c_i|) <= 2^-23 sqrt(D) (||q|| + r)
-  // with slack.  form 0 (BF16): each operand rounded to 8 significant bits
-  // (2 * 2^-8 ||q|| r for the product term), 32 FP32 accumulations; used only
-  // to stop examining (no proof).  Twice the operand width (gradient
-  // features of 5 x 5 patches, K = 160 or 64) doubles the accumulation
-  // terms: the coefficients are doubled (the kernel doubles the relative
-  // term of its FP32 rerank for D > 25 too).
-  const int prec = form == 1 ? 0 : (form == 0 ? 1 : 2);
-  const float wide = tc_kc(d, prec) > (prec == 0 ? 10 : 4) ? 2.f : 1.f;
-  const float c_qr = wide * (form == 1 ? 6.f / 65536.f : form == 2 ? 1.05f / 512.f : 1.05f / 128.f);
-  const float c_sq = wide * (form == 0 ? 1.f / 262144.f : 1.f / 65536.f);
-  const float c_abs = 1.1920929e-07f * sqrtf((float)d);   // 2^-23 sqrt(D)
+  const FilterError fe = tc_filter_error(d, form == 1 ? 0 : (form == 0 ? 1 : 2));
+  const float c_qr = fe.c_qr, c_sq = fe.c_sq, c_abs = fe.c_abs;
   const int exact = form != 0;
 #define ZOOM_RR(DD, MM)                                                                          \
   return rerank_k<DD, MM>(K, qfeat, dpad, qn, qkeys, nq, dfeat, dkeys, nd, L, tmin, ld, li, nsplit, \

@@ -415,6 +415,25 @@ zoom_status zoom_build_index(zoom_dict d, const zoom_lsh_params* lsh, const floa
   ix->proj_dist = drawn_a.empty() ? 0 : lsh->proj_dist;
   ix->seed = drawn_a.empty() ? 0 : lsh->seed;
   ix->nd_rows = tc_rows_padded(N, true);   // whole 256-row steps for the wide-step filter
+  // the search order (a capped index walks its bins and never searches densely)
+  if (ix->cap == 0 && N >= kPruneMinEntries && N <= kPruneMaxEntries) {
+    ix->tree_tiles = (N + 255) / 256;
+    tree_depths(N, &ix->tree_d1, &ix->tree_d2);
+  }
+  const int64_t nt = ix->tree_tiles, ns = (nt + 15) / 16;
+  auto carve_tree = [&](Carver& c) {
+    if (!nt) return;
+    ix->tree_basis = c.take<float>((size_t)d->d * 16);
+    ix->tree_node1 = c.take<uint64_t>((size_t)1 << ix->tree_d1);
+    ix->tree_node2 = c.take<uint64_t>((size_t)1 << (ix->tree_d1 + ix->tree_d2));
+    ix->tree_order = c.take<int32_t>(N);
+    ix->tree_f1 = c.take<uint16_t>(nt * 256 * tc_kc(d->d, 2) * 8);
+    ix->tree_bf = c.take<uint16_t>(nt * 256 * tc_kc(d->d, 1) * 8);
+    ix->tree_box = c.take<char>(nt * 64);
+    ix->tree_sbox = c.take<char>(ns * 64);
+    ix->tree_mid = c.take<float>(nt * 16);
+    ix->tree_smid = c.take<float>(ns * 16);
+  };
   {
     Carver c(nullptr);
     c.take<float>((size_t)L * k * d->d);
@@ -427,6 +446,7 @@ zoom_status zoom_build_index(zoom_dict d, const zoom_lsh_params* lsh, const floa
     c.take<uint16_t>(ix->nd_rows * tc_kc(d->d, 0) * 8);
     c.take<uint16_t>(ix->nd_rows * tc_kc(d->d, 1) * 8);
     c.take<uint16_t>(ix->nd_rows * tc_kc(d->d, 2) * 8);
+    carve_tree(c);
     ix->bytes = c.off + 256;
   }
   void* mem = zoom_alloc(ctx, ix->bytes, st);
@@ -445,6 +465,7 @@ zoom_status zoom_build_index(zoom_dict d, const zoom_lsh_params* lsh, const floa
   ix->dop16 = c.take<uint16_t>(ix->nd_rows * tc_kc(d->d, 0) * 8);
   ix->dopbf = c.take<uint16_t>(ix->nd_rows * tc_kc(d->d, 1) * 8);
   ix->dopf1 = c.take<uint16_t>(ix->nd_rows * tc_kc(d->d, 2) * 8);
+  carve_tree(c);
   zoom_status rc = ZOOM_OK;
   cudaError_t e = cudaMemcpyAsync(ix->alpha, alpha, (size_t)L * k * d->d * 4, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(ix->beta, beta, (size_t)L * k * 4, cudaMemcpyHostToDevice, st);
@@ -458,11 +479,12 @@ zoom_status zoom_build_index(zoom_dict d, const zoom_lsh_params* lsh, const floa
     e = launch_operand(d->feat, d->dpad, d->d, N, ix->nd_rows, 1, 2, ix->dopf1, nullptr, st);
   if (e == cudaSuccess) {
     Scratch scr(ctx, st);
-    size_t sb = csr_build_scratch_bytes(N, L);
-    if (!scr.get(sb)) {
+    const size_t sb = csr_build_scratch_bytes(N, L), tb = nt ? tree_scratch_bytes(N) : 0;
+    if (!scr.get(std::max(sb, tb))) {   // one after the other on the stream
       rc = fail(ZOOM_ERR_OOM, "index build scratch");
     } else {
-      e = build_csr_tables(ix, scr.p, sb, st);
+      if (nt) e = build_search_tree(ix, scr.p, tb, st);
+      if (e == cudaSuccess) e = build_csr_tables(ix, scr.p, sb, st);
     }
     if (e == cudaSuccess && rc == ZOOM_OK) e = cudaStreamSynchronize(st);
   }
@@ -524,11 +546,39 @@ struct SearchPlan {
   // cap2) run again through the FP16-split filter, nsplit2 dictionary parts
   int64_t cap2 = 0, q_rows2 = 0;
   int MC2 = 16, nsplit2 = 1;
+  // search over the dictionary's search order; the queries it cannot prove
+  // go through the split filter: the first cap2 of them over nsplit2
+  // dictionary parts, the rest as one part, then the scan
+  bool pruned = false;
+  PrunePlan pp;
+  size_t tail_off = 0;   // workspace offset shared by the pruned search and the large split stage
   size_t bytes = 0;
 };
 
+// Scratch of the split filter on up to n queries (a compacted subset).
+struct SplitBufs {
+  float* feat;
+  uint64_t* keys;
+  uint16_t* qop;
+  float *qn, *ld, *pd;
+  int32_t *li, *pi;
+};
+SplitBufs take_split(Carver& c, zoom_index ix, int64_t n, int nsplit, int MC) {
+  zoom_dict d = ix->dict;
+  SplitBufs b;
+  b.feat = c.take<float>((size_t)n * d->dpad);
+  b.keys = c.take<uint64_t>((size_t)n * ix->L);
+  b.qop = c.take<uint16_t>((size_t)tc_rows_padded(n, true) * tc_kc(d->d, 0) * 8);
+  b.qn = c.take<float>(n);
+  b.ld = c.take<float>((size_t)nsplit * n * MC);
+  b.li = c.take<int32_t>((size_t)nsplit * n * MC);
+  b.pd = c.take<float>(tc_part_floats(d->ctx->n_sm, MC));
+  b.pi = c.take<int32_t>(tc_part_floats(d->ctx->n_sm, MC));
+  return b;
+}
+
 SearchPlan plan_search(zoom_index ix, const zoom_upscale_params* prm, int64_t nq, int nsplit_override,
-                       int mc_override) {
+                       int mc_override, bool may_prune = true) {
   zoom_dict d = ix->dict;
   SearchPlan p;
   if (ix->cap > 0) {
@@ -547,6 +597,25 @@ SearchPlan plan_search(zoom_index ix, const zoom_upscale_params* prm, int64_t nq
   p.prec = prm->precision == 1 ? 1 : (prm->search == 3 ? 0 : 2);
   p.MC = mc_override > 0 ? mc_override : tc_list_size(p.prec, prm->K, prm->rerank_mult);
   p.KCH = tc_kc(d->d, p.prec) * 8;
+  // automatic search and the precision form: over the search order where the
+  // dictionary has one
+  if (may_prune && prm->search == 0 && prm->precision == 0 && prune_plan(ix, p.prec, prm->K, nq, &p.pp)) {
+    p.pruned = true;
+    p.cap2 = std::min<int64_t>(nq, std::max<int64_t>(8192, nq / 64));
+    p.MC2 = tc_list_size(0, prm->K, prm->rerank_mult);
+    p.nsplit2 = (int)std::min<int64_t>(8, ix->nd_rows / 128);
+    Carver c(nullptr);
+    c.take<unsigned long long>(4);
+    c.take<int32_t>(nq);
+    c.take<int32_t>(nq);
+    c.take<int32_t>(nq);
+    take_split(c, ix, p.cap2, p.nsplit2, p.MC2);
+    p.tail_off = (c.off + 255) & ~(size_t)255;
+    Carver t(nullptr);
+    take_split(t, ix, nq, 1, p.MC2);
+    p.bytes = p.tail_off + std::max(prune_ws_bytes(ix, p.pp, nq), t.off) + 256;
+    return p;
+  }
   // the narrow forms step through the dictionary 256 rows at a time
   const int64_t unit_rows = tc_wide_form(p.prec, p.KCH / 8) ? 256 : 128;
   const int64_t nd_tiles = ix->nd_rows / unit_rows;
@@ -630,6 +699,28 @@ __global__ void k_add_fallback_counts(const unsigned long long* __restrict__ cnt
   counters[CNT_FALLBACK2] += cnt[1];
 }
 
+// The split filter on the queries listed in idx[0 .. *cnt) (at most cap of
+// them; the rest are appended to over / *over_cnt), over nsplit dictionary
+// parts; what its proof leaves joins left / *left_cnt.
+cudaError_t run_split_stage(zoom_index ix, const QueryBufs& q, int64_t nq, int K, int64_t cap, int nsplit, int MC,
+                            const SplitBufs& b, const int32_t* idx, const unsigned long long* cnt, int32_t* over,
+                            unsigned long long* over_cnt, int32_t* left, unsigned long long* left_cnt,
+                            cudaStream_t st) {
+  zoom_dict d = ix->dict;
+  zoom_ctx ctx = d->ctx;
+  cudaError_t e = launch_gather_queries(idx, cnt, nq, cap, q.feat, d->dpad, q.keys, ix->L, b.feat, b.keys, over,
+                                        over_cnt, st);
+  if (e == cudaSuccess)
+    e = launch_operand(b.feat, d->dpad, d->d, cap, tc_rows_padded(cap, true), 0, 0, b.qop, b.qn, st, cnt);
+  if (e == cudaSuccess)
+    e = launch_knn_tc(b.qop, b.qn, cap, ix->dop16, d->n, 0, tc_kc(d->d, 0), MC, nsplit, 0, ctx->n_sm, b.ld, b.li,
+                      ctx->d_status, st, cnt, ctx->wait_ns, ctx->inject, b.pd, b.pi);
+  if (e == cudaSuccess)
+    e = launch_rerank(d->d, MC, K, b.feat, d->dpad, b.qn, b.keys, cap, d->feat, ix->dkeys, d->n, ix->L, ix->t, b.ld,
+                      b.li, nsplit, 1, q.nbr, q.dist, left, left_cnt, st, idx, cnt);
+  return e;
+}
+
 // Neighbour search with a caller-provided workspace of plan.bytes: SIMT
 // scan, or the capped walk, or the tensor-core search in its stages (the
 // queries a stage leaves go to the next one, the lists counted in the
@@ -644,9 +735,34 @@ cudaError_t run_search_ws(zoom_index ix, const zoom_upscale_params* prm, const Q
     return launch_knn_exact(ix, b.feat, b.keys, nq, K, b.nbr, b.dist, ctx->d_counters, nullptr,
                             nullptr, st);
   Carver s2(ws);
-  unsigned long long* cnt = s2.take<unsigned long long>(2);   // [0] first list, [1] second
-  cudaError_t e = cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned long long), st);
+  // [0] first list, [1] second (pruned: [0] unproven, [1] left to the scan, [2] past cap2)
+  unsigned long long* cnt = s2.take<unsigned long long>(pl.pruned ? 4 : 2);
+  cudaError_t e = cudaMemsetAsync(cnt, 0, (pl.pruned ? 4 : 2) * sizeof(unsigned long long), st);
   if (e != cudaSuccess) return e;
+  if (pl.pruned) {
+    int32_t* fb = s2.take<int32_t>(nq);
+    int32_t* more = s2.take<int32_t>(nq);
+    int32_t* fb2 = s2.take<int32_t>(nq);
+    const SplitBufs sa = take_split(s2, ix, pl.cap2, pl.nsplit2, pl.MC2);
+    char* tail = (char*)ws + pl.tail_off;
+    e = run_pruned(ix, pl.pp, b.feat, b.keys, nq, K, b.nbr, b.dist, tail, fb, cnt, st);
+    if (e == cudaSuccess)
+      e = run_split_stage(ix, b, nq, K, pl.cap2, pl.nsplit2, pl.MC2, sa, fb, cnt, more, cnt + 2, fb2, cnt + 1, st);
+    // the pruned search's buffers are free now: the queries past cap2, as
+    // one dictionary part each
+    if (e == cudaSuccess && pl.cap2 < nq) {
+      Carver t(tail);
+      const SplitBufs sb = take_split(t, ix, nq, 1, pl.MC2);
+      e = run_split_stage(ix, b, nq, K, nq, 1, pl.MC2, sb, more, cnt + 2, nullptr, nullptr, fb2, cnt + 1, st);
+    }
+    if (e == cudaSuccess)
+      e = launch_knn_exact(ix, b.feat, b.keys, nq, K, b.nbr, b.dist, ctx->d_counters, fb2, cnt + 1, st);
+    if (e == cudaSuccess) {
+      k_add_fallback_counts<<<1, 1, 0, st>>>(cnt, ctx->d_counters);
+      e = cudaGetLastError();
+    }
+    return e;
+  }
   if (pl.capped) {
     int32_t* cand = s2.take<int32_t>((size_t)nq * ix->cap);
     int32_t* fb = s2.take<int32_t>(nq);
@@ -711,10 +827,15 @@ cudaError_t run_search_ws(zoom_index ix, const zoom_upscale_params* prm, const Q
 
 cudaError_t run_search(zoom_index ix, const zoom_upscale_params* prm, const QueryBufs& b, int64_t nq,
                        cudaStream_t st, bool& oom) {
-  const SearchPlan pl = plan_search(ix, prm, nq, 0, 0);
+  SearchPlan pl = plan_search(ix, prm, nq, 0, 0);
   if (!pl.tc && !pl.capped) return run_search_ws(ix, prm, b, nq, pl, nullptr, st);
   Scratch scr(ix->dict->ctx, st);
-  if (!scr.get(pl.bytes)) {
+  bool got = scr.get(pl.bytes);
+  if (!got && pl.pruned) {   // no room for the query lists: the dense search
+    pl = plan_search(ix, prm, nq, 0, 0, false);
+    got = scr.get(pl.bytes);
+  }
+  if (!got) {
     oom = true;
     return cudaSuccess;
   }
@@ -1246,7 +1367,8 @@ zoom_status zoom_upscale_batch(const zoom_index* ixs, int32_t n_indexes, int32_t
           return fail(ZOOM_ERR_CUDA, std::string("batch features: ") + cudaGetErrorString(e));
         }
       }
-      if (!g.images.empty() && plan_search(g.ix, prm, g.nq, 0, 0).tc) {
+      const SearchPlan first = plan_search(g.ix, prm, g.nq, 0, 0);
+      if (!g.images.empty() && first.tc && !first.pruned) {
         zoom_status rs = autotune_group(g, prm, st);
         if (rs != ZOOM_OK) {
           free_record(ctx, rec);
@@ -1254,17 +1376,25 @@ zoom_status zoom_upscale_batch(const zoom_index* ixs, int32_t n_indexes, int32_t
         }
       }
     }
-    // search scratch per group, with the tuned plan
+    // search scratch per group, with the tuned plan; without room for the
+    // query lists of the search order, the dense plan
     size_t extra = 0;
+    void* ws = nullptr;
     TuneMap& tm = *(TuneMap*)ctx->tuned;
-    for (auto& g : groups) {
-      if (g.images.empty()) continue;
-      const TuneKey tk{g.ix, qbucket(g.nq), prm->precision, prm->K};
-      const TuneChoice ch = tm.count(tk) ? tm[tk] : TuneChoice();
-      g.plan = plan_search(g.ix, prm, g.nq, ch.nsplit, ch.mc);
-      extra += (g.plan.bytes + 255) / 256 * 256;
+    for (const bool may_prune : {true, false}) {
+      extra = 0;
+      bool pruned = false;
+      for (auto& g : groups) {
+        if (g.images.empty()) continue;
+        const TuneKey tk{g.ix, qbucket(g.nq), prm->precision, prm->K};
+        const TuneChoice ch = tm.count(tk) ? tm[tk] : TuneChoice();
+        g.plan = plan_search(g.ix, prm, g.nq, ch.nsplit, ch.mc, may_prune);
+        pruned = pruned || g.plan.pruned;
+        extra += (g.plan.bytes + 255) / 256 * 256;
+      }
+      ws = extra ? zoom_alloc(ctx, extra, st) : nullptr;
+      if (ws || !extra || !pruned) break;
     }
-    void* ws = extra ? zoom_alloc(ctx, extra, st) : nullptr;
     if (extra && !ws) {
       free_record(ctx, rec);
       return fail(ZOOM_ERR_OOM, "batch search workspace");

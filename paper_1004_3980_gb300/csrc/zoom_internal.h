@@ -83,6 +83,21 @@ struct zoom_index_s {
   uint16_t* dopbf = nullptr; // BF16 single term, tc_kc(d, 1) chunks of 8 per row
   uint16_t* dopf1 = nullptr; // FP16 single term, tc_kc(d, 2) chunks of 8 per row
   int64_t nd_rows = 0;       // rows of the operands (N rounded up to 128)
+  // search order (kernels_tree.cu): entries sorted along a splitting tree in
+  // tiles of 256 with bounding boxes; tree_tiles 0: none (small, capped or
+  // very large dictionaries)
+  int64_t tree_tiles = 0;
+  int tree_d1 = 0, tree_d2 = 0;
+  float* tree_basis = nullptr;    // [d][16] bound coordinates z = B^T f
+  void* tree_node1 = nullptr;     // TreeNode [1 << d1]
+  void* tree_node2 = nullptr;     // TreeNode [1 << d1][1 << d2]
+  int32_t* tree_order = nullptr;  // [N] entry ID at each position of the order
+  uint16_t* tree_f1 = nullptr;    // single-term FP16 operand in search order
+  uint16_t* tree_bf = nullptr;    // BF16 operand in search order
+  void* tree_box = nullptr;       // [tiles] FP16 box (64 bytes)
+  void* tree_sbox = nullptr;      // [super tiles] the same
+  float* tree_mid = nullptr;      // [tiles][16] mean bound coordinates
+  float* tree_smid = nullptr;     // [super tiles][16]
   size_t bytes = 0;
 };
 
@@ -123,6 +138,16 @@ cudaError_t build_csr_tables(zoom_index ix, void* scratch, size_t scratch_bytes,
 size_t csr_scratch_bytes(int64_t n);
 // scratch of build_csr_tables: the radix sort's plus the key compaction's
 size_t csr_build_scratch_bytes(int64_t n, int L);
+
+// stable sort by 16-bit ranks below 2^bits
+size_t sort_rank16_scratch_bytes(int64_t n);
+cudaError_t sort_rank16(const uint16_t* rank, int64_t n, int bits, int32_t* ids, void* scratch,
+                        size_t scratch_bytes, cudaStream_t st);
+
+// search order of the dictionary (kernels_tree.cu)
+void tree_depths(int64_t n, int* d1, int* d2);
+size_t tree_scratch_bytes(int64_t n);
+cudaError_t build_search_tree(zoom_index ix, void* scratch, size_t scratch_bytes, cudaStream_t st);
 
 // per-query steps (kernels_query.cu)
 // F: feature mode (0 pixels minus mean, 1 / 2 first / second-order gradients)
@@ -179,7 +204,49 @@ bool tc_wide_form(int precision, int kc);
 cudaError_t launch_knn_tc(const uint16_t* qop, const float* qn, int64_t nq, const uint16_t* dop,
                           int64_t nd, int precision, int kc, int MC, int nsplit, int tail_split, int grid,
                           float* out_d, int32_t* out_id, unsigned int* status, cudaStream_t st,
-                          const unsigned long long* nq_dev = nullptr, uint64_t wait_ns = 0, int inject = 0);
+                          const unsigned long long* nq_dev = nullptr, uint64_t wait_ns = 0, int inject = 0,
+                          float* part_d = nullptr, int32_t* part_id = nullptr);
+// elements of part_d / part_id (with nq_dev): with them a small count's
+// lists are made in pieces over all SMs and joined
+int64_t tc_part_floats(int grid, int MC);
+// The wide-step filter over a list of 256-row steps per 256 queries: pair p
+// of queries sees the steps seeds[p][0 .. kPruneSeeds) of the dictionary
+// operand; one list of the MC best chunks per query.
+constexpr int kPruneSeeds = 64;
+cudaError_t launch_knn_seeds(const uint16_t* qop, const float* qn, int64_t nq, const uint16_t* dop, int64_t nd,
+                             int precision, int kc, int MC, const int32_t* seeds, int grid, float* out_d,
+                             int32_t* out_id, unsigned int* status, cudaStream_t st, uint64_t wait_ns, int inject);
+// Bound on |d~ - d| of a filter form (0 split, 1 BF16, 2 single-term FP16)
+// for an entry with ||c|| <= rho: c_qr ||q|| rho + c_sq (rho^2 + ||q||^2) +
+// c_abs (||q|| + rho) + c_rel d.
+struct FilterError {
+  float c_qr, c_sq, c_abs, c_rel;
+};
+FilterError tc_filter_error(int d, int precision);
+
+// search over the dictionary's search order (kernels_prune.cu)
+constexpr int64_t kPruneMinEntries = 65536;   // dictionaries that get a search order
+constexpr int64_t kPruneMaxEntries = int64_t{2048} * 16 * 256;
+// The searches that use it.  The stages before the filter cost about 300 us
+// whatever the size.  Against the dense search (L = 8..16, K = 8, one
+// image's queries; auto / dense us): 24,382 queries 468 / 596 with 70,000
+// entries and 733 / 993 with 200,000; 9,312 queries 567 / 394 with 200,000,
+// 593 / 652 with 300,000; 4,224 queries 535 / 500 with 300,000.
+constexpr int64_t kPruneMinQueries = 20000;        // ... or
+constexpr int64_t kPruneMinPairs = 2500000000;     // queries x entries
+struct PrunePlan {
+  int form = 2, kc = 4, mc = 16, r = 12;
+  int64_t slab = 0;      // queries per round of visits and filter steps
+  uint32_t cap = 0;      // candidates per query
+};
+bool prune_plan(zoom_index ix, int form, int K, int64_t nq, PrunePlan* p);
+size_t prune_ws_bytes(zoom_index ix, const PrunePlan& p, int64_t nq);
+// Neighbours of nq queries into nbr / dist; those it cannot prove are
+// appended to fb (count *fb_count, zeroed by the caller).
+cudaError_t run_pruned(zoom_index ix, const PrunePlan& p, const float* qfeat, const uint64_t* qkeys, int64_t nq,
+                       int K, int32_t* nbr, float* dist, void* ws, int32_t* fb, unsigned long long* fb_count,
+                       cudaStream_t st);
+
 // ld/li: per split and query the MC best 32-entry chunks (filter minimum d~,
 // chunk index), ascending; form 1 for the FP16-split filter, 2 for the
 // single-term FP16 filter (both: proof and fallback flags), 0 for the BF16
