@@ -294,7 +294,7 @@ __device__ __forceinline__ float filter_error(float T, float qn, const FilterErr
 // passes.
 template <int FORM>
 __global__ void k_radius(const float* __restrict__ ld, int MC, int r, const float* __restrict__ qn, int64_t nq,
-                         FilterError fe, int D, int row_len, float* __restrict__ rad, float* __restrict__ vis,
+                         FilterError fe, float trunc, int D, int row_len, float* __restrict__ rad, float* __restrict__ vis,
                          uint16_t* __restrict__ qrow, uint16_t* __restrict__ pad) {
   const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   auto bits = [](float x, float& back) -> uint16_t {
@@ -316,12 +316,23 @@ __global__ void k_radius(const float* __restrict__ ld, int MC, int r, const floa
   const float n = qn[q];
   const float v = ld[q * MC + r - 1];
   const bool ok = n < 1000.f && v < 1000.f && v > -1000.f;   // false for NaN
-  float T = -1.f, vs = -1.f;
+  float T = -1.f, vs = -1.f;   // nothing is visited, nothing proven
   if (ok) {
     T = fmaxf(v, 0.f);
+    if (FORM == 1) T *= 1.f + trunc;
     T = fmaxf(T, filter_error(T, n, fe));
     const float dl = filter_error(T, n, fe);
-    vs = T * (PT_SCALE * PT_SCALE) * 1.01f + 1e-5f;
+    vs = T;
+    if (FORM == 1) {
+      // every entry with d~ <= T is a candidate: those of the tiles left out
+      // have d > vs, hence d~ > vs - (error at vs) >= T
+      vs = T + filter_error(T + 2.f * dl, n, fe);
+      if (vs > T + 2.f * dl) {   // (the error grows slower than that)
+        rad[q] = vis[q] = -1.f;
+        return;
+      }
+    }
+    vs = vs * (PT_SCALE * PT_SCALE) * 1.01f + 1e-5f;
     float x = n - (T + dl + (T + dl + n) * 1e-6f + 2e-7f);   // - thr
     uint16_t* o = qrow + q * row_len + D + 3;
 #pragma unroll
@@ -931,18 +942,62 @@ __global__ void __maxnreg__(80) k_knn_tg(TgArgs a) {
 
 // ---------------------------------------------------------------------------
 // exact selection among a query's candidates: one warp per query, one
-// candidate per lane and round (the records expanded in shared memory) (FP32 difference form in the order of the
-// other searches, so the distances are the same bits).  Queries whose K-th
-// member is not within the radius are listed in fb.
+// candidate per lane and round, the records expanded in shared memory (FP32
+// difference form in the order of the other searches, so the distances are
+// the same bits).  Queries whose K-th member is not within the radius are
+// listed in fb.
+//
+// FORM 1, the precision form: its result is the K best members among the
+// entries of the `chunks` dictionary chunks (32 consecutive entries) with the
+// smallest BF16 distance d~.  That is the exact result here wherever the K
+// members' chunks are all listed, and they are if no more than `chunks`
+// chunks have an entry with d~ <= M, the largest d~ of the K members.  The
+// candidates hold every entry with d~ <= T (k_radius), so it is enough to
+// compute d~ of the candidates (BF16 operands, FP32 sums; mg bounds what the
+// sums' order and the norm's three terms can change, and `trunc` the rounding
+// of packed list keys) and count the chunks up to M + mg.  A query that
+// fails this is searched by the dense filter like any query before:
+// those past tail_q0, whose lists that filter cuts into parts, are listed
+// apart.
 // ---------------------------------------------------------------------------
+constexpr int kDtRoom = 128;   // d~ kept per query: chunks past it fail the count anyway
+
 template <int D>
+__device__ __forceinline__ float bf16_distance(const float4* __restrict__ r4, const float4* q4, float qn) {
+  // ||q||^2 + ||c||^2 - 2 q~ . c~
+  float n2 = 0.f, dot = 0.f;
+#pragma unroll
+  for (int k = 0; k < (D + 3) / 4; ++k) {
+    const float4 v4 = __ldg(r4 + k);
+    const float x4[4] = {v4.x, v4.y, v4.z, v4.w};
+    const float4 b4 = q4[k];
+    const float b[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      if (4 * k + t < D) {
+        n2 = fmaf(x4[t], x4[t], n2);
+        dot = fmaf(b[t], __bfloat162float(__float2bfloat16_rn(x4[t])), dot);
+      }
+    }
+  }
+  return qn + (n2 - 2.f * dot);
+}
+
+template <int D, int FORM>
 __global__ void __launch_bounds__(128) k_rerank_list(
     const int32_t* __restrict__ perm, const float* __restrict__ rad, int nslab, const uint32_t* __restrict__ qcnt,
     const uint2* __restrict__ cand, uint32_t cap, const int32_t* __restrict__ order, int64_t nd,
     const float* __restrict__ qfeat, int dpad, const uint64_t* __restrict__ qkeys, const float* __restrict__ dfeat,
-    const uint64_t* __restrict__ dkeys, int L, int tmin, int K, int32_t* __restrict__ nbr, float* __restrict__ dist,
-    int32_t* __restrict__ fb_list, unsigned long long* __restrict__ fb_count) {
+    const uint64_t* __restrict__ dkeys, int L, int tmin, int K, FilterError fe, int chunks, float trunc,
+    int64_t tail_q0, int32_t* __restrict__ nbr, float* __restrict__ dist, int32_t* __restrict__ fb_list,
+    unsigned long long* __restrict__ fb_count, int32_t* __restrict__ tail_list,
+    unsigned long long* __restrict__ tail_count) {
   constexpr int kRow4 = (D + 3) / 4;
+  __shared__ float4 s_qb[FORM == 1 ? 4 : 1][kRow4];            // the query in BF16
+  __shared__ float s_dt[FORM == 1 ? 4 : 1][kDtRoom];           // d~ <= T of the candidates
+  __shared__ int s_ch[FORM == 1 ? 4 : 1][kDtRoom];             // and their chunks
+  uint32_t kept = 0;
+  float qn = 0.f, mg = 0.f;
   __shared__ uint64_t s_qk[4][32];
   __shared__ float4 s_q4[4][kRow4];
   __shared__ float2 s_m[4][32];
@@ -958,6 +1013,29 @@ __global__ void __launch_bounds__(128) k_rerank_list(
     if (lane < L) s_qk[wib][lane] = qkeys[oq * L + lane];
     if (lane < kRow4) s_q4[wib][lane] = reinterpret_cast<const float4*>(qfeat + oq * dpad)[lane];
     __syncwarp();
+    if constexpr (FORM == 1) {
+      const float4* q4 = s_q4[wib];
+#pragma unroll
+      for (int k = 0; k < kRow4; ++k) {
+        const float4 v = q4[k];
+        if (4 * k < D) qn = fmaf(v.x, v.x, qn);
+        if (4 * k + 1 < D) qn = fmaf(v.y, v.y, qn);
+        if (4 * k + 2 < D) qn = fmaf(v.z, v.z, qn);
+        if (4 * k + 3 < D) qn = fmaf(v.w, v.w, qn);
+      }
+      if (lane < kRow4) {
+        float4 v = q4[lane];
+        v.x = __bfloat162float(__float2bfloat16_rn(v.x));
+        v.y = __bfloat162float(__float2bfloat16_rn(v.y));
+        v.z = __bfloat162float(__float2bfloat16_rn(v.z));
+        v.w = __bfloat162float(__float2bfloat16_rn(v.w));
+        s_qb[wib][lane] = v;
+      }
+      const float rc = sqrtf(qn) + sqrtf(T) * 1.1f;
+      // twice the sums' bound for the member that sets M and for the other entry
+      mg = 4.f * (fe.c_sq * (rc * rc + qn) + fe.c_abs * (sqrtf(qn) + rc)) + 1e-12f;
+      __syncwarp();
+    }
     float bd = FLT_MAX, dK = FLT_MAX;
     int bi = INT_MAX, iK = INT_MAX, members = 0;
     // the records' positions, 32 records at a time, then 32 entries at a time
@@ -1007,6 +1085,21 @@ __global__ void __launch_bounds__(128) k_rerank_list(
           }
         }
       }
+      if constexpr (FORM == 1) {
+        bool keep = false;
+        float dt = 0.f;
+        if (eid != INT_MAX) {
+          dt = bf16_distance<D>(reinterpret_cast<const float4*>(dfeat + (int64_t)eid * dpad), s_qb[wib], qn);
+          keep = dt <= T;
+        }
+        const unsigned km = __ballot_sync(kFull, keep);
+        const uint32_t at = kept + (uint32_t)__popc(km & lanes_below(lane));
+        if (keep && at < (uint32_t)kDtRoom) {
+          s_dt[wib][at] = dt;
+          s_ch[wib][at] = eid >> 5;
+        }
+        kept += (uint32_t)__popc(km);
+      }
       // ascending (distance, ID); membership is tested in that order until K
       // members of this round are known (no later one can enter) or the
       // entries lie past the K best of the rounds before
@@ -1044,12 +1137,45 @@ __global__ void __launch_bounds__(128) k_rerank_list(
       }
     }
     flagged = members < K || !(dK <= T);
+    if constexpr (FORM == 1) {
+      if (!flagged) {   // warp-uniform
+        float M = -FLT_MAX;
+        if (lane < K)
+          M = bf16_distance<D>(reinterpret_cast<const float4*>(dfeat + (int64_t)bi * dpad), s_qb[wib], qn);
+#pragma unroll
+        for (int o = 16; o; o >>= 1) M = fmaxf(M, __shfl_xor_sync(kFull, M, o));
+        M += fabsf(M) * trunc + mg;
+        flagged = !(M <= T) || kept > (uint32_t)kDtRoom;
+        if (!flagged) {
+          __syncwarp();
+          // distinct chunks with d~ <= M: an entry counts if no earlier one
+          // of its chunk does
+          uint32_t c = 0;
+          for (uint32_t i = lane; i < kept; i += 32)
+            c += s_dt[wib][i] <= M ? 1u : 0u;
+          c = __reduce_add_sync(kFull, c);
+          if (c > (uint32_t)chunks) {
+            c = 0;
+            for (uint32_t i = lane; i < kept; i += 32) {
+              bool first = s_dt[wib][i] <= M;
+              for (uint32_t j = 0; first && j < i; ++j) first = !(s_dt[wib][j] <= M && s_ch[wib][j] == s_ch[wib][i]);
+              c += first ? 1u : 0u;
+            }
+            c = __reduce_add_sync(kFull, c);
+          }
+          flagged = c > (uint32_t)chunks;
+        }
+      }
+    }
     if (!flagged && lane < K) {
       nbr[oq * K + lane] = bi;
       dist[oq * K + lane] = bd;
     }
   }
-  if (flagged && lane == 0) fb_list[atomicAdd(fb_count, 1ull)] = (int32_t)oq;
+  if (flagged && lane == 0) {
+    if (FORM == 1 && oq >= tail_q0) tail_list[atomicAdd(tail_count, 1ull)] = (int32_t)oq;
+    else fb_list[atomicAdd(fb_count, 1ull)] = (int32_t)oq;
+  }
 }
 
 template <int KC, uint32_t T>
@@ -1151,7 +1277,7 @@ size_t prune_ws_bytes(zoom_index ix, const PrunePlan& p, int64_t nq) {
 
 cudaError_t run_pruned(zoom_index ix, const PrunePlan& p, const float* qfeat, const uint64_t* qkeys, int64_t nq,
                        int K, int32_t* nbr, float* dist, void* ws, int32_t* fb, unsigned long long* fb_count,
-                       cudaStream_t st) {
+                       int32_t* fb_tail, unsigned long long* tail_count, cudaStream_t st) {
   zoom_dict d = ix->dict;
   zoom_ctx ctx = d->ctx;
   PruneBufs b;
@@ -1202,9 +1328,9 @@ cudaError_t run_pruned(zoom_index ix, const PrunePlan& p, const float* qfeat, co
   {
     const unsigned blocks = (unsigned)((nq + 255) / 256);
     if (p.form == 1)
-      k_radius<1><<<blocks, 256, 0, st>>>(b.ld, p.mc, p.r, b.qn, nq, fe, d->d, p.kc * 8, b.rad, b.vis, b.qrow, pad);
+      k_radius<1><<<blocks, 256, 0, st>>>(b.ld, p.mc, p.r, b.qn, nq, fe, p.trunc, d->d, p.kc * 8, b.rad, b.vis, b.qrow, pad);
     else
-      k_radius<2><<<blocks, 256, 0, st>>>(b.ld, p.mc, p.r, b.qn, nq, fe, d->d, p.kc * 8, b.rad, b.vis, b.qrow, pad);
+      k_radius<2><<<blocks, 256, 0, st>>>(b.ld, p.mc, p.r, b.qn, nq, fe, p.trunc, d->d, p.kc * 8, b.rad, b.vis, b.qrow, pad);
   }
   // enough warps to fill the SMs: a warp takes 32 queries and every parts-th
   // group of 32 super tiles
@@ -1240,15 +1366,19 @@ cudaError_t run_pruned(zoom_index ix, const PrunePlan& p, const float* qfeat, co
     if (p.form == 1) e = p.kc == 4 ? run_tg<4, 1>(a, ctx->n_sm, st) : run_tg<8, 1>(a, ctx->n_sm, st);
     else e = p.kc == 4 ? run_tg<4, 0>(a, ctx->n_sm, st) : run_tg<8, 0>(a, ctx->n_sm, st);
     if (e != cudaSuccess) return e;
-#define ZOOM_PR_LIST(DD)                                                                                         \
-  k_rerank_list<DD><<<(m + 3) / 4, 128, 0, st>>>(b.perm + q0, b.rad + q0, m, b.qcnt, b.cand, p.cap, ix->tree_order, \
-                                                 d->n, qfeat, d->dpad, qkeys, d->feat, ix->dkeys, ix->L, tmin, K,   \
-                                                 nbr, dist, fb, fb_count)
-    switch (d->d) {
-      case 9: ZOOM_PR_LIST(9); break;
-      case 25: ZOOM_PR_LIST(25); break;
-      case 18: ZOOM_PR_LIST(18); break;
-      default: ZOOM_PR_LIST(50); break;
+#define ZOOM_PR_LIST(DD, FF)                                                                                      \
+  k_rerank_list<DD, FF><<<(m + 3) / 4, 128, 0, st>>>(                                                           \
+      b.perm + q0, b.rad + q0, m, b.qcnt, b.cand, p.cap, ix->tree_order, d->n, qfeat, d->dpad, qkeys, d->feat,  \
+      ix->dkeys, ix->L, tmin, K, fe, p.chunks, p.trunc, p.tail_q0, nbr, dist, fb, fb_count, fb_tail, tail_count)
+    switch (d->d + (p.form == 1 ? 100 : 0)) {
+      case 9: ZOOM_PR_LIST(9, 2); break;
+      case 25: ZOOM_PR_LIST(25, 2); break;
+      case 18: ZOOM_PR_LIST(18, 2); break;
+      case 50: ZOOM_PR_LIST(50, 2); break;
+      case 109: ZOOM_PR_LIST(9, 1); break;
+      case 125: ZOOM_PR_LIST(25, 1); break;
+      case 118: ZOOM_PR_LIST(18, 1); break;
+      default: ZOOM_PR_LIST(50, 1); break;
     }
 #undef ZOOM_PR_LIST
     e = cudaGetLastError();

@@ -148,12 +148,12 @@ __device__ __forceinline__ int64_t searched_queries(const TcArgs& a) {
 }
 
 // Pieces per list of a search over a device count of `pairs` query pairs: the
-// largest power of two (at most 16) that still gives every CTA of `grid` two
-// items at most, so that the pieces' lists fit the 2 * grid places of
+// largest power of two (at most 128 pieces in all) that still gives every CTA
+// of `grid` two items at most, so that the pieces' lists fit the 2 * grid places of
 // part_d; 1 = no pieces.
 __device__ __forceinline__ int fan_out(int pairs, int nsplit, int grid) {
   int m = 1;
-  while (m < 16 && pairs * nsplit * 2 * m <= 2 * grid) m *= 2;
+  while (m * nsplit < 128 && pairs * nsplit * 2 * m <= 2 * grid) m *= 2;
   return m;
 }
 

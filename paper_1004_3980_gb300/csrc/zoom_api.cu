@@ -563,12 +563,12 @@ struct SplitBufs {
   float *qn, *ld, *pd;
   int32_t *li, *pi;
 };
-SplitBufs take_split(Carver& c, zoom_index ix, int64_t n, int nsplit, int MC) {
+SplitBufs take_split(Carver& c, zoom_index ix, int64_t n, int nsplit, int MC, int prec = 0) {
   zoom_dict d = ix->dict;
   SplitBufs b;
   b.feat = c.take<float>((size_t)n * d->dpad);
   b.keys = c.take<uint64_t>((size_t)n * ix->L);
-  b.qop = c.take<uint16_t>((size_t)tc_rows_padded(n, true) * tc_kc(d->d, 0) * 8);
+  b.qop = c.take<uint16_t>((size_t)tc_rows_padded(n, true) * tc_kc(d->d, prec) * 8);
   b.qn = c.take<float>(n);
   b.ld = c.take<float>((size_t)nsplit * n * MC);
   b.li = c.take<int32_t>((size_t)nsplit * n * MC);
@@ -599,7 +599,32 @@ SearchPlan plan_search(zoom_index ix, const zoom_upscale_params* prm, int64_t nq
   p.KCH = tc_kc(d->d, p.prec) * 8;
   // automatic search and the precision form: over the search order where the
   // dictionary has one
-  if (may_prune && prm->search == 0 && prm->precision == 0 && prune_plan(ix, p.prec, prm->K, nq, &p.pp)) {
+  if (may_prune && p.prec == 1) {
+    // the precision form's dense plan says what its lists are
+    const SearchPlan dense = plan_search(ix, prm, nq, 0, 0, false);
+    if (prune_plan(ix, 1, prm->K, nq, &p.pp)) {
+      p.pruned = true;
+      p.pp.chunks = p.MC;
+      // packed list keys keep 6 mantissa bits at least
+      p.pp.trunc = p.MC == 32 ? 1.05f / 64.f : 0.f;
+      // queries before tail_q0 have one list, the others nsplit
+      p.nsplit = dense.nsplit;
+      const int64_t pairs = (nq + 255) / 256, grid = d->ctx->n_sm;
+      p.pp.tail_q0 = dense.tail_split > 0 ? std::min<int64_t>(nq, pairs / grid * grid * 256) : 0;
+      Carver c(nullptr);
+      c.take<unsigned long long>(4);
+      c.take<int32_t>(nq);
+      c.take<int32_t>(nq);
+      c.take<int32_t>(nq);
+      p.tail_off = (c.off + 255) & ~(size_t)255;
+      Carver t(nullptr), t2(nullptr);
+      take_split(t, ix, p.pp.tail_q0, 1, p.MC, 1);
+      take_split(t2, ix, nq - p.pp.tail_q0, p.nsplit, p.MC, 1);
+      p.bytes = p.tail_off + std::max(prune_ws_bytes(ix, p.pp, nq), std::max(t.off, t2.off)) + 256;
+      return p;
+    }
+  }
+  if (may_prune && prm->search == 0 && p.prec == 2 && prune_plan(ix, 2, prm->K, nq, &p.pp)) {
     p.pruned = true;
     p.cap2 = std::min<int64_t>(nq, std::max<int64_t>(8192, nq / 64));
     p.MC2 = tc_list_size(0, prm->K, prm->rerank_mult);
@@ -692,17 +717,20 @@ SearchPlan plan_search(zoom_index ix, const zoom_upscale_params* prm, int64_t nq
   return p;
 }
 
-// Adds a search's fallback counts to the context's statistics.
+// Adds a search's fallback counts to the context's statistics (tail: a
+// second list's count of queries the first stage left).
 __global__ void k_add_fallback_counts(const unsigned long long* __restrict__ cnt,
-                                      unsigned long long* __restrict__ counters) {
-  counters[CNT_FALLBACK] += cnt[0];
+                                      unsigned long long* __restrict__ counters,
+                                      const unsigned long long* __restrict__ tail = nullptr) {
+  counters[CNT_FALLBACK] += cnt[0] + (tail ? *tail : 0ull);
   counters[CNT_FALLBACK2] += cnt[1];
 }
 
-// The split filter on the queries listed in idx[0 .. *cnt) (at most cap of
-// them; the rest are appended to over / *over_cnt), over nsplit dictionary
-// parts; what its proof leaves joins left / *left_cnt.
-cudaError_t run_split_stage(zoom_index ix, const QueryBufs& q, int64_t nq, int K, int64_t cap, int nsplit, int MC,
+// The split filter (prec 0) or the precision form's filter (1) on the queries
+// listed in idx[0 .. *cnt) (at most cap of them; the rest are appended to
+// over / *over_cnt), over nsplit dictionary parts; what its rerank leaves
+// joins left / *left_cnt.
+cudaError_t run_split_stage(zoom_index ix, const QueryBufs& q, int prec, int64_t nq, int K, int64_t cap, int nsplit, int MC,
                             const SplitBufs& b, const int32_t* idx, const unsigned long long* cnt, int32_t* over,
                             unsigned long long* over_cnt, int32_t* left, unsigned long long* left_cnt,
                             cudaStream_t st) {
@@ -711,13 +739,13 @@ cudaError_t run_split_stage(zoom_index ix, const QueryBufs& q, int64_t nq, int K
   cudaError_t e = launch_gather_queries(idx, cnt, nq, cap, q.feat, d->dpad, q.keys, ix->L, b.feat, b.keys, over,
                                         over_cnt, st);
   if (e == cudaSuccess)
-    e = launch_operand(b.feat, d->dpad, d->d, cap, tc_rows_padded(cap, true), 0, 0, b.qop, b.qn, st, cnt);
+    e = launch_operand(b.feat, d->dpad, d->d, cap, tc_rows_padded(cap, true), 0, prec, b.qop, b.qn, st, cnt);
   if (e == cudaSuccess)
-    e = launch_knn_tc(b.qop, b.qn, cap, ix->dop16, d->n, 0, tc_kc(d->d, 0), MC, nsplit, 0, ctx->n_sm, b.ld, b.li,
-                      ctx->d_status, st, cnt, ctx->wait_ns, ctx->inject, b.pd, b.pi);
+    e = launch_knn_tc(b.qop, b.qn, cap, prec == 1 ? ix->dopbf : ix->dop16, d->n, prec, tc_kc(d->d, prec), MC, nsplit, 0,
+                      ctx->n_sm, b.ld, b.li, ctx->d_status, st, cnt, ctx->wait_ns, ctx->inject, b.pd, b.pi);
   if (e == cudaSuccess)
     e = launch_rerank(d->d, MC, K, b.feat, d->dpad, b.qn, b.keys, cap, d->feat, ix->dkeys, d->n, ix->L, ix->t, b.ld,
-                      b.li, nsplit, 1, q.nbr, q.dist, left, left_cnt, st, idx, cnt);
+                      b.li, nsplit, prec == 1 ? 0 : 1, q.nbr, q.dist, left, left_cnt, st, idx, cnt);
   return e;
 }
 
@@ -743,17 +771,41 @@ cudaError_t run_search_ws(zoom_index ix, const zoom_upscale_params* prm, const Q
     int32_t* fb = s2.take<int32_t>(nq);
     int32_t* more = s2.take<int32_t>(nq);
     int32_t* fb2 = s2.take<int32_t>(nq);
-    const SplitBufs sa = take_split(s2, ix, pl.cap2, pl.nsplit2, pl.MC2);
     char* tail = (char*)ws + pl.tail_off;
-    e = run_pruned(ix, pl.pp, b.feat, b.keys, nq, K, b.nbr, b.dist, tail, fb, cnt, st);
+    e = run_pruned(ix, pl.pp, b.feat, b.keys, nq, K, b.nbr, b.dist, tail, fb, cnt, more, cnt + 2, st);
+    if (pl.prec == 1) {
+      // the queries whose lists might leave out one of the K neighbours: the
+      // dense filter on just those, in the lists it would use for them (the
+      // pruned search's buffers are free now)
+      const int64_t q0 = pl.pp.tail_q0;
+      if (e == cudaSuccess && q0 > 0) {
+        Carver t(tail);
+        const SplitBufs sb = take_split(t, ix, q0, 1, pl.MC, 1);
+        e = run_split_stage(ix, b, 1, nq, K, q0, 1, pl.MC, sb, fb, cnt, nullptr, nullptr, fb2, cnt + 1, st);
+      }
+      if (e == cudaSuccess && q0 < nq) {
+        Carver t(tail);
+        const SplitBufs sb = take_split(t, ix, nq - q0, pl.nsplit, pl.MC, 1);
+        e = run_split_stage(ix, b, 1, nq, K, nq - q0, pl.nsplit, pl.MC, sb, more, cnt + 2, nullptr, nullptr, fb2,
+                            cnt + 1, st);
+      }
+      if (e == cudaSuccess)
+        e = launch_knn_exact(ix, b.feat, b.keys, nq, K, b.nbr, b.dist, ctx->d_counters, fb2, cnt + 1, st);
+      if (e == cudaSuccess) {
+        k_add_fallback_counts<<<1, 1, 0, st>>>(cnt, ctx->d_counters, cnt + 2);
+        e = cudaGetLastError();
+      }
+      return e;
+    }
+    const SplitBufs sa = take_split(s2, ix, pl.cap2, pl.nsplit2, pl.MC2);
     if (e == cudaSuccess)
-      e = run_split_stage(ix, b, nq, K, pl.cap2, pl.nsplit2, pl.MC2, sa, fb, cnt, more, cnt + 2, fb2, cnt + 1, st);
+      e = run_split_stage(ix, b, 0, nq, K, pl.cap2, pl.nsplit2, pl.MC2, sa, fb, cnt, more, cnt + 2, fb2, cnt + 1, st);
     // the pruned search's buffers are free now: the queries past cap2, as
     // one dictionary part each
     if (e == cudaSuccess && pl.cap2 < nq) {
       Carver t(tail);
       const SplitBufs sb = take_split(t, ix, nq, 1, pl.MC2);
-      e = run_split_stage(ix, b, nq, K, nq, 1, pl.MC2, sb, more, cnt + 2, nullptr, nullptr, fb2, cnt + 1, st);
+      e = run_split_stage(ix, b, 0, nq, K, nq, 1, pl.MC2, sb, more, cnt + 2, nullptr, nullptr, fb2, cnt + 1, st);
     }
     if (e == cudaSuccess)
       e = launch_knn_exact(ix, b.feat, b.keys, nq, K, b.nbr, b.dist, ctx->d_counters, fb2, cnt + 1, st);

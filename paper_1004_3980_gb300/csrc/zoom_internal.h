@@ -238,14 +238,20 @@ struct PrunePlan {
   int form = 2, kc = 4, mc = 16, r = 12;
   int64_t slab = 0;      // queries per round of visits and filter steps
   uint32_t cap = 0;      // candidates per query
+  // precision form: chunks the dense filter lists, the relative rounding of
+  // its list keys, and the first query whose lists it cuts into parts
+  int chunks = 16;
+  float trunc = 0.f;
+  int64_t tail_q0 = 0;
 };
 bool prune_plan(zoom_index ix, int form, int K, int64_t nq, PrunePlan* p);
 size_t prune_ws_bytes(zoom_index ix, const PrunePlan& p, int64_t nq);
 // Neighbours of nq queries into nbr / dist; those it cannot prove are
-// appended to fb (count *fb_count, zeroed by the caller).
+// appended to fb (count *fb_count, zeroed by the caller); in the precision
+// form those from p.tail_q0 on to fb_tail (*tail_count).
 cudaError_t run_pruned(zoom_index ix, const PrunePlan& p, const float* qfeat, const uint64_t* qkeys, int64_t nq,
                        int K, int32_t* nbr, float* dist, void* ws, int32_t* fb, unsigned long long* fb_count,
-                       cudaStream_t st);
+                       int32_t* fb_tail, unsigned long long* tail_count, cudaStream_t st);
 
 // ld/li: per split and query the MC best 32-entry chunks (filter minimum d~,
 // chunk index), ascending; form 1 for the FP16-split filter, 2 for the
