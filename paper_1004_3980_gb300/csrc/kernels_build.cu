@@ -58,89 +58,171 @@ __global__ void k_degrade_exact(const float* __restrict__ hr, int H, int W, int 
   lr[(size_t)i * w + j] = shi + slo;
 }
 
+// Patch pairs of the dictionary: one thread computes an entry's LR patch and
+// feature, the block then writes its 128 entries' rows through shared memory
+// and copies their HR patches, neighbouring lanes on neighbouring values.
+// Bound by the rows written (620 bytes an entry at P = 5, s = 2).  With each
+// thread writing its own rows every store instruction touched 32 lines: 1M
+// entries 935 us, 225 us so.
+constexpr int kGatherRows = 128;
+
 template <int P, int F>
-__global__ void k_dict_gather(const float* const* __restrict__ lr_images,
-                              const int32_t* __restrict__ lr_h, const int32_t* __restrict__ lr_w,
-                              const float* const* __restrict__ hr_images,
-                              const int32_t* __restrict__ hr_w, const int32_t* __restrict__ pos,
-                              int64_t n, int s, int dpad, int ph2pad, float* __restrict__ lr_pix,
-                              float* __restrict__ feat, float* __restrict__ mu,
-                              float* __restrict__ norm2, float* __restrict__ hr_res) {
+__global__ void __launch_bounds__(kGatherRows) k_dict_gather(
+    const float* const* __restrict__ lr_images, const int32_t* __restrict__ lr_h,
+    const int32_t* __restrict__ lr_w, const float* const* __restrict__ hr_images,
+    const int32_t* __restrict__ hr_w, const int32_t* __restrict__ pos, int64_t n, int s, int ph2pad,
+    float* __restrict__ lr_pix, float* __restrict__ feat, float* __restrict__ mu,
+    float* __restrict__ norm2, float* __restrict__ hr_res) {
   constexpr int P2 = P * P;
   constexpr int D = zoom_feature_dim(P, F);
-  int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= n) return;
-  int m = pos[e * 3 + 0], i = pos[e * 3 + 1], j = pos[e * 3 + 2];
-  const float* lr = lr_images[m];
-  int lw = lr_w[m];
-  float px[P2], v[P2], mean, n2;
+  constexpr int DP = (D + 3) / 4 * 4;
+  __shared__ float s_pix[kGatherRows * P2];
+  __shared__ float s_feat[F == 0 ? 1 : kGatherRows * (D | 1)];   // odd stride: no bank conflicts
+  __shared__ const float* s_hr[kGatherRows];   // the entry's HR patch
+  __shared__ int s_hw[kGatherRows];
+  __shared__ float s_mean[kGatherRows];
+  const int r = threadIdx.x;
+  const int64_t e0 = (int64_t)blockIdx.x * kGatherRows, e = e0 + r;
+  const int rows = (int)(n - e0 < kGatherRows ? n - e0 : kGatherRows);
+  if (r < rows) {
+    const int m = pos[e * 3 + 0], i = pos[e * 3 + 1], j = pos[e * 3 + 2];
+    const float* lr = lr_images[m];
+    const int lw = lr_w[m];
+    float px[P2], v[P2], mean, n2;
 #pragma unroll
-  for (int a = 0; a < P; ++a)
+    for (int a = 0; a < P; ++a)
 #pragma unroll
-    for (int b = 0; b < P; ++b) px[a * P + b] = lr[(size_t)(i + a) * lw + j + b];
-  zoom_patch_feature<P2>(px, v, mean, n2);
+      for (int b = 0; b < P; ++b) px[a * P + b] = lr[(size_t)(i + a) * lw + j + b];
+    zoom_patch_feature<P2>(px, v, mean, n2);
 #pragma unroll
-  for (int q = 0; q < P2; ++q) lr_pix[e * P2 + q] = px[q];
-  if constexpr (F == 0) {
-    for (int q = 0; q < dpad; ++q) feat[e * dpad + q] = q < D ? v[q] : 0.f;
-  } else {
-    float g[D];
-    zoom_gradient_feature<P, F>(lr, lr_h[m], lw, (size_t)lw, i, j, g, n2);
-    for (int q = 0; q < dpad; ++q) feat[e * dpad + q] = q < D ? g[q] : 0.f;
+    for (int q = 0; q < P2; ++q) s_pix[r * P2 + q] = px[q];
+    if constexpr (F != 0) {
+      float g[D];
+      zoom_gradient_feature<P, F>(lr, lr_h[m], lw, (size_t)lw, i, j, g, n2);
+#pragma unroll
+      for (int q = 0; q < D; ++q) s_feat[r * (D | 1) + q] = g[q];
+    }
+    mu[e] = mean;
+    norm2[e] = n2;
+    const int hw = hr_w[m];
+    s_hr[r] = hr_images[m] + (size_t)(s * i) * hw + s * j;
+    s_hw[r] = hw;
+    s_mean[r] = mean;
   }
-  mu[e] = mean;
-  norm2[e] = n2;
-  const float* hr = hr_images[m];
-  int hw = hr_w[m];
-  int PH = s * P;
-  for (int a = 0; a < PH; ++a)
-    for (int b = 0; b < PH; ++b)
-      hr_res[e * ph2pad + a * PH + b] = hr[(size_t)(s * i + a) * hw + s * j + b] - mean;
-  for (int q = PH * PH; q < ph2pad; ++q) hr_res[e * ph2pad + q] = 0.f;
+  __syncthreads();
+  for (int t = r; t < rows * P2; t += kGatherRows) lr_pix[e0 * P2 + t] = s_pix[t];
+  for (int t = r; t < rows * DP; t += kGatherRows) {
+    const int x = t / DP, q = t % DP;
+    float f = 0.f;
+    // a mean-free patch is the pixels less their mean (zoom_patch_feature)
+    if (q < D) f = F == 0 ? s_pix[x * P2 + q] - s_mean[x] : s_feat[x * (D | 1) + q];
+    feat[e0 * DP + t] = f;
+  }
+  // a warp per HR patch, four entries at a time in flight
+  const int PH = s * P, ph2 = PH * PH;
+  const float inv = 1.f / (float)PH;   // (q + 0.5) / PH is far enough from whole numbers
+  const int lane = r & 31;
+  for (int q = lane; q < ph2pad; q += 32) {
+    const int a = (int)(((float)q + 0.5f) * inv), b = q - a * PH;
+#pragma unroll 4
+    for (int x = r >> 5; x < rows; x += kGatherRows / 32) {
+      float o = 0.f;
+      if (q < ph2) o = s_hr[x][(size_t)a * s_hw[x] + b] - s_mean[x];
+      hr_res[(e0 + x) * ph2pad + q] = o;
+    }
+  }
 }
 
-// Eq. 10 for every projection and the key fold of every table; one thread
-// per feature row.  alpha/beta are staged in shared memory.
-template <int D>
-__global__ void k_hash(const float* __restrict__ feat, int dpad, int64_t n,
-                       const float* __restrict__ alpha, const float* __restrict__ beta, int L, int k,
-                       float w, uint64_t* __restrict__ keys) {
+// Eq. 10 for every projection and the key fold of every table; a thread takes
+// R feature rows and the block's tables (blockIdx.y: a share of the L), whose
+// alpha / beta are staged in shared memory.  Bound by the multiply-adds (L k D
+// a row) and the operations beside them:
+// - two rows a thread share each 16-byte read of the projections;
+// - floor(t / w) comes from a multiplication with 1 / w unless the product
+//   lies within its error of a whole number (or is not finite, or so small
+//   that it could have been rounded to 0), which takes the division;
+// - a pair of keys leaves in one 16-byte store.
+// 1M rows, D = 25, L = k = 16: 755 us with one row a thread and a division a
+// projection, 631 us so.  Few rows split the tables over blocks instead.
+template <int D, int R>
+__global__ void __launch_bounds__(128) k_hash(const float* __restrict__ feat, int dpad, int64_t n,
+                                              const float* __restrict__ alpha, const float* __restrict__ beta,
+                                              int L, int per, int k, float w, uint64_t* __restrict__ keys) {
   // projections staged with rows padded to DP floats (16-byte loads; the
   // multiply-adds keep the order of the feature's values)
   constexpr int DP = (D + 3) / 4 * 4;
   extern __shared__ float4 s_ab4[];
   float* s_ab = reinterpret_cast<float*>(s_ab4);
-  int nproj = L * k;
+  const int l0 = blockIdx.y * per, l1 = min(L, l0 + per);
+  const int nproj = (l1 - l0) * k, p0 = l0 * k;
   for (int t = threadIdx.x; t < nproj * DP; t += blockDim.x) {
     const int pj = t / DP, q = t % DP;
-    s_ab[t] = q < D ? alpha[pj * D + q] : 0.f;
+    s_ab[t] = q < D ? alpha[(p0 + pj) * D + q] : 0.f;
   }
-  for (int t = threadIdx.x; t < nproj; t += blockDim.x) s_ab[nproj * DP + t] = beta[t];
+  for (int t = threadIdx.x; t < nproj; t += blockDim.x) s_ab[nproj * DP + t] = beta[p0 + t];
   __syncthreads();
-  int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= n) return;
-  float v[DP];
+  const int64_t r0 = (int64_t)blockIdx.x * (128 * R) + threadIdx.x;
+  if (r0 >= n) return;
+  float v[R][DP];
 #pragma unroll
-  for (int q = 0; q < DP; ++q) v[q] = q < D ? feat[r * dpad + q] : 0.f;
+  for (int y = 0; y < R; ++y) {
+    const int64_t r = r0 + y * 128 < n ? r0 + y * 128 : r0;   // past the end: the first row again, not stored
+    const float4* f4 = reinterpret_cast<const float4*>(feat + r * dpad);
+#pragma unroll
+    for (int q4 = 0; q4 < DP / 4; ++q4) {
+      const float4 x = f4[q4];
+      v[y][4 * q4] = x.x;
+      v[y][4 * q4 + 1] = x.y;
+      v[y][4 * q4 + 2] = x.z;
+      v[y][4 * q4 + 3] = x.w;
+    }
+  }
   const float* s_beta = s_ab + nproj * DP;
-  for (int l = 0; l < L; ++l) {
-    uint64_t x = (uint64_t)l;
+  const float rw = w < 1e37f ? __frcp_rn(w) : NAN;   // a reciprocal too small for 24 bits: always divide
+  // rows of keys start on 16 bytes (l0 is even; a caller's buffer may not)
+  const bool pairs = (L & 1) == 0 && ((uintptr_t)keys & 15) == 0;
+  uint64_t held[R];
+  for (int l = l0; l < l1; ++l) {
+    uint64_t x[R];
+#pragma unroll
+    for (int y = 0; y < R; ++y) x[y] = (uint64_t)l;
     for (int j = 0; j < k; ++j) {
-      const float4* a4 = s_ab4 + (l * k + j) * (DP / 4);
-      float acc = 0.f;
+      const int pj = (l - l0) * k + j;
+      const float4* a4 = s_ab4 + pj * (DP / 4);
+      float acc[R];
+#pragma unroll
+      for (int y = 0; y < R; ++y) acc[y] = 0.f;
 #pragma unroll
       for (int q4 = 0; q4 < DP / 4; ++q4) {
         const float4 av = a4[q4];
-        acc = fmaf(av.x, v[4 * q4], acc);
-        if (4 * q4 + 1 < D) acc = fmaf(av.y, v[4 * q4 + 1], acc);
-        if (4 * q4 + 2 < D) acc = fmaf(av.z, v[4 * q4 + 2], acc);
-        if (4 * q4 + 3 < D) acc = fmaf(av.w, v[4 * q4 + 3], acc);
+#pragma unroll
+        for (int y = 0; y < R; ++y) {
+          acc[y] = fmaf(av.x, v[y][4 * q4], acc[y]);
+          if (4 * q4 + 1 < D) acc[y] = fmaf(av.y, v[y][4 * q4 + 1], acc[y]);
+          if (4 * q4 + 2 < D) acc[y] = fmaf(av.z, v[y][4 * q4 + 2], acc[y]);
+          if (4 * q4 + 3 < D) acc[y] = fmaf(av.w, v[y][4 * q4 + 3], acc[y]);
+        }
       }
-      float t = acc + s_beta[l * k + j];
-      int h = (int)floorf(__fdiv_rn(t, w));
-      x = zoom_fold_step(x, h, j);
+      const float be = s_beta[pj];
+#pragma unroll
+      for (int y = 0; y < R; ++y) {
+        const float t = acc[y] + be;
+        // t * rw is within 2^-23 |t / w| of t / w, the quotient within 2^-24
+        const float u = t * rw;
+        float fl = floorf(u);
+        const float off = fabsf(u - rintf(u));
+        if (!(off > 4e-7f * fabsf(u) && off > 1e-30f && fabsf(u) < 1e9f)) fl = floorf(__fdiv_rn(t, w));
+        x[y] = zoom_fold_step(x[y], (int)fl, j);
+      }
     }
-    keys[r * L + l] = x;
+#pragma unroll
+    for (int y = 0; y < R; ++y) {
+      const int64_t r = r0 + y * 128;
+      if (r >= n) continue;
+      if (!pairs) keys[r * L + l] = x[y];
+      else if (l & 1) *reinterpret_cast<ulonglong2*>(keys + r * L + l - 1) = make_ulonglong2(held[y], x[y]);
+      held[y] = x[y];
+    }
   }
 }
 
@@ -605,11 +687,11 @@ cudaError_t launch_dict_gather(const float* const* d_lr_images, const int32_t* d
                                const int32_t* d_lr_w, const float* const* d_hr_images,
                                const int32_t* d_hr_w, const int32_t* d_pos, int64_t n, int P, int s,
                                zoom_dict d, cudaStream_t st) {
-  int blocks = (int)((n + 127) / 128);
+  int blocks = (int)((n + kGatherRows - 1) / kGatherRows);
 #define ZOOM_GATHER(PP, FF)                                                                     \
-  k_dict_gather<PP, FF><<<blocks, 128, 0, st>>>(d_lr_images, d_lr_h, d_lr_w, d_hr_images, d_hr_w, \
-                                                d_pos, n, s, d->dpad, d->ph2pad, d->lr_pix,      \
-                                                d->feat, d->mu, d->norm2, d->hr_res)
+  k_dict_gather<PP, FF><<<blocks, kGatherRows, 0, st>>>(d_lr_images, d_lr_h, d_lr_w, d_hr_images, \
+                                                        d_hr_w, d_pos, n, s, d->ph2pad, d->lr_pix, \
+                                                        d->feat, d->mu, d->norm2, d->hr_res)
   if (P == 3 && d->feature == 0) ZOOM_GATHER(3, 0);
   else if (P == 5 && d->feature == 0) ZOOM_GATHER(5, 0);
   else if (P == 3 && d->feature == 1) ZOOM_GATHER(3, 1);
@@ -624,13 +706,29 @@ cudaError_t launch_dict_gather(const float* const* d_lr_images, const int32_t* d
 cudaError_t launch_hash(const float* feat, int dpad, int d, int64_t n, const float* alpha,
                         const float* beta, int L, int k, float w, uint64_t* keys, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
-  size_t smem = (size_t)L * k * ((d + 3) / 4 * 4 + 1) * sizeof(float);
-  int blocks = (int)((n + 127) / 128);
-#define ZOOM_HASH(DD)                                                                       \
-  do {                                                                                      \
-    if (smem > 48 * 1024)                                                                   \
-      cudaFuncSetAttribute(k_hash<DD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
-    k_hash<DD><<<blocks, 128, smem, st>>>(feat, dpad, n, alpha, beta, L, k, w, keys);        \
+  // two rows a thread where that leaves two blocks of 128 for each of about
+  // 150 SMs, else one, with the tables (in twos: see the stores) over blocks
+  // until there are as many (the 2x zoom of
+  // 64x64 with 3,844 queries: 189.6 us on 31 blocks, 182.9 us so)
+  const bool two = n >= 2 * 128 * 304;
+  const int64_t rows = two ? 256 : 128, blocks = (n + rows - 1) / rows;
+  int per = (L + 1) / 2 * 2;
+  while (per > 2 && blocks * ((L + per - 1) / per) < 304) per = (per / 2 + 1) / 2 * 2;
+  const size_t smem = (size_t)(per < L ? per : L) * k * ((d + 3) / 4 * 4 + 1) * sizeof(float);
+  const dim3 grid((unsigned)blocks, (unsigned)((L + per - 1) / per));
+#define ZOOM_HASH1(DD, RR)                                                                                  \
+  do {                                                                                                      \
+    if (smem > 48 * 1024) {                                                                                 \
+      const cudaError_t e =                                                                                 \
+          cudaFuncSetAttribute(k_hash<DD, RR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);     \
+      if (e != cudaSuccess) return e;                                                                       \
+    }                                                                                                       \
+    k_hash<DD, RR><<<grid, 128, smem, st>>>(feat, dpad, n, alpha, beta, L, per, k, w, keys);                \
+  } while (0)
+#define ZOOM_HASH(DD)            \
+  do {                           \
+    if (two) ZOOM_HASH1(DD, 2);  \
+    else ZOOM_HASH1(DD, 1);      \
   } while (0)
   switch (d) {
     case 9: ZOOM_HASH(9); break;
@@ -639,6 +737,7 @@ cudaError_t launch_hash(const float* feat, int dpad, int d, int64_t n, const flo
     case 50: ZOOM_HASH(50); break;
     default: return cudaErrorInvalidValue;
   }
+#undef ZOOM_HASH1
 #undef ZOOM_HASH
   return cudaGetLastError();
 }
