@@ -6,21 +6,33 @@
 // All reductions are deterministic (fixed order, no atomics on values).
 #include <math.h>
 
+#include <algorithm>
+
 #include "device_common.cuh"
 #include "zoom_internal.h"
 
 namespace {
 
-// P[n][p] = mu_n + sum_m w_nm R[nbr_nm][p]; one thread per (patch, pixel).
-__global__ void k_patches(const int32_t* __restrict__ nbr, const float* __restrict__ wgt,
-                          const float* __restrict__ mu, const float* __restrict__ hr_res, int ph2pad,
-                          int K, int64_t nq, int ph2, float* __restrict__ P) {
+// P[n][p] = mu_n + sum_m w_nm R[nbr_nm][p], rows of ph2pad values; one thread
+// per 4 pixels of a patch (the residual rows are padded alike).
+__global__ void __launch_bounds__(256) k_patches(const int32_t* __restrict__ nbr, const float* __restrict__ wgt,
+                                                 const float* __restrict__ mu, const float4* __restrict__ hr_res,
+                                                 int row4, int K, int64_t nq, float4* __restrict__ P) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= nq * ph2) return;
-  const int64_t n = t / ph2;
-  const int p = (int)(t % ph2);
-  float v = mu[n];
-  for (int m = 0; m < K; ++m) v = fmaf(wgt[n * K + m], hr_res[(int64_t)nbr[n * K + m] * ph2pad + p], v);
+  if (t >= nq * row4) return;
+  const int64_t n = t / row4;
+  const int p = (int)(t - n * row4);
+  const float m0 = mu[n];
+  float4 v = make_float4(m0, m0, m0, m0);
+#pragma unroll 4
+  for (int m = 0; m < K; ++m) {
+    const float wm = wgt[n * K + m];
+    const float4 r = __ldg(hr_res + (int64_t)nbr[n * K + m] * row4 + p);
+    v.x = fmaf(wm, r.x, v.x);
+    v.y = fmaf(wm, r.y, v.y);
+    v.z = fmaf(wm, r.z, v.z);
+    v.w = fmaf(wm, r.w, v.w);
+  }
   P[t] = v;
 }
 
@@ -46,6 +58,19 @@ __global__ void k_degrade(const float* __restrict__ x, int H, int W, int h, int 
   y[(int64_t)i * w + j] = sub ? acc - sub[(int64_t)i * w + j] : acc;
 }
 
+// Weight of HR position X in the window of LR position j: one of the window's
+// weights inside, the sum of those that the clamp brings to an edge there.
+__device__ __forceinline__ float window_weight(int X, int N, int s, int j, const Wts& wt) {
+  if (X > 0 && X < N - 1) {
+    const int b = X - s * j + 1;
+    return b >= 0 && b < wt.n ? wt.w[b] : 0.f;
+  }
+  float v = 0.f;
+  for (int b = 0; b < wt.n; ++b)
+    if (zoom_clampi(s * j + b - 1, 0, N - 1) == X) v += wt.w[b];
+  return v;
+}
+
 // g = alpha * B^T D^T r in gather form: HR pixel (Y, X) collects, from every
 // LR pixel (i, j) whose window reads it (through the clamp), the weights
 // W_a(i -> Y) W_b(j -> X) times r(i, j).
@@ -59,76 +84,190 @@ __global__ void k_degrade_adjoint(const float* __restrict__ r, int h, int w, int
   const int j0 = max(0, (X - s) / s - 1), j1 = min(w - 1, (X + 1) / s + 1);
   float acc = 0.f;
   for (int i = i0; i <= i1; ++i) {
-    float wy = 0.f;
-    for (int a = 0; a < wt.n; ++a)
-      if (zoom_clampi(s * i + a - 1, 0, H - 1) == Y) wy += wt.w[a];
+    const float wy = window_weight(Y, H, s, i, wt);
     if (wy == 0.f) continue;
     float row = 0.f;
-    for (int j = j0; j <= j1; ++j) {
-      float wx = 0.f;
-      for (int b = 0; b < wt.n; ++b)
-        if (zoom_clampi(s * j + b - 1, 0, W - 1) == X) wx += wt.w[b];
-      row = fmaf(wx, r[(int64_t)i * w + j], row);
-    }
+    for (int j = j0; j <= j1; ++j) row = fmaf(window_weight(X, W, s, j, wt), r[(int64_t)i * w + j], row);
     acc = fmaf(wy, row, acc);
   }
   g[(int64_t)Y * W + X] = alpha * acc;
 }
 
+// The patch pixel p = (a, b): a, b and a / s, b / s, a byte each (PH <= 20).
+__device__ __forceinline__ uint32_t pixel_code(int p, int PH, int s) {
+  const int a = p / PH, b = p - a * PH;
+  return (uint32_t)a | ((uint32_t)b << 8) | ((uint32_t)(a / s) << 16) | ((uint32_t)(b / s) << 24);
+}
+constexpr int kMaxPatchPixels = 400;   // (s P)^2 at s = 4, P = 5
+
 // dE/dP[n][p] = gx(Y, X) / n_cov(Y, X) + lambda * 2 * sum over the 4 LR-grid
-// neighbour patches q overlapping pixel p of (P_n - P_q) at that pixel.
-__global__ void k_patch_grad(const float* __restrict__ gx, const float* __restrict__ P, int h, int w, int s,
-                             int Pp, float lambda, float* __restrict__ gP) {
+// neighbour patches q overlapping pixel p of (P_n - P_q) at that pixel.  A
+// warp per patch, lanes over its pixels, rows of ph2pad values (the padding
+// is written 0).  Bound by the rows written; with a thread per value, which
+// divided for its patch, pixel and counts, 119,691 patches of 15 x 15 took
+// 214 us, 87 us so.
+__global__ void __launch_bounds__(256) k_patch_grad(const float* __restrict__ gx, const float* __restrict__ P,
+                                                    int h, int w, int s, int Pp, int ph2pad, float lambda,
+                                                    float* __restrict__ gP) {
+  __shared__ uint32_t s_px[kMaxPatchPixels];
   const int PH = s * Pp, ph2 = PH * PH;
-  const int nh = h - Pp + 1, nw = w - Pp + 1;
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (int64_t)nh * nw * ph2) return;
-  const int64_t n = t / ph2;
-  const int p = (int)(t % ph2);
-  const int i = (int)(n / nw), j = (int)(n % nw);
-  const int a = p / PH, b = p % PH;
-  const int Y = s * i + a, X = s * j + b;
-  const int W = s * w;
-  const int ci = min(Y / s, nh - 1) - (Y >= PH ? (Y - PH) / s + 1 : 0) + 1;
-  const int cj = min(X / s, nw - 1) - (X >= PH ? (X - PH) / s + 1 : 0) + 1;
-  float g = gx[(int64_t)Y * W + X] / (float)(ci * cj);
-  if (lambda != 0.f) {   // P is read only for the prior term
-    const float pv = P[t];
-    float pr = 0.f;
-    if (j + 1 < nw && b >= s) pr += pv - P[(n + 1) * ph2 + a * PH + (b - s)];
-    if (j > 0 && b < PH - s) pr += pv - P[(n - 1) * ph2 + a * PH + (b + s)];
-    if (i + 1 < nh && a >= s) pr += pv - P[(n + nw) * ph2 + (a - s) * PH + b];
-    if (i > 0 && a < PH - s) pr += pv - P[(n - nw) * ph2 + (a + s) * PH + b];
-    g = fmaf(2.f * lambda, pr, g);
+  const int nh = h - Pp + 1, nw = w - Pp + 1, W = s * w;
+  for (int p = threadIdx.x; p < ph2; p += blockDim.x) s_px[p] = pixel_code(p, PH, s);
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  const int64_t nq = (int64_t)nh * nw, nwarp = (int64_t)gridDim.x * (blockDim.x >> 5);
+  for (int64_t n = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); n < nq; n += nwarp) {
+    const int i = (int)(n / nw), j = (int)(n - (int64_t)i * nw);
+    const float* g0 = gx + (int64_t)(s * i) * W + s * j;
+    for (int p = lane; p < ph2pad; p += 32) {
+      float g = 0.f;
+      if (p < ph2) {
+        const uint32_t c = s_px[p];
+        const int a = c & 255, b = (c >> 8) & 255, as = (c >> 16) & 255, bs = c >> 24;
+        // patches covering HR row Y = s i + a: min(Y / s, nh - 1) down to
+        // (Y - PH) / s + 1 (0 where Y < PH); Y / s = i + a / s
+        const int ci = min(i + as, nh - 1) - max(0, i + as - Pp + 1) + 1;
+        const int cj = min(j + bs, nw - 1) - max(0, j + bs - Pp + 1) + 1;
+        g = g0[a * W + b] / (float)(ci * cj);
+        if (lambda != 0.f) {   // P is read only for the prior term
+          const float* pn = P + n * ph2pad;
+          const float pv = pn[p];
+          float pr = 0.f;
+          if (j + 1 < nw && b >= s) pr += pv - pn[ph2pad + p - s];
+          if (j > 0 && b < PH - s) pr += pv - pn[p + s - ph2pad];
+          if (i + 1 < nh && a >= s) pr += pv - pn[(int64_t)nw * ph2pad + p - s * PH];
+          if (i > 0 && a < PH - s) pr += pv - pn[p + s * PH - (int64_t)nw * ph2pad];
+          g = fmaf(2.f * lambda, pr, g);
+        }
+      }
+      gP[n * ph2pad + p] = g;
+    }
   }
-  gP[t] = g;
+}
+
+// acc += sum over the uses [u0, u1) of w[u] * gP[u / K], 4 pixels a lane and V
+// such groups: the uses' numbers and weights are read 32 at a time, and the
+// rows of U uses are in flight together, added in order.
+template <int V, int U>
+__device__ __forceinline__ void add_uses(int u0, int u1, const int32_t* __restrict__ sorted_use,
+                                         const float* __restrict__ wgt, const float4* __restrict__ gP, int K,
+                                         int row4, int lane, float4 (&acc)[V]) {
+  for (int ub = u0; ub < u1; ub += 32) {
+    const int use = ub + lane < u1 ? sorted_use[ub + lane] : 0;
+    const float wu = ub + lane < u1 ? wgt[use] : 0.f;
+    const int row = use / K;
+    const int n = min(32, u1 - ub);
+    for (int t0 = 0; t0 < n; t0 += U) {
+      float4 x[U][V];
+#pragma unroll
+      for (int t = 0; t < U; ++t) {
+        const float4* g = gP + (int64_t)__shfl_sync(0xffffffffu, row, t0 + t) * row4;
+#pragma unroll
+        for (int v = 0; v < V; ++v)
+          if (t0 + t < n && v * 32 + lane < row4) x[t][v] = __ldg(g + v * 32 + lane);
+      }
+#pragma unroll
+      for (int t = 0; t < U; ++t) {
+        const float wt = __shfl_sync(0xffffffffu, wu, t0 + t);
+        if (t0 + t < n) {
+#pragma unroll
+          for (int v = 0; v < V; ++v) {
+            if (v * 32 + lane < row4) {
+              acc[v].x = fmaf(wt, x[t][v].x, acc[v].x);
+              acc[v].y = fmaf(wt, x[t][v].y, acc[v].y);
+              acc[v].z = fmaf(wt, x[t][v].z, acc[v].z);
+              acc[v].w = fmaf(wt, x[t][v].w, acc[v].w);
+            }
+          }
+        }
+      }
+    }
+  }
+}
+
+template <int V>
+__device__ __forceinline__ void store_grad(float* out, int ph2, int lane, int v, float4 a) {
+  const int p = 4 * (v * 32 + lane);
+  if (p < ph2) out[p] = a.x;
+  if (p + 1 < ph2) out[p + 1] = a.y;
+  if (p + 2 < ph2) out[p + 2] = a.z;
+  if (p + 3 < ph2) out[p + 3] = a.w;
 }
 
 // grad_R[id][p] = sum over the uses u of entry id (sorted, ascending) of
-// w[u] * gP[u / K][p]; one block per used entry, one thread per pixel.
-__global__ void k_dict_grad(const int32_t* __restrict__ sorted_use, const int32_t* __restrict__ offs,
-                            const uint64_t* __restrict__ ukeys, const int32_t* __restrict__ nuniq,
-                            const float* __restrict__ wgt, const float* __restrict__ gP, int K, int ph2,
-                            int ph2pad_out, float* __restrict__ grad) {
-  const int seg = blockIdx.x;
-  if (seg >= *nuniq) return;
-  const int id = (int)ukeys[seg];
-  for (int p = threadIdx.x; p < ph2; p += blockDim.x) {
-    float acc = 0.f;
-    for (int u = offs[seg]; u < offs[seg + 1]; ++u) {
-      const int use = sorted_use[u];
-      acc = fmaf(wgt[use], gP[(int64_t)(use / K) * ph2 + p], acc);
+// w[u] * gP[u / K][p].  A warp per used entry; entries with more than kDgLong
+// uses (flat patches are near thousands of queries) are listed for
+// k_dict_grad_long: a block each, a sixteenth of the uses per warp, the warps'
+// sums added in order.  Bound by the rows read, K times each; with a block per
+// entry and one use after the other 119,691 patches of 15 x 15 with K = 8
+// took 340 us and 63,504 of 10 x 10 129 us, the longest entries most of it:
+// 202 and 80 us so.
+constexpr int kDgWarps = 16;
+
+template <int V>
+__global__ void __launch_bounds__(128) k_dict_grad(const int32_t* __restrict__ sorted_use,
+                                                   const int32_t* __restrict__ offs,
+                                                   const uint64_t* __restrict__ ukeys,
+                                                   const int32_t* __restrict__ nuniq,
+                                                   const float* __restrict__ wgt, const float4* __restrict__ gP,
+                                                   int K, int row4, int ph2, int out_stride,
+                                                   float* __restrict__ grad, int32_t* __restrict__ long_list) {
+  const int seg = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (seg >= *nuniq) return;   // warp-uniform
+  const int u0 = offs[seg], u1 = offs[seg + 1];
+  if (u1 - u0 > kDgLong) {
+    if (lane == 0) long_list[1 + atomicAdd(long_list, 1)] = seg;
+    return;
+  }
+  float4 acc[V];
+#pragma unroll
+  for (int v = 0; v < V; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+  add_uses<V, 4 / V>(u0, u1, sorted_use, wgt, gP, K, row4, lane, acc);
+  float* out = grad + (int64_t)ukeys[seg] * out_stride;
+#pragma unroll
+  for (int v = 0; v < V; ++v) store_grad<V>(out, ph2, lane, v, acc[v]);
+}
+
+template <int V>
+__global__ void __launch_bounds__(kDgWarps * 32) k_dict_grad_long(
+    const int32_t* __restrict__ sorted_use, const int32_t* __restrict__ offs, const uint64_t* __restrict__ ukeys,
+    const float* __restrict__ wgt, const float4* __restrict__ gP, int K, int row4, int ph2, int out_stride,
+    float* __restrict__ grad, const int32_t* __restrict__ long_list) {
+  __shared__ float4 s_part[kDgWarps][V * 32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int count = long_list[0];
+  for (int k = blockIdx.x; k < count; k += gridDim.x) {
+    const int seg = long_list[1 + k];
+    const int b0 = offs[seg], n = offs[seg + 1] - b0;
+    float4 acc[V];
+#pragma unroll
+    for (int v = 0; v < V; ++v) acc[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+    add_uses<V, 8 / V>(b0 + (int)((int64_t)n * warp / kDgWarps), b0 + (int)((int64_t)n * (warp + 1) / kDgWarps),
+                       sorted_use, wgt, gP, K, row4, lane, acc);
+#pragma unroll
+    for (int v = 0; v < V; ++v) s_part[warp][v * 32 + lane] = acc[v];
+    __syncthreads();
+    if (warp < V) {
+      float4 a = s_part[0][warp * 32 + lane];
+      for (int j = 1; j < kDgWarps; ++j) {
+        const float4 x = s_part[j][warp * 32 + lane];
+        a.x += x.x;
+        a.y += x.y;
+        a.z += x.z;
+        a.w += x.w;
+      }
+      store_grad<V>(grad + (int64_t)ukeys[seg] * out_stride, ph2, lane, warp, a);
     }
-    grad[(int64_t)id * ph2pad_out + p] = acc;
+    __syncthreads();   // the sums have been read
   }
 }
 
 // grad_mu[n] = sum_p OA^T(g)[n][p] (the patch mean enters every pixel).
-__global__ void k_mu_grad(const float* __restrict__ gP, int64_t nq, int ph2, float* __restrict__ gmu) {
+__global__ void k_mu_grad(const float* __restrict__ gP, int64_t nq, int ph2, int ph2pad, float* __restrict__ gmu) {
   const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= nq) return;
   float acc = 0.f;
-  for (int p = 0; p < ph2; ++p) acc += gP[n * ph2 + p];
+  for (int p = 0; p < ph2; ++p) acc += gP[n * ph2pad + p];
   gmu[n] = acc;
 }
 
@@ -147,30 +286,72 @@ __global__ void k_sumsq_partials(const float* __restrict__ r, int64_t n, double*
   if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
 }
 
+// (s, c) += (a - b)^2, a sum in two floats: the difference and its square are
+// exact in two floats but for terms below 2^-48 of the square, as is what the
+// sum leaves out of each addition.
+__device__ __forceinline__ void add_sqdiff(float a, float b, float& s, float& c) {
+  const float d = a - b, bb = d - a;
+  const float dl = (a - (d - bb)) - (b + bb);   // a - b = d + dl
+  const float p = d * d;
+  const float e = fmaf(2.f * d, dl, fmaf(d, d, -p));
+  const float t = s + p, v = t - s;
+  c += ((s - (t - v)) + (p - v)) + e;
+  s = t;
+}
+
 // per-block partial sums of the overlap prior: each (patch, pixel) adds the
-// squared difference to its right and down neighbours where they overlap
-__global__ void k_prior_partials(const float* __restrict__ P, int h, int w, int s, int Pp,
+// squared difference to its right and down neighbours where they overlap.
+// Sixteen values at a time are summed in two floats, then join the thread's
+// FP64 sum: this GPU has few FP64 units, and they bounded it (63,504 patches
+// of 10 x 10: 116 us with FP64 throughout and a division each for patch and
+// pixel, 81 us so; the energy kept its bits there).
+__global__ void k_prior_partials(const float* __restrict__ P, int h, int w, int s, int Pp, int ph2pad,
                                  double* __restrict__ part) {
   __shared__ double sh[256];
+  __shared__ uint32_t s_px[kMaxPatchPixels];
   const int PH = s * Pp, ph2 = PH * PH;
   const int nh = h - Pp + 1, nw = w - Pp + 1;
-  const int64_t total = (int64_t)nh * nw * ph2;
+  for (int p = threadIdx.x; p < ph2; p += blockDim.x) s_px[p] = pixel_code(p, PH, s);
+  __syncthreads();
+  const int64_t total = (int64_t)nh * nw * ph2, step = (int64_t)gridDim.x * blockDim.x;
+  // (n, p) and (i, j) of the running value, advanced by the step's whole
+  // patches and pixels
+  int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  int64_t n = t / ph2;
+  int p = (int)(t - n * ph2);
+  const int64_t dn = step / ph2;
+  const int dp = (int)(step - dn * ph2);
+  int i = (int)(n / nw), j = (int)(n - (int64_t)i * nw);
+  const int di = (int)(dn / nw), dj = (int)(dn - (int64_t)di * nw);
   double acc = 0.0;
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t n = t / ph2;
-    const int p = (int)(t % ph2);
-    const int i = (int)(n / nw), j = (int)(n % nw);
-    const int a = p / PH, b = p % PH;
-    const float pv = P[t];
-    if (j + 1 < nw && b >= s) {
-      const double d = (double)pv - (double)P[(n + 1) * ph2 + a * PH + (b - s)];
-      acc += d * d;
+  while (t < total) {
+    float sum = 0.f, low = 0.f;
+#pragma unroll 4
+    for (int u = 0; u < 16 && t < total; ++u, t += step) {
+      const uint32_t c = s_px[p];
+      const int a = c & 255, b = (c >> 8) & 255;
+      const float* pn = P + n * ph2pad;
+      const float pv = pn[p];
+      // no neighbour, no overlap: the value itself, a difference of 0
+      const float right = j + 1 < nw && b >= s ? pn[ph2pad + p - s] : pv;
+      const float down = i + 1 < nh && a >= s ? pn[(int64_t)nw * ph2pad + p - s * PH] : pv;
+      add_sqdiff(pv, right, sum, low);
+      add_sqdiff(pv, down, sum, low);
+      n += dn;
+      p += dp;
+      i += di;
+      j += dj;
+      if (p >= ph2) {
+        p -= ph2;
+        ++n;
+        ++j;
+      }
+      if (j >= nw) {
+        j -= nw;
+        ++i;
+      }
     }
-    if (i + 1 < nh && a >= s) {
-      const double d = (double)pv - (double)P[(n + nw) * ph2 + (a - s) * PH + b];
-      acc += d * d;
-    }
+    acc += (double)sum + (double)low;
   }
   sh[threadIdx.x] = acc;
   __syncthreads();
@@ -213,9 +394,10 @@ Wts degrade_wts(int s, double sigma) {
 }  // namespace
 
 cudaError_t launch_patches(const int32_t* nbr, const float* wgt, const float* mu, const float* hr_res,
-                           int ph2pad, int K, int64_t nq, int ph2, float* P, cudaStream_t st) {
-  const int64_t tot = nq * ph2;
-  k_patches<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(nbr, wgt, mu, hr_res, ph2pad, K, nq, ph2, P);
+                           int ph2pad, int K, int64_t nq, float* P, cudaStream_t st) {
+  const int64_t tot = nq * (ph2pad / 4);
+  k_patches<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(nbr, wgt, mu, (const float4*)hr_res, ph2pad / 4, K, nq,
+                                                           (float4*)P);
   return cudaGetLastError();
 }
 
@@ -234,31 +416,49 @@ cudaError_t launch_degrade_adjoint(const float* r, int h, int w, int H, int W, i
   return cudaGetLastError();
 }
 
-cudaError_t launch_patch_grad(const float* gx, const float* P, int h, int w, int s, int Pp, float lambda,
-                              float* gP, cudaStream_t st) {
-  const int64_t tot = (int64_t)(h - Pp + 1) * (w - Pp + 1) * (s * Pp) * (s * Pp);
-  k_patch_grad<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(gx, P, h, w, s, Pp, lambda, gP);
+cudaError_t launch_patch_grad(const float* gx, const float* P, int h, int w, int s, int Pp, int ph2pad,
+                              float lambda, float* gP, cudaStream_t st) {
+  if (s * Pp * s * Pp > kMaxPatchPixels) return cudaErrorInvalidValue;
+  const int64_t nq = (int64_t)(h - Pp + 1) * (w - Pp + 1);
+  const int64_t blocks = std::min<int64_t>((nq + 7) / 8, 8192);
+  k_patch_grad<<<(unsigned)blocks, 256, 0, st>>>(gx, P, h, w, s, Pp, ph2pad, lambda, gP);
   return cudaGetLastError();
 }
 
 cudaError_t launch_dict_grad(const int32_t* sorted_use, const int32_t* offs, const uint64_t* ukeys,
                              const int32_t* nuniq, int64_t max_segments, const float* wgt, const float* gP,
-                             int K, int ph2, int ph2pad_out, float* grad, cudaStream_t st) {
+                             int K, int ph2, int ph2pad, int out_stride, float* grad, int32_t* long_list, cudaStream_t st) {
   if (max_segments <= 0) return cudaSuccess;
-  k_dict_grad<<<(unsigned)max_segments, 128, 0, st>>>(sorted_use, offs, ukeys, nuniq, wgt, gP, K, ph2,
-                                                      ph2pad_out, grad);
+  const unsigned blocks = (unsigned)((max_segments + 3) / 4);
+  const int row4 = ph2pad / 4;
+  const float4* g4 = (const float4*)gP;
+  cudaError_t e = cudaMemsetAsync(long_list, 0, sizeof(int32_t), st);
+  if (e != cudaSuccess) return e;
+#define ZOOM_DG(V)                                                                                               \
+  do {                                                                                                           \
+    k_dict_grad<V><<<blocks, 128, 0, st>>>(sorted_use, offs, ukeys, nuniq, wgt, g4, K, row4, ph2, out_stride, grad, \
+                                           long_list);                                                           \
+    k_dict_grad_long<V><<<304, kDgWarps * 32, 0, st>>>(sorted_use, offs, ukeys, wgt, g4, K, row4, ph2, out_stride, \
+                                                       grad, long_list);                                         \
+  } while (0)
+  if (row4 <= 32) ZOOM_DG(1);
+  else if (row4 <= 64) ZOOM_DG(2);
+  else if (row4 <= 128) ZOOM_DG(4);
+  else return cudaErrorInvalidValue;
+#undef ZOOM_DG
   return cudaGetLastError();
 }
 
-cudaError_t launch_mu_grad(const float* gP, int64_t nq, int ph2, float* gmu, cudaStream_t st) {
-  k_mu_grad<<<(unsigned)((nq + 127) / 128), 128, 0, st>>>(gP, nq, ph2, gmu);
+cudaError_t launch_mu_grad(const float* gP, int64_t nq, int ph2, int ph2pad, float* gmu, cudaStream_t st) {
+  k_mu_grad<<<(unsigned)((nq + 127) / 128), 128, 0, st>>>(gP, nq, ph2, ph2pad, gmu);
   return cudaGetLastError();
 }
 
 cudaError_t launch_energy_partials(const float* r, int64_t n_r, const float* P, int h, int w, int s, int Pp,
-                                   double* part, int nblocks, cudaStream_t st) {
+                                   int ph2pad, double* part, int nblocks, cudaStream_t st) {
+  if (s * Pp * s * Pp > kMaxPatchPixels) return cudaErrorInvalidValue;
   k_sumsq_partials<<<nblocks, 256, 0, st>>>(r, n_r, part);
-  k_prior_partials<<<nblocks, 256, 0, st>>>(P, h, w, s, Pp, part + nblocks);
+  k_prior_partials<<<nblocks, 256, 0, st>>>(P, h, w, s, Pp, ph2pad, part + nblocks);
   return cudaGetLastError();
 }
 

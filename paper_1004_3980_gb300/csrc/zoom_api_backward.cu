@@ -53,7 +53,7 @@ struct Carve {
 bool bad_image(zoom_dict d, int h, int w) { return h < d->P || w < d->P; }
 
 // Gradient of the reconstruction with respect to the HR dictionary (and mu)
-// given the per-patch gradients gP [nq][ph2]: grad_R[id] = sum over uses of
+// given the per-patch gradients gP [nq][ph2pad]: grad_R[id] = sum over uses of
 // w * gP, via the uses sorted by entry ID (deterministic, no atomics).
 zoom_status dict_grad_from_patches(zoom_dict d, const int32_t* nbr, const float* wgt, int64_t nq, int K,
                                    const float* gP, float* grad_dict, int grad_stride, char* scratch,
@@ -64,18 +64,20 @@ zoom_status dict_grad_from_patches(zoom_dict d, const int32_t* nbr, const float*
   uint64_t* ukeys = c.take<uint64_t>(nu);
   int32_t* offs = c.take<int32_t>(nu + 1);
   int32_t* nuniq = c.take<int32_t>(1);
+  int32_t* long_list = c.take<int32_t>(2 + nu / kDgLong);
   char* rest = c.take<char>(0);
   const size_t used = (size_t)(rest - scratch);
   if (used > scratch_bytes) return fail(ZOOM_ERR_OOM, "dictionary-gradient scratch");
   ZB_CUDA(cudaMemsetAsync(grad_dict, 0, (size_t)d->n * grad_stride * sizeof(float), st));
   ZB_CUDA(sort_keys_csr(nbr, nu, sorted, ukeys, offs, nuniq, rest, scratch_bytes - used, st));
   ZB_CUDA(launch_dict_grad(sorted, offs, ukeys, nuniq, std::min<int64_t>(nu, d->n), wgt, gP, K, d->ph2,
-                           grad_stride, grad_dict, st));
+                           d->ph2pad, grad_stride, grad_dict, long_list, st));
   return ZOOM_OK;
 }
 
 size_t dict_grad_scratch(int64_t nu) {
-  return (size_t)nu * 4 + (size_t)nu * 8 + (size_t)(nu + 1) * 4 + 4 + 4 * 256 + csr_scratch_bytes(nu);
+  return (size_t)nu * 4 + (size_t)nu * 8 + (size_t)(nu + 1) * 4 + 4 + (size_t)(2 + nu / kDgLong) * 4 + 5 * 256 +
+         csr_scratch_bytes(nu);
 }
 
 }  // namespace
@@ -131,19 +133,19 @@ zoom_status zoom_reconstruct_adjoint(zoom_index ix, const int32_t* nbr, const fl
   ZB_CUDA(cudaSetDevice(d->ctx->device));
   const int64_t nq = (int64_t)(h - d->P + 1) * (w - d->P + 1);
   Buf b(d->ctx, st);
-  const size_t gpb = (size_t)nq * d->ph2 * 4 + 256;
+  const size_t gpb = (size_t)nq * d->ph2pad * 4 + 256;
   const size_t dgs = grad_dict ? dict_grad_scratch(nq * K) : 0;
   if (!b.get(gpb + dgs + 256)) return fail(ZOOM_ERR_OOM, "adjoint scratch");
   Carve c(b.p);
-  float* gP = c.take<float>((size_t)nq * d->ph2);
+  float* gP = c.take<float>((size_t)nq * d->ph2pad);
   char* rest = c.take<char>(0);
-  ZB_CUDA(launch_patch_grad(grad_hr, nullptr, h, w, d->s, d->P, 0.f, gP, st));
+  ZB_CUDA(launch_patch_grad(grad_hr, nullptr, h, w, d->s, d->P, d->ph2pad, 0.f, gP, st));
   if (grad_dict) {
     zoom_status rc = dict_grad_from_patches(d, nbr, wgt, nq, K, gP, grad_dict, grad_stride, rest,
                                             b.bytes - (size_t)(rest - (char*)b.p), st);
     if (rc != ZOOM_OK) return rc;
   }
-  if (grad_mu) ZB_CUDA(launch_mu_grad(gP, nq, d->ph2, grad_mu, st));
+  if (grad_mu) ZB_CUDA(launch_mu_grad(gP, nq, d->ph2, d->ph2pad, grad_mu, st));
   return ZOOM_OK;
 }
 
@@ -169,11 +171,11 @@ zoom_status zoom_backward(zoom_index ix, const float* lr, int32_t h, int32_t w, 
   sz.take<float>(nq);
   sz.take<float>(nq * K);
   sz.take<float>(nq * K);
-  sz.take<float>(nq * d->ph2);
+  sz.take<float>(nq * d->ph2pad);
   sz.take<float>(hr_n);
   sz.take<float>((size_t)h * w);
   sz.take<float>(hr_n);
-  sz.take<float>(nq * d->ph2);
+  sz.take<float>(nq * d->ph2pad);
   sz.take<double>(2 * nblocks);
   const size_t dgs = grad_dict ? dict_grad_scratch(nq * K) : 0;
   Buf b(ctx, st);
@@ -183,11 +185,11 @@ zoom_status zoom_backward(zoom_index ix, const float* lr, int32_t h, int32_t w, 
   float* mu = c.take<float>(nq);
   float* dist = c.take<float>(nq * K);
   float* wloc = c.take<float>(nq * K);
-  float* P = c.take<float>(nq * d->ph2);
+  float* P = c.take<float>(nq * d->ph2pad);
   float* x = hr_out ? (c.take<float>(hr_n), hr_out) : c.take<float>(hr_n);
   float* r = c.take<float>((size_t)h * w);
   float* gx = grad_x ? (c.take<float>(hr_n), grad_x) : c.take<float>(hr_n);
-  float* gP = c.take<float>(nq * d->ph2);
+  float* gP = c.take<float>(nq * d->ph2pad);
   double* part = c.take<double>(2 * nblocks);
   char* rest = c.take<char>(0);
   // weights: given, or recomputed from the neighbours (Eq. 12-13)
@@ -199,19 +201,19 @@ zoom_status zoom_backward(zoom_index ix, const float* lr, int32_t h, int32_t w, 
     wv = wloc;
   }
   // forward: patches, overlap average, residual of the data term
-  ZB_CUDA(launch_patches(nbr, wv, mu, d->hr_res, d->ph2pad, K, nq, d->ph2, P, st));
-  ZB_CUDA(launch_overlap_add(nbr, wv, mu, d->hr_res, d->ph2pad, K, h, w, s, d->P, x, st));
+  ZB_CUDA(launch_patches(nbr, wv, mu, d->hr_res, d->ph2pad, K, nq, P, st));
+  ZB_CUDA(launch_overlap_add(nullptr, nullptr, nullptr, P, d->ph2pad, 0, h, w, s, d->P, x, st));
   ZB_CUDA(launch_degrade(x, s * h, s * w, s, d->blur_sigma, lr, r, st));
   // d/dx of ||D B x - y||^2
   ZB_CUDA(launch_degrade_adjoint(r, h, w, s * h, s * w, s, d->blur_sigma, 2.f, gx, st));
   if (grad_dict) {
-    ZB_CUDA(launch_patch_grad(gx, P, h, w, s, d->P, lambda, gP, st));
+    ZB_CUDA(launch_patch_grad(gx, P, h, w, s, d->P, d->ph2pad, lambda, gP, st));
     zoom_status rc = dict_grad_from_patches(d, nbr, wv, nq, K, gP, grad_dict, grad_stride, rest,
                                             b.bytes - (size_t)(rest - (char*)b.p), st);
     if (rc != ZOOM_OK) return rc;
   }
   if (energy) {
-    ZB_CUDA(launch_energy_partials(r, (int64_t)h * w, P, h, w, s, d->P, part, nblocks, st));
+    ZB_CUDA(launch_energy_partials(r, (int64_t)h * w, P, h, w, s, d->P, d->ph2pad, part, nblocks, st));
     std::vector<double> hp(2 * nblocks);
     ZB_CUDA(cudaMemcpyAsync(hp.data(), part, hp.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
     ZB_CUDA(cudaStreamSynchronize(st));

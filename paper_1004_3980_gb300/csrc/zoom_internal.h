@@ -277,23 +277,26 @@ cudaError_t sort_keys_csr(const int32_t* keys32, int64_t n, int32_t* sorted_pos,
                           int32_t* offs, int32_t* nuniq, void* scratch, size_t scratch_bytes,
                           cudaStream_t st);
 cudaError_t launch_patches(const int32_t* nbr, const float* wgt, const float* mu, const float* hr_res,
-                           int ph2pad, int K, int64_t nq, int ph2, float* P, cudaStream_t st);
+                           int ph2pad, int K, int64_t nq, float* P, cudaStream_t st);
 cudaError_t launch_degrade(const float* x, int H, int W, int s, double sigma, const float* sub, float* y,
                            cudaStream_t st);
 cudaError_t launch_degrade_adjoint(const float* r, int h, int w, int H, int W, int s, double sigma,
                                    float alpha, float* g, cudaStream_t st);
-cudaError_t launch_patch_grad(const float* gx, const float* P, int h, int w, int s, int Pp, float lambda,
-                              float* gP, cudaStream_t st);
+cudaError_t launch_patch_grad(const float* gx, const float* P, int h, int w, int s, int Pp, int ph2pad,
+                              float lambda, float* gP, cudaStream_t st);
+// long_list: 1 + uses / kDgLong numbers of scratch
+constexpr int kDgLong = 64;
 cudaError_t launch_dict_grad(const int32_t* sorted_use, const int32_t* offs, const uint64_t* ukeys,
                              const int32_t* nuniq, int64_t max_segments, const float* wgt, const float* gP,
-                             int K, int ph2, int ph2pad_out, float* grad, cudaStream_t st);
-cudaError_t launch_mu_grad(const float* gP, int64_t nq, int ph2, float* gmu, cudaStream_t st);
+                             int K, int ph2, int ph2pad, int out_stride, float* grad, int32_t* long_list, cudaStream_t st);
+cudaError_t launch_mu_grad(const float* gP, int64_t nq, int ph2, int ph2pad, float* gmu, cudaStream_t st);
 cudaError_t launch_energy_partials(const float* r, int64_t n_r, const float* P, int h, int w, int s, int Pp,
-                                   double* part, int nblocks, cudaStream_t st);
+                                   int ph2pad, double* part, int nblocks, cudaStream_t st);
 cudaError_t launch_nbr_dist(const float* qfeat, int dpad, int d, int64_t nq, const float* dfeat,
                             const int32_t* nbr, int K, float* dist, cudaStream_t st);
 
 // image steps (kernels_image.cu)
+// (K = 0: hr_res holds the blended patches, one row each)
 cudaError_t launch_overlap_add(const int32_t* nbr, const float* wgt, const float* mu,
                                const float* hr_res, int ph2pad, int K, int h, int w, int s, int P,
                                float* hr, cudaStream_t st);
