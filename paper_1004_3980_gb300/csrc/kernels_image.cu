@@ -202,21 +202,57 @@ struct Wts1D {
   float w[8];
 };
 
-__global__ void k_bp_error(const float* __restrict__ x, int H, int W, const float* __restrict__ y,
-                           int h, int w, int s, Wts1D wt, float* __restrict__ e) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  const int i = blockIdx.y * blockDim.y + threadIdx.y;
+// An NR x NC window of x at (r0, c0) into shared memory, borders clamped: all of
+// a thread's loads are issued before the first is stored.
+template <int NR, int NC, int STRIDE>
+__device__ __forceinline__ void load_window(const float* __restrict__ x, int H, int W, int r0, int c0, int tid,
+                                            float (*dst)[STRIDE]) {
+  constexpr int N = NR * NC, IT = (N + 255) / 256;
+  float v[IT];
+#pragma unroll
+  for (int k = 0; k < IT; ++k) {
+    const int i = min(tid + k * 256, N - 1);
+    const int r = i / NC, c = i - r * NC;
+    v[k] = __ldg(x + (int64_t)zoom_clampi(r0 + r, 0, H - 1) * W + zoom_clampi(c0 + c, 0, W - 1));
+  }
+#pragma unroll
+  for (int k = 0; k < IT; ++k) {
+    const int i = tid + k * 256;
+    if (i < N) dst[i / NC][i % NC] = v[k];
+  }
+}
+
+// A block takes 32 x 8 LR pixels: their HR rows and columns in shared memory
+// (clamped), the weighted row sums of every HR row, then the column sums; the
+// same products and sums in the same order for every pixel as one thread's
+// double loop.  Bound by the image read once; with each thread reading its
+// (s + 2)^2 values from memory 1920 x 1080 at 3x took 61 us, and as much
+// with one load of the window in flight a thread; 32 us so.
+constexpr int kErrW = 32, kErrH = 8;
+
+template <int S>
+__global__ void __launch_bounds__(256) k_bp_error(const float* __restrict__ x, int H, int W,
+                                                  const float* __restrict__ y, int h, int w, Wts1D wt,
+                                                  float* __restrict__ e) {
+  constexpr int NR = S * kErrH + 2, NC = S * kErrW + 2;
+  __shared__ float xs[NR][NC];
+  __shared__ float rows[NR][kErrW];
+  const int j0 = blockIdx.x * kErrW, i0 = blockIdx.y * kErrH;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  load_window<NR, NC, NC>(x, H, W, S * i0 - 1, S * j0 - 1, tid, xs);
+  __syncthreads();
+  for (int r = warp; r < NR; r += kErrH) {
+    float row = 0.f;
+#pragma unroll
+    for (int b = 0; b < S + 2; ++b) row = fmaf(wt.w[b], xs[r][S * lane + b], row);
+    rows[r][lane] = row;
+  }
+  __syncthreads();
+  const int i = i0 + warp, j = j0 + lane;
   if (i >= h || j >= w) return;
   float acc = 0.f;
-  for (int a = 0; a < wt.n; ++a) {
-    const int r = zoom_clampi(s * i + a - 1, 0, H - 1);
-    float row = 0.f;
-    for (int b = 0; b < wt.n; ++b) {
-      const int c = zoom_clampi(s * j + b - 1, 0, W - 1);
-      row = fmaf(wt.w[b], x[(int64_t)r * W + c], row);
-    }
-    acc = fmaf(wt.w[a], row, acc);
-  }
+#pragma unroll
+  for (int a = 0; a < S + 2; ++a) acc = fmaf(wt.w[a], rows[S * warp + a][lane], acc);
   e[(int64_t)i * w + j] = acc - y[(int64_t)i * w + j];
 }
 
@@ -235,7 +271,11 @@ struct Gauss1D {
 // double loop (columns t within a row, then rows u), so the result is the
 // same bit for bit; x is read from memory once (with the halo) instead of
 // (2R+1)^2 times, and the LR row and column of every clamped tile row and
-// column are computed once per block.
+// column are computed once per block.  Bound by shared-memory reads: a thread
+// sums eight neighbouring columns of a row, then eight neighbouring rows of a
+// column, from registers, and a thread's loads are issued together (5760 x
+// 3240, R = 3: 125 us with 2R + 1 reads a sum and one load in flight, 93 us so;
+// issue-bound now).
 constexpr int kBpTileW = 32, kBpTileH = 64;
 template <int R>
 __global__ void __launch_bounds__(256) k_bp_update(const float* __restrict__ x, float* __restrict__ xo, int H,
@@ -243,8 +283,10 @@ __global__ void __launch_bounds__(256) k_bp_update(const float* __restrict__ x, 
                                                    float inv_two_sr2) {
   constexpr int T = 2 * R + 1;
   constexpr int NW = kBpTileW + 2 * R, NH = kBpTileH + 2 * R;   // the tile with its halo
-  __shared__ float xs[NH][NW + 1];      // x, clamped
-  __shared__ float hs[NH][kBpTileW];    // row box sums
+  constexpr int kRun = 8;               // columns, then rows, a thread sums side by side
+  constexpr int XP = (NW | 1);          // odd strides: lanes on neighbouring rows hit different banks
+  __shared__ float xs[NH][XP];          // x, clamped
+  __shared__ float hs[NH][kBpTileW + 1];   // row box sums
   __shared__ float hg[NH][kBpTileW];    // per LR row: Gaussian row sums of the replicated error
   __shared__ int lrow[NH], lcol[NW];    // LR row (relative to lr0) / column of each clamped tile row / column
   const int X0 = blockIdx.x * kBpTileW, Y0 = blockIdx.y * kBpTileH;
@@ -253,10 +295,7 @@ __global__ void __launch_bounds__(256) k_bp_update(const float* __restrict__ x, 
   const int nlr = zoom_clampi(Y0 + kBpTileH - 1 + R, 0, H - 1) / s - lr0 + 1;
   for (int i = tid; i < NH; i += 256) lrow[i] = zoom_clampi(Y0 - R + i, 0, H - 1) / s - lr0;
   for (int i = tid; i < NW; i += 256) lcol[i] = zoom_clampi(X0 - R + i, 0, W - 1) / s;
-  for (int i = tid; i < NH * NW; i += 256) {
-    const int r = i / NW, c = i % NW;
-    xs[r][c] = x[(int64_t)zoom_clampi(Y0 - R + r, 0, H - 1) * W + zoom_clampi(X0 - R + c, 0, W - 1)];
-  }
+  load_window<NH, NW, XP>(x, H, W, Y0 - R, X0 - R, tid, xs);
   __syncthreads();
   for (int i = tid; i < nlr * kBpTileW; i += 256) {
     const int r = i / kBpTileW, c = i % kBpTileW;
@@ -266,28 +305,42 @@ __global__ void __launch_bounds__(256) k_bp_update(const float* __restrict__ x, 
     for (int t = 0; t < T; ++t) grow = fmaf(g.c[t], er[lcol[c + t]], grow);
     hg[r][c] = grow;
   }
-  for (int i = tid; i < NH * kBpTileW; i += 256) {
-    const int r = i / kBpTileW, c = i % kBpTileW;
-    float brow = 0.f;
+  for (int i = tid; i < NH * (kBpTileW / kRun); i += 256) {
+    const int r = i % NH, c = i / NH * kRun;
+    float v[kRun + 2 * R];
 #pragma unroll
-    for (int t = 0; t < T; ++t) brow += xs[r][c + t];
-    hs[r][c] = brow;
+    for (int t = 0; t < kRun + 2 * R; ++t) v[t] = xs[r][c + t];
+#pragma unroll
+    for (int k = 0; k < kRun; ++k) {
+      float brow = 0.f;
+#pragma unroll
+      for (int t = 0; t < T; ++t) brow += v[k + t];
+      hs[r][c + k] = brow;
+    }
   }
   __syncthreads();
-  const int c = threadIdx.x;
+  static_assert(kBpTileH == kRun * 8 && kBpTileW == 32, "one run of rows a thread");
+  const int c = threadIdx.x, y0 = threadIdx.y * kRun;
   const int X = X0 + c;
   if (X >= W) return;
-  for (int y = threadIdx.y; y < kBpTileH; y += blockDim.y) {
-    const int Y = Y0 + y;
+  float b[kRun + 2 * R], q[kRun + 2 * R];
+#pragma unroll
+  for (int t = 0; t < kRun + 2 * R; ++t) {
+    b[t] = hs[y0 + t][c];
+    q[t] = hg[lrow[y0 + t]][c];
+  }
+#pragma unroll
+  for (int k = 0; k < kRun; ++k) {
+    const int Y = Y0 + y0 + k;
     if (Y >= H) break;
     float gs = 0.f, box = 0.f;
 #pragma unroll
     for (int u = 0; u < T; ++u) {
-      gs = fmaf(g.c[u], hg[lrow[y + u]][c], gs);
-      box += hs[y + u][c];
+      gs = fmaf(g.c[u], q[k + u], gs);
+      box += b[k + u];
     }
     const float m = box / (float)(T * T);
-    const float xv = xs[y + R][c + R];
+    const float xv = xs[y0 + k + R][c + R];
     const float dv = xv - m;
     const float r = expf(-dv * dv * inv_two_sr2);
     xo[(int64_t)Y * W + X] = xv - r * gs;
@@ -353,8 +406,14 @@ cudaError_t launch_bp_iteration(const float* x, float* x_out, const float* lr, f
     for (int d = 0; d < 16; ++d) g.c[d] = d < 2 * radius + 1 ? (float)(c[d] / tot) : 0.f;
   }
   dim3 blk(32, 8);
-  dim3 g1((w + 31) / 32, (h + 7) / 8);
-  k_bp_error<<<g1, blk, 0, st>>>(x, H, W, lr, h, w, s, wt, err);
+  dim3 g1((w + kErrW - 1) / kErrW, (h + kErrH - 1) / kErrH);
+  switch (s) {
+    case 1: k_bp_error<1><<<g1, 256, 0, st>>>(x, H, W, lr, h, w, wt, err); break;
+    case 2: k_bp_error<2><<<g1, 256, 0, st>>>(x, H, W, lr, h, w, wt, err); break;
+    case 3: k_bp_error<3><<<g1, 256, 0, st>>>(x, H, W, lr, h, w, wt, err); break;
+    case 4: k_bp_error<4><<<g1, 256, 0, st>>>(x, H, W, lr, h, w, wt, err); break;
+    default: return cudaErrorInvalidValue;
+  }
   dim3 g2((W + kBpTileW - 1) / kBpTileW, (H + kBpTileH - 1) / kBpTileH);
   const float inv = (float)(1.0 / (2.0 * (double)sigma_r * (double)sigma_r));
   switch (radius) {
