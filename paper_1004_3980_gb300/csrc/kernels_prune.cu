@@ -4,8 +4,8 @@
 //
 // Steps, for queries sorted along the same tree (neighbouring queries need
 // nearly the same tiles):
-//  1. seeds: 256 queries at a time against the 32 tiles nearest their mean
-//     (the dense wide-step filter over a tile list); the r-th smallest chunk
+//  1. seeds: 256 queries at a time against 64 tiles near them (k_seed_tiles;
+//     the dense wide-step filter over a tile list); the r-th smallest chunk
 //     minimum, r a little above K, is the query's radius T;
 //  2. visits: every (query, tile) pair whose box bound does not exceed T,
 //     appended to the tile's query list (k_visit);

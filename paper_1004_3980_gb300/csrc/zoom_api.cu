@@ -420,7 +420,8 @@ zoom_status zoom_build_index(zoom_dict d, const zoom_lsh_params* lsh, const floa
     ix->tree_tiles = (N + 255) / 256;
     tree_depths(N, &ix->tree_d1, &ix->tree_d2);
   }
-  const int64_t nt = ix->tree_tiles, ns = (nt + 15) / 16;
+  int64_t nt = ix->tree_tiles;
+  const int64_t ns = (nt + 15) / 16;
   auto carve_tree = [&](Carver& c) {
     if (!nt) return;
     ix->tree_basis = c.take<float>((size_t)d->d * 16);
@@ -434,7 +435,7 @@ zoom_status zoom_build_index(zoom_dict d, const zoom_lsh_params* lsh, const floa
     ix->tree_mid = c.take<float>(nt * 16);
     ix->tree_smid = c.take<float>(ns * 16);
   };
-  {
+  auto count_bytes = [&]() {
     Carver c(nullptr);
     c.take<float>((size_t)L * k * d->d);
     c.take<float>((size_t)L * k);
@@ -447,9 +448,15 @@ zoom_status zoom_build_index(zoom_dict d, const zoom_lsh_params* lsh, const floa
     c.take<uint16_t>(ix->nd_rows * tc_kc(d->d, 1) * 8);
     c.take<uint16_t>(ix->nd_rows * tc_kc(d->d, 2) * 8);
     carve_tree(c);
-    ix->bytes = c.off + 256;
-  }
+    return c.off + 256;
+  };
+  ix->bytes = count_bytes();
   void* mem = zoom_alloc(ctx, ix->bytes, st);
+  if (!mem && nt) {   // no room for the search order (4 + 128 bytes an entry at D <= 25): an index without
+    nt = ix->tree_tiles = 0;
+    ix->bytes = count_bytes();
+    mem = zoom_alloc(ctx, ix->bytes, st);
+  }
   if (!mem) {
     delete ix;
     return fail(ZOOM_ERR_OOM, "index arrays");
@@ -480,7 +487,12 @@ zoom_status zoom_build_index(zoom_dict d, const zoom_lsh_params* lsh, const floa
   if (e == cudaSuccess) {
     Scratch scr(ctx, st);
     const size_t sb = csr_build_scratch_bytes(N, L), tb = nt ? tree_scratch_bytes(N) : 0;
-    if (!scr.get(std::max(sb, tb))) {   // one after the other on the stream
+    bool got = scr.get(std::max(sb, tb));   // one after the other on the stream
+    if (!got && tb > sb) {
+      nt = ix->tree_tiles = 0;
+      got = scr.get(sb);
+    }
+    if (!got) {
       rc = fail(ZOOM_ERR_OOM, "index build scratch");
     } else {
       if (nt) e = build_search_tree(ix, scr.p, tb, st);

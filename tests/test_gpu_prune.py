@@ -127,6 +127,27 @@ def test_refused_query_lists_fall_back_to_the_dense_search():
     assert torch.equal(got["nbr"], ref["nbr"]) and torch.equal(got["dist"], ref["dist"])
 
 
+def test_index_without_room_for_the_search_order():
+    import paper_1004_3980_gb300 as Z
+    A = Limited()
+    train = [S.make_image(300 + i, 256, 256) for i in range(10)]
+    pos = S.sample_positions(5, 10, 128, 128, 5, 70000)
+    a, b = S.lsh_draws(6, 8, 12, 25, 4.0)
+    ctx = Z.Context(0, allocator=A)
+    dic = Z.Dictionary(ctx, [torch.from_numpy(x).cuda() for x in train], pos, 2, 5)
+    A.sizes = []
+    ref = Z.Index(dic, 8, 12, 4.0, a, b)
+    A.limit = max(A.sizes) - 1   # the index arrays with the order
+    ix = Z.Index(dic, 8, 12, 4.0, a, b)
+    assert A.refused == 1
+    A.limit = None
+    lr = torch.from_numpy(S.make_image(1, 151, 163)).cuda()
+    for prec in (0, 1):
+        p = Z.UpscaleParams(K=8, precision=prec)
+        got, want = Z.query(ix, lr, p), Z.query(ref, lr, p)
+        assert torch.equal(got["nbr"], want["nbr"]) and torch.equal(got["dist"], want["dist"])
+
+
 def test_batch_equals_single_images():
     import paper_1004_3980_gb300 as Z
     ctx, ix = _build(70001)
