@@ -388,8 +388,23 @@ def launches_per_step(wl: S.Workload, precision: int) -> int:
     (gather, split operand, split filter, rerank), the SIMT re-run and the
     fallback-count update (9); BF16 form: operand, filter, rerank, SIMT
     re-run, fallback count (5) --; LLE, the two overlap-average passes, and
-    two per back-projection step."""
+    two per back-projection step.  Searches over the dictionary's search
+    order launch order_launches() more."""
     return 3 + (9 if precision == 0 else 5) + 3 + 2 * wl.bp_iters
+
+
+def order_launches(nq: int, n_pairs: int, precision: int) -> int:
+    """Kernels that a search of nq queries over the search order launches
+    beyond the dense search's (0 where the dense one is taken): queries
+    sorted (3), seeds (2) and radii; per round of queries the visits, the
+    steps (2), the list filter and the rerank; the queries left over through
+    the dense filter in two parts (gather, operand, filter, lists joined,
+    rerank each), the SIMT re-run and the fallback count."""
+    if not 65_536 <= n_pairs <= 2048 * 16 * 256 or (nq < 20_000 and nq * n_pairs < 2_500_000_000):
+        return 0
+    tiles = -(-n_pairs // 256)
+    per_round = min(2**31 // (2 * tiles) // 256 * 256, 65_280, -(-nq // 256) * 256)
+    return 6 + 5 * -(-nq // per_round) + 10 + 2 - (9 if precision == 0 else 5)
 
 
 def max_over_ranks(ms: float, world: int, device: str) -> float:
@@ -583,6 +598,17 @@ def run_single(a, wl, config, rank, world, local):
     def filt_roofline(kernel, kms, kdepth, form):
         if kms <= 0:
             return None
+        if order_launches(nq, wl.n_pairs, 1):
+            # the search over the search order skips most pairs, so a rate over all of them would exceed the
+            # peak: the bytes it cannot do without, each dictionary and query feature read once and the
+            # neighbours written, over the stage's time
+            byts = 4 * (wl.n_pairs + nq) * wl.patch ** 2 + 8 * nq * wl.K
+            gbs = byts / (kms / 1e3) / 1e9
+            return {"kernel": "k_knn_tw (seeds), k_radius, k_visit, k_step_scan, k_steps, k_knn_tg, k_rerank_list",
+                    "bound": "issue and hand-offs (not HBM)", "achieved": gbs, "peak": hbm_peak, "unit": "GB/s",
+                    "frac": gbs / hbm_peak, "kernel_ms": kms,
+                    "work": f"features of {wl.n_pairs} entries and {nq} queries read once, neighbours written",
+                    "dense_pairs": dense, "dense_note": "pairs a dense search computes; most are skipped here"}
         ach = pairs * 2.0 * kdepth / (kms / 1e3) / 1e12
         ach_dense = dense * 2.0 * kdepth / (kms / 1e3) / 1e12
         return {"kernel": kernel, "bound": "tensor", "achieved": ach, "peak": tc_peak, "unit": "TFLOP/s",
@@ -599,7 +625,7 @@ def run_single(a, wl, config, rank, world, local):
                           stage_bf.get("knn_filter_kernel", 0.0), 32, "one BF16 term, K = 32 per pair")
     rf_ex = filt_roofline("k_knn_tw<4,16,0> (tcgen05 M128 x N256 single-term FP16 filter of the exact form)",
                           stage_ex.get("knn_filter_kernel", 0.0), 32, "one FP16 term, K = 32 per pair")
-    if rf_bf:
+    if rf_bf and rf_bf["bound"] == "tensor":
         rf_bf["traffic"] = profiled_traffic("paper_1004_3980_gb300/csrc/kernels_tc.cu",
                                             "profiles/knn_tw_bf16_zoom3x_1920x1080_dict4m.md")
         rf_bf["traffic_source"] = ("ncu dram__bytes_read.sum + dram__bytes_write.sum per launch "
@@ -618,7 +644,10 @@ def run_single(a, wl, config, rank, world, local):
     # queries).  Algorithmic bytes: the FP32 rows of the top 4K candidates gathered per query; the kernel
     # reads whole 32-row chunks instead (from L2 mostly), about 8 of them per query
     rr_ms = stage_bf.get("knn", 0.0) - stage_bf.get("knn_filter_kernel", 0.0)
-    if rr_ms > 0:
+    if order_launches(nq, wl.n_pairs, 1):
+        kernels["search_rest"] = {"ms": rr_ms, "note": "queries sorted and seeded before, the queries left over "
+                                                       "searched densely after the timed filter stage"}
+    elif rr_ms > 0:
         rr_bytes = nq * 4 * wl.K * wl.patch ** 2 * 4
         gbs = rr_bytes / (rr_ms / 1e3) / 1e9
         kernels["rerank"] = {"ms": rr_ms, "algorithmic_bytes": rr_bytes, "GB/s": gbs, "frac_hbm": gbs / hbm_peak,
@@ -639,11 +668,11 @@ def run_single(a, wl, config, rank, world, local):
                           "lr_patch_queries_per_s": world * nq / (ms_ex / 1e3), "dtype": "f32",
                           "roofline": rf_ex, "stage_ms_per_step": stage_ex, "clocks": clk_ex,
                           "filter_fallback_queries": stats_ex["n_filter_fallback"],
-                          "gpu_launches_per_step": launches_per_step(wl, 0)},
+                          "gpu_launches_per_step": launches_per_step(wl, 0) + order_launches(nq, wl.n_pairs, 0)},
            "bf16_speedup_over_fp32_exact": ms_ex / ms_bf,
            "bf16_vs_fp32_exact": bf_vs_ex, "vs_oracle": vs_oracle,
            "roofline": rf_bf, "kernels_hbm": kernels, "e2e": e2e,
-           "gpu_launches": launches_per_step(wl, 1) * a.steps, "clocks": clk,
+           "gpu_launches": (launches_per_step(wl, 1) + order_launches(nq, wl.n_pairs, 1)) * a.steps, "clocks": clk,
            "stage_ms_per_step": stage_bf, "mean_candidate_fraction": frac_c,
            "mean_bucket_sum_per_query": stats_bf["mean_bucket_sum"],
            "dictionary_build_ms": dict_ms, "index_build_ms": index_ms,
@@ -709,8 +738,11 @@ def all_extras(a, wl, ctx, d, ix, lr, hr_exact, params, train, pos, st, world, h
     for _ in range(2):
         Z.upscale(ixg, lr, pg, out=out)
     ms4 = timed_steps(lambda: Z.upscale(ixg, lr, pg, out=out), a.steps, st, torch, world)
-    fg = stage_profile(ctx, lambda: Z.upscale(ixg, lr, pg, out=out)).get("knn_filter_kernel", 0.0)
+    Z.upscale(ixg, lr, pg, out=out)
     st_g = ctx.stats()
+    # the filter's rate: the dense search, which computes every pair
+    pd = params(search=2)
+    fg = stage_profile(ctx, lambda: Z.upscale(ixg, lr, pd, out=out)).get("knn_filter_kernel", 0.0)
     ach_g = nq * wl.n_pairs * 2.0 * 64 / (fg / 1e3) / 1e12 if fg > 0 else None
     res["gradient_features"] = {
         "value": world * hr_px / 1e6 / (ms4 / 1e3), "unit": UNIT, "ms_per_step": ms4,
@@ -775,6 +807,8 @@ def run_batch(a, rank, world, local, steps: int, warmup: int):
     lrs = [(s, torch.from_numpy(x).cuda()) for s, x in lr_np]
     hr_px = sum(s * s * x.shape[0] * x.shape[1] for s, x in lrs)
     nq = sum((x.shape[0] - 4) * (x.shape[1] - 4) for _, x in lrs)
+    more = sum(order_launches(sum((x.shape[0] - 4) * (x.shape[1] - 4) for s2, x in lrs if s2 == s), 1_000_000, 1)
+               for s in (2, 3))
     # the batched form's lists: the best 16 chunks (rerank_mult * K = 16;
     # the best-32 reading belongs to the single 3x image)
     p1 = Z.UpscaleParams(K=8, bp_iters=5, precision=1, rerank_mult=2)
@@ -842,7 +876,7 @@ def run_batch(a, rank, world, local, steps: int, warmup: int):
             "fp32_exact_batch": {"value": world * hr_px / 1e6 / (ms_exact / 1e3), "ms_per_batch": ms_exact,
                                  "identical_to_exact_loop": same},
             "psnr_bf16_batch_vs_fp32_exact_db": 10 * np.log10(1.0 / max(mse, 1e-30)),
-            "clocks": clk, "gpu_launches": batch_launches(shapes, 5, 1) * steps,
+            "clocks": clk, "gpu_launches": (batch_launches(shapes, 5, 1) + more) * steps,
             "e2e": {"value": world * hr_px / 1e6 / e2e_s, "unit": UNIT, "h2d_bytes_per_step": h2d,
                     "d2h_bytes_per_step": d2h}}
 
