@@ -312,7 +312,8 @@ zoom_status zoom_upscale(zoom_index ix, const float* lr, int32_t h, int32_t w, i
  * may change).  per_image_ms (host, optional): device time from the start of
  * the batch to the completion of image i (synchronises `stream`).  The
  * recording keeps its scratch memory until zoom_batch_release, a call with
- * a different set, or zoom_ctx_destroy. */
+ * a different set, zoom_index_destroy of one of its indexes (which then
+ * synchronises the device), or zoom_ctx_destroy. */
 zoom_status zoom_upscale_batch(const zoom_index* ixs, int32_t n_indexes, int32_t n_images,
                                const float* const* lr, const int32_t* h, const int32_t* w,
                                const int32_t* scale, const zoom_upscale_params* prm,

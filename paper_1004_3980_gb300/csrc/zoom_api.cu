@@ -514,6 +514,7 @@ zoom_status zoom_build_index(zoom_dict d, const zoom_lsh_params* lsh, const floa
 void zoom_index_destroy(zoom_index ix) {
   if (!ix) return;
   cudaSetDevice(ix->dict->ctx->device);
+  zoom_forget_index(ix->dict->ctx, ix);
   ix->dict->index_refs--;
   zoom_free(ix->dict->ctx, ix->alpha, ix->bytes, nullptr);
   delete ix;
@@ -1246,6 +1247,23 @@ void release_batch(zoom_ctx ctx) {
   free_record(ctx, r);
   ctx->batch = nullptr;
 }
+
+}  // namespace
+
+// The recorded batch reads the index's arrays and is found by the handle's
+// address, which a later index may get; so are the tuned choices.
+void zoom_forget_index(zoom_ctx ctx, zoom_index ix) {
+  if (BatchRecord* r = (BatchRecord*)ctx->batch)
+    for (const Group& g : r->groups)
+      if (g.ix == ix) {
+        release_batch(ctx);
+        break;
+      }
+  if (TuneMap* tm = (TuneMap*)ctx->tuned)
+    for (auto it = tm->begin(); it != tm->end();) it = it->first.ix == ix ? tm->erase(it) : std::next(it);
+}
+
+namespace {
 
 int64_t qbucket(int64_t nq) {
   int64_t b = 1;

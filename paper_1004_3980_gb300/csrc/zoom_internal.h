@@ -49,6 +49,8 @@ struct zoom_ctx_s {
 void zoom_stage_mark(zoom_ctx ctx, int i, cudaStream_t st);
 // Frees the context's recorded batch and autotuning choices.
 void zoom_release_batch(zoom_ctx ctx);
+// Frees what of these refers to an index (before its memory is freed).
+void zoom_forget_index(zoom_ctx ctx, zoom_index ix);
 
 struct zoom_dict_s {
   zoom_ctx ctx = nullptr;

@@ -1,0 +1,71 @@
+"""The recorded batch of a context (zoom_upscale_batch) and its tuned search
+choices: a record is replayed only for the call it was made from, and neither
+outlives what it refers to."""
+import numpy as np
+import pytest
+
+import synth_inputs as S
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+class LiveAllocator:
+    """PyTorch's caching allocator with the live allocations recorded."""
+
+    def __init__(self):
+        self.live = {}
+
+    def alloc(self, nbytes, stream, user):
+        p = torch.cuda.caching_allocator_alloc(int(nbytes), 0, int(stream or 0))
+        self.live[p] = int(nbytes)
+        return p
+
+    def free(self, ptr, nbytes, stream, user):
+        assert self.live.pop(ptr) == nbytes
+        torch.cuda.caching_allocator_delete(ptr)
+
+
+def _context():
+    import paper_1004_3980_gb300 as Z
+    A = LiveAllocator()
+    return Z.Context(0, allocator=A), A
+
+
+def _index(ctx, n_pairs=5000, n_train=3, hr=96):
+    import paper_1004_3980_gb300 as Z
+    train = [S.make_image(3000 + i, hr, hr) for i in range(n_train)]
+    pos = S.sample_positions(7, n_train, hr // 2, hr // 2, 5, n_pairs)
+    alpha, beta = S.lsh_draws(11, 8, 10, 25, 4.0)
+    d = Z.Dictionary(ctx, [torch.from_numpy(x).cuda() for x in train], pos, 2, 5)
+    return Z.Index(d, 8, 10, 4.0, alpha, beta)
+
+
+def _images(*shapes):
+    return [(2, torch.from_numpy(S.make_image(3100 + i, h, w)).cuda()) for i, (h, w) in enumerate(shapes)]
+
+
+def test_destroying_an_index_frees_the_batch_recorded_from_it():
+    # (seen in the allocator: the graph of a destroyed index is never run)
+    import paper_1004_3980_gb300 as Z
+    ctx, A = _context()
+    ix = _index(ctx)
+    other = _index(ctx)
+    torch.cuda.synchronize()
+    held = dict(A.live)
+    p = Z.UpscaleParams(K=8, bp_iters=1)
+    lrs = _images((20, 24), (31, 17))
+    outs, _ = Z.upscale_batch([ix], lrs, p)
+    torch.cuda.synchronize()
+    record = {a: n for a, n in A.live.items() if a not in held}
+    assert record
+    other.close()                                  # not the record's: it stays
+    assert all(A.live.get(a) == n for a, n in record.items())
+    ix.close()
+    assert not any(a in A.live for a in record)
+    ix = _index(ctx)                               # the same sizes: the handle's address may come back
+    got, _ = Z.upscale_batch([ix], lrs, p, outs=outs)
+    for (_, x), o in zip(lrs, got):
+        assert torch.equal(o, Z.upscale(ix, x, p))
+    Z.batch_release(ctx)
