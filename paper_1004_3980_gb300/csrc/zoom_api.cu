@@ -1265,6 +1265,13 @@ void zoom_forget_index(zoom_ctx ctx, zoom_index ix) {
 
 namespace {
 
+template <typename T>
+int64_t float_bits(T x) {
+  int64_t v = 0;
+  memcpy(&v, &x, sizeof(x));
+  return v;
+}
+
 int64_t qbucket(int64_t nq) {
   int64_t b = 1;
   while (b < nq) b <<= 1;
@@ -1365,10 +1372,12 @@ zoom_status zoom_upscale_batch(const zoom_index* ixs, int32_t n_indexes, int32_t
                       (int64_t)scale[i]})
       key.push_back(v);
   }
+  // what the launches carry besides: every parameter, the floating ones by
+  // their bits, and the waits' testing aids
   for (int64_t v : {(int64_t)prm->K, (int64_t)prm->bp_iters, (int64_t)prm->precision,
                     (int64_t)prm->rerank_mult, (int64_t)prm->search, (int64_t)prm->bp_radius,
-                    (int64_t)(prm->reg_rel * 1e9f), (int64_t)(prm->sigma_spatial * 1e6f),
-                    (int64_t)(prm->sigma_range * 1e6f)})
+                    float_bits(prm->reg_rel), float_bits(prm->sigma_spatial), float_bits(prm->sigma_range),
+                    float_bits(prm->fp64_cond_threshold), (int64_t)ctx->inject, (int64_t)ctx->wait_ns})
     key.push_back(v);
   if (!ctx->tuned) ctx->tuned = new TuneMap();
   BatchRecord* rec = (BatchRecord*)ctx->batch;

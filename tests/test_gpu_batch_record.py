@@ -69,3 +69,28 @@ def test_destroying_an_index_frees_the_batch_recorded_from_it():
     for (_, x), o in zip(lrs, got):
         assert torch.equal(o, Z.upscale(ix, x, p))
     Z.batch_release(ctx)
+
+
+@pytest.mark.parametrize("change", [dict(fp64_cond_threshold=1.0), dict(reg_rel=9e-10), dict(sigma_spatial=1.5000005)],
+                         ids=lambda c: next(iter(c)))
+def test_a_changed_parameter_is_not_a_replay(change):
+    # each call's images must be those of single calls with its parameters
+    import dataclasses
+    import paper_1004_3980_gb300 as Z
+    ctx, _ = _context()
+    ix = _index(ctx)
+    p = Z.UpscaleParams(K=8, bp_iters=2, reg_rel=2e-10 if "reg_rel" in change else 1e-3)
+    lrs = _images((40, 44), (31, 17))
+    outs, _ = Z.upscale_batch([ix], lrs, p)
+    first = [o.clone() for o in outs]
+    q = dataclasses.replace(p, **change)
+    outs, _ = Z.upscale_batch([ix], lrs, q, outs=outs)
+    second = [o.clone() for o in outs]
+    n_fp64 = ctx.stats()["n_fp64_solves"]
+    for (_, x), a, b in zip(lrs, first, second):
+        assert torch.equal(a, Z.upscale(ix, x, p))
+        assert torch.equal(b, Z.upscale(ix, x, q))
+    assert not all(torch.equal(a, b) for a, b in zip(first, second))
+    if "fp64_cond_threshold" in change:
+        assert n_fp64 > 0
+    Z.batch_release(ctx)
