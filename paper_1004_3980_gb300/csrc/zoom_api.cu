@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <map>
 #include <string>
+#include <tuple>
 #include <vector>
 
 #include "zoom_internal.h"
@@ -1176,17 +1177,16 @@ zoom_status zoom_sync_status(zoom_ctx ctx, void* stream) {
 
 namespace {
 
-// Search choices picked by the autotuner, per (index, query count bucket,
-// precision, K).
+// Search choices picked by the autotuner, per index, query count bucket and
+// the parameters that decide the searches it compares (the precision form's
+// list size follows from rerank_mult, so a choice for one is none for another).
 struct TuneKey {
   const void* ix;
   int64_t qbucket;
-  int prec, K;
+  int prec, K, rerank_mult, search;
   bool operator<(const TuneKey& o) const {
-    if (ix != o.ix) return ix < o.ix;
-    if (qbucket != o.qbucket) return qbucket < o.qbucket;
-    if (prec != o.prec) return prec < o.prec;
-    return K < o.K;
+    return std::tie(ix, qbucket, prec, K, rerank_mult, search) <
+           std::tie(o.ix, o.qbucket, o.prec, o.K, o.rerank_mult, o.search);
   }
 };
 struct TuneChoice {
@@ -1278,13 +1278,17 @@ int64_t qbucket(int64_t nq) {
   return b;
 }
 
+TuneKey tune_key(const Group& g, const zoom_upscale_params* prm) {
+  return TuneKey{g.ix, qbucket(g.nq), prm->precision, prm->K, prm->rerank_mult, prm->search};
+}
+
 // Times each candidate (splits x list size) of one group's search on a
 // sample of its queries and remembers the fastest.
 zoom_status autotune_group(Group& g, const zoom_upscale_params* prm, cudaStream_t st) {
   zoom_ctx ctx = g.ix->dict->ctx;
   if (g.ix->cap > 0) return ZOOM_OK;   // the capped walk has nothing to tune
   TuneMap& tm = *(TuneMap*)ctx->tuned;
-  const TuneKey key{g.ix, qbucket(g.nq), prm->precision, prm->K};
+  const TuneKey key = tune_key(g, prm);
   if (tm.count(key)) return ZOOM_OK;
   const int64_t ns = std::min<int64_t>(g.nq, 131072);
   std::vector<std::pair<int, int>> cands;
@@ -1477,7 +1481,7 @@ zoom_status zoom_upscale_batch(const zoom_index* ixs, int32_t n_indexes, int32_t
       bool pruned = false;
       for (auto& g : groups) {
         if (g.images.empty()) continue;
-        const TuneKey tk{g.ix, qbucket(g.nq), prm->precision, prm->K};
+        const TuneKey tk = tune_key(g, prm);
         const TuneChoice ch = tm.count(tk) ? tm[tk] : TuneChoice();
         g.plan = plan_search(g.ix, prm, g.nq, ch.nsplit, ch.mc, may_prune);
         pruned = pruned || g.plan.pruned;

@@ -94,3 +94,33 @@ def test_a_changed_parameter_is_not_a_replay(change):
     if "fp64_cond_threshold" in change:
         assert n_fp64 > 0
     Z.batch_release(ctx)
+
+
+@pytest.mark.parametrize("n_pairs, first, second", [(256, (20, 24), (21, 24)),            # dense both times
+                                                    (65536, (120, 160), (150, 160))],      # then over the search order
+                         ids=["dense", "search order"])
+def test_list_sizes_follow_the_calls_own_rerank_mult(n_pairs, first, second):
+    # A precision-form batch with rerank_mult 2 (16 chunks a query) tunes the
+    # searches of its query count; one with rerank_mult 4 (32 chunks) and as
+    # many queries, to a power of two, must not search 16.  The list size is
+    # seen in the search workspace, the batch's largest allocations (a
+    # dictionary of 256 entries is one step, so the tuned splits are 1).
+    import paper_1004_3980_gb300 as Z
+
+    def sizes(calls):
+        ctx, A = _context()
+        ix = _index(ctx, n_pairs, *((3, 96) if n_pairs < 5000 else (10, 256)))
+        torch.cuda.synchronize()
+        held = dict(A.live)
+        for shape, mult in calls:
+            lrs = _images(shape)
+            p = Z.UpscaleParams(K=8, bp_iters=1, precision=1, rerank_mult=mult)
+            outs, _ = Z.upscale_batch([ix], lrs, p)
+        torch.cuda.synchronize()
+        single = Z.upscale(ix, lrs[0][1], p)
+        assert torch.equal(outs[0], single)
+        got = sorted(n for a, n in A.live.items() if a not in held)
+        Z.batch_release(ctx)
+        return got
+
+    assert sizes([(first, 2), (second, 4)]) == sizes([(second, 4)])
