@@ -286,25 +286,11 @@ __global__ void k_sumsq_partials(const float* __restrict__ r, int64_t n, double*
   if (threadIdx.x == 0) part[blockIdx.x] = sh[0];
 }
 
-// (s, c) += (a - b)^2, a sum in two floats: the difference and its square are
-// exact in two floats but for terms below 2^-48 of the square, as is what the
-// sum leaves out of each addition.
-__device__ __forceinline__ void add_sqdiff(float a, float b, float& s, float& c) {
-  const float d = a - b, bb = d - a;
-  const float dl = (a - (d - bb)) - (b + bb);   // a - b = d + dl
-  const float p = d * d;
-  const float e = fmaf(2.f * d, dl, fmaf(d, d, -p));
-  const float t = s + p, v = t - s;
-  c += ((s - (t - v)) + (p - v)) + e;
-  s = t;
-}
-
 // per-block partial sums of the overlap prior: each (patch, pixel) adds the
-// squared difference to its right and down neighbours where they overlap.
-// Sixteen values at a time are summed in two floats, then join the thread's
-// FP64 sum: this GPU has few FP64 units, and they bounded it (63,504 patches
-// of 10 x 10: 116 us with FP64 throughout and a division each for patch and
-// pixel, 81 us so; the energy kept its bits there).
+// squared difference to its right and down neighbours where they overlap, in
+// FP64 throughout.  Bound by the GPU's few FP64 units (63,504 patches of 10 x
+// 10: 114 us; 81 us with sixteen values at a time in pairs of floats, which
+// loses bits and FP64's range).
 __global__ void k_prior_partials(const float* __restrict__ P, int h, int w, int s, int Pp, int ph2pad,
                                  double* __restrict__ part) {
   __shared__ double sh[256];
@@ -324,34 +310,33 @@ __global__ void k_prior_partials(const float* __restrict__ P, int h, int w, int 
   int i = (int)(n / nw), j = (int)(n - (int64_t)i * nw);
   const int di = (int)(dn / nw), dj = (int)(dn - (int64_t)di * nw);
   double acc = 0.0;
-  while (t < total) {
-    float sum = 0.f, low = 0.f;
 #pragma unroll 4
-    for (int u = 0; u < 16 && t < total; ++u, t += step) {
-      const uint32_t c = s_px[p];
-      const int a = c & 255, b = (c >> 8) & 255;
-      const float* pn = P + n * ph2pad;
-      const float pv = pn[p];
-      // no neighbour, no overlap: the value itself, a difference of 0
-      const float right = j + 1 < nw && b >= s ? pn[ph2pad + p - s] : pv;
-      const float down = i + 1 < nh && a >= s ? pn[(int64_t)nw * ph2pad + p - s * PH] : pv;
-      add_sqdiff(pv, right, sum, low);
-      add_sqdiff(pv, down, sum, low);
-      n += dn;
-      p += dp;
-      i += di;
-      j += dj;
-      if (p >= ph2) {
-        p -= ph2;
-        ++n;
-        ++j;
-      }
-      if (j >= nw) {
-        j -= nw;
-        ++i;
-      }
+  for (; t < total; t += step) {
+    const uint32_t c = s_px[p];
+    const int a = c & 255, b = (c >> 8) & 255;
+    const float* pn = P + n * ph2pad;
+    const double pv = (double)pn[p];
+    if (j + 1 < nw && b >= s) {
+      const double d = pv - (double)pn[ph2pad + p - s];
+      acc += d * d;
     }
-    acc += (double)sum + (double)low;
+    if (i + 1 < nh && a >= s) {
+      const double d = pv - (double)pn[(int64_t)nw * ph2pad + p - s * PH];
+      acc += d * d;
+    }
+    n += dn;
+    p += dp;
+    i += di;
+    j += dj;
+    if (p >= ph2) {
+      p -= ph2;
+      ++n;
+      ++j;
+    }
+    if (j >= nw) {
+      j -= nw;
+      ++i;
+    }
   }
   sh[threadIdx.x] = acc;
   __syncthreads();
