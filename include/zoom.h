@@ -117,14 +117,16 @@ typedef struct {
  * FP32 exact rerank of those chunks' entries.
  * fp64_cond_threshold: the LLE solve runs in FP64 for a query whose
  * condition bound (trace(G) + eps) / eps exceeds it.
- * search (precision 0 only): 0 = automatic (tensor cores from 4096
- * dictionary entries), 1 = SIMT scan of the dictionary in FP32 difference
- * form, 2 = tensor-core search with a proven exact FP32 rerank: a filter with
+ * search: 0 = automatic (tensor cores from 4096 dictionary entries, over the
+ * index's search order where it has one and the call is large enough), 1 =
+ * SIMT scan of the dictionary in FP32 difference form, 2 = tensor-core search
+ * of the whole dictionary with a proven exact FP32 rerank: a filter with
  * one FP16 term per feature value (K = 32), then, for the queries its error
  * bound cannot settle, the FP16 hi/lo-split filter (K = 80) on just those
  * queries, then the SIMT scan for any left; 3 = the split filter alone (then
  * the SIMT scan).  All four give the same neighbours bit for bit.  Precision 1
- * always uses the tensor cores; it needs rerank_mult * K <= 32. */
+ * knows 0 and, for 1 to 3 alike, the filter over the whole dictionary; it
+ * always uses the tensor cores and needs rerank_mult * K <= 32. */
 typedef struct {
   int32_t K;
   float reg_rel;

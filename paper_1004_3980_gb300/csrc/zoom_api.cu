@@ -611,8 +611,9 @@ SearchPlan plan_search(zoom_index ix, const zoom_upscale_params* prm, int64_t nq
   p.prec = prm->precision == 1 ? 1 : (prm->search == 3 ? 0 : 2);
   p.MC = mc_override > 0 ? mc_override : tc_list_size(p.prec, prm->K, prm->rerank_mult);
   p.KCH = tc_kc(d->d, p.prec) * 8;
-  // automatic search and the precision form: over the search order where the
-  // dictionary has one
+  // automatic search, in both forms: over the search order where the
+  // dictionary has one (search 1 to 3: the dense searches)
+  may_prune = may_prune && prm->search == 0;
   if (may_prune && p.prec == 1) {
     // the precision form's dense plan says what its lists are
     const SearchPlan dense = plan_search(ix, prm, nq, 0, 0, false);
@@ -638,7 +639,7 @@ SearchPlan plan_search(zoom_index ix, const zoom_upscale_params* prm, int64_t nq
       return p;
     }
   }
-  if (may_prune && prm->search == 0 && p.prec == 2 && prune_plan(ix, 2, prm->K, nq, &p.pp)) {
+  if (may_prune && p.prec == 2 && prune_plan(ix, 2, prm->K, nq, &p.pp)) {
     p.pruned = true;
     p.cap2 = std::min<int64_t>(nq, std::max<int64_t>(8192, nq / 64));
     p.MC2 = tc_list_size(0, prm->K, prm->rerank_mult);

@@ -131,3 +131,31 @@ def test_bf16_32_chunk_lists_past_the_packed_key_limit(big):
     assert int(nb.min()) >= 0 and int(nb.max()) < n
     ix.close()
     d.close()
+
+
+def test_bf16_form_over_the_search_order_equals_the_dense_filter_3x(big):
+    # every query; the dense filter's 32-chunk lists are packed keys here
+    a = big["Z"].query(big["ix"], big["lr_t"], G.params(big["wl"], precision=1, rerank_mult=4, search=2))
+    b = big["q_bf"]
+    assert torch.equal(a["nbr"], b["nbr"]) and torch.equal(a["dist"], b["dist"])
+
+
+def test_more_entries_than_full_rounds_of_queries_have_room_for(big):
+    # 4,300,001 entries: the tiles' query lists (2 GB) hold 63,744 queries a
+    # round, so 65,536 take two; the dense BF16 filter keeps its 32-chunk lists
+    # as (value, index) pairs
+    Z, wl = big["Z"], big["wl"]
+    n = 4_300_001
+    lrs = wl.train_hr // wl.scale
+    pos = S.sample_positions(wl.pos_seed + 2, len(big["train"]), lrs, lrs, wl.patch, n)
+    d = Z.Dictionary(big["ctx"], [torch.from_numpy(x).cuda() for x in big["train"]], pos, wl.scale, wl.patch,
+                     wl.blur_sigma)
+    ix = Z.Index(d, wl.L, wl.k, wl.w, big["alpha"], big["beta"])
+    lr_c = big["lr_t"][:260, :260].contiguous()
+    for kw in (dict(), dict(precision=1, rerank_mult=4)):
+        a = Z.query(ix, lr_c, G.params(wl, **kw))
+        b = Z.query(ix, lr_c, G.params(wl, search=2 if kw else 1, **kw))
+        big["ctx"].sync_status()
+        assert torch.equal(a["nbr"], b["nbr"]) and torch.equal(a["dist"], b["dist"]), kw
+    ix.close()
+    d.close()
