@@ -892,21 +892,55 @@ cudaError_t run_search_ws(zoom_index ix, const zoom_upscale_params* prm, const Q
   return e;
 }
 
+// The dense search of a call in two parts of its queries, one after the other
+// in the same scratch: for a caller whose memory does not hold all of it at
+// once.  Every query is searched in the lists it has in one part (the precision
+// form's result depends on them): the queries of whole rounds in one list, the
+// others in the plan's nsplit.
+struct HalvedSearch {
+  int64_t q0 = 0;   // first query of the second part
+  SearchPlan pl[2];
+  size_t bytes() const { return std::max(pl[0].bytes, pl[1].bytes); }
+};
+HalvedSearch halve_search(zoom_index ix, const zoom_upscale_params* prm, int64_t nq) {
+  const SearchPlan whole = plan_search(ix, prm, nq, 0, 0, false);
+  const int64_t round = (int64_t)ix->dict->ctx->n_sm * 256;
+  const int64_t rounds = (nq + 255) / 256 * 256 / round * round;   // queries of whole rounds
+  const bool cut = whole.tail_split > 1 && rounds < nq;
+  HalvedSearch h;
+  h.q0 = cut ? rounds : (nq / 2 + 255) / 256 * 256;
+  if (h.q0 <= 0 || h.q0 >= nq) h.q0 = 0;
+  else {
+    h.pl[0] = plan_search(ix, prm, h.q0, cut ? 1 : whole.nsplit, 0, false);
+    h.pl[1] = plan_search(ix, prm, nq - h.q0, whole.nsplit, 0, false);
+  }
+  return h;
+}
+
 cudaError_t run_search(zoom_index ix, const zoom_upscale_params* prm, const QueryBufs& b, int64_t nq,
                        cudaStream_t st, bool& oom) {
   SearchPlan pl = plan_search(ix, prm, nq, 0, 0);
   if (!pl.tc && !pl.capped) return run_search_ws(ix, prm, b, nq, pl, nullptr, st);
   Scratch scr(ix->dict->ctx, st);
-  bool got = scr.get(pl.bytes);
-  if (!got && pl.pruned) {   // no room for the query lists: the dense search
+  if (scr.get(pl.bytes)) return run_search_ws(ix, prm, b, nq, pl, scr.p, st);
+  if (pl.pruned) {   // no room for the query lists: the dense search
     pl = plan_search(ix, prm, nq, 0, 0, false);
-    got = scr.get(pl.bytes);
+    if (scr.get(pl.bytes)) return run_search_ws(ix, prm, b, nq, pl, scr.p, st);
   }
-  if (!got) {
-    oom = true;
-    return cudaSuccess;
+  if (pl.tc) {
+    const HalvedSearch h = halve_search(ix, prm, nq);
+    if (h.q0 > 0 && h.bytes() < pl.bytes && scr.get(h.bytes())) {
+      QueryBufs b2 = b;   // the second part's (what the search reads and writes)
+      b2.feat += h.q0 * ix->dict->dpad;
+      b2.keys += h.q0 * ix->L;
+      b2.nbr += h.q0 * prm->K;
+      b2.dist += h.q0 * prm->K;
+      const cudaError_t e = run_search_ws(ix, prm, b, h.q0, h.pl[0], scr.p, st);
+      return e != cudaSuccess ? e : run_search_ws(ix, prm, b2, nq - h.q0, h.pl[1], scr.p, st);
+    }
   }
-  return run_search_ws(ix, prm, b, nq, pl, scr.p, st);
+  oom = true;
+  return cudaSuccess;
 }
 
 zoom_status run_query_steps(zoom_index ix, const float* lr, int h, int w,

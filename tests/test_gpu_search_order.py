@@ -28,3 +28,21 @@ def test_search_2_takes_the_dense_filter_in_both_forms(prec):
         size.append(max(ctx.test_allocator.sizes))
     assert size[1] < size[0] / 2
     assert _equal(*got)
+
+
+@pytest.mark.parametrize("h,w", [(60, 71), (230, 201)])   # fewer than 152 x 256 queries, and a round and a part
+@pytest.mark.parametrize("prm", [dict(search=2), dict(search=3), dict(precision=1, search=2)], ids=str)
+def test_a_refused_dense_search_runs_in_two_parts(h, w, prm):
+    import paper_1004_3980_gb300 as Z
+    ctx, ix = _build(30001)
+    A = ctx.test_allocator
+    lr = torch.from_numpy(S.make_image(3, h, w)).cuda()
+    A.sizes = []
+    ref = Z.query(ix, lr, Z.UpscaleParams(K=8, **prm))
+    A.limit, A.refused = max(A.sizes) - 1, 0
+    got = Z.query(ix, lr, Z.UpscaleParams(K=8, **prm))
+    torch.cuda.synchronize()
+    assert A.refused == 1 and _equal(got, ref)
+    A.limit = 1000   # no room at all
+    with pytest.raises(Exception, match="OOM"):
+        Z.query(ix, lr, Z.UpscaleParams(K=8, **prm))
