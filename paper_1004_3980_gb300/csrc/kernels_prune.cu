@@ -549,7 +549,7 @@ __global__ void k_steps(const uint32_t* __restrict__ tcnt, int nt, const uint32_
 // The operand rows of the queries carry -thr (three terms against ones of the
 // dictionary's rows), so an accumulator is negative exactly where the entry
 // may lie within the query's radius.
-//   warps 18..23  gather the queries' operand rows (64 or 128 bytes each)
+//   warps 18..23  gather the queries' operand rows (64 bytes each)
 //                 through registers into a ring of stages, a step each in turn
 //   warps 0, 1    issue the MMAs of the even / odd steps, M = 128 queries x
 //                 N = 256 entries, into an accumulator each (the two fill the
@@ -576,19 +576,19 @@ constexpr int kGather = 6;   // gathering warps
 // polls of an accumulator's barrier before the suspending wait (1 to 32 the
 // same; 256 made a step 5 % longer: the polling warps slow the others)
 constexpr int kAccPolls = 8;
-__host__ __device__ constexpr int tg_stages(int KC) { return KC <= 4 ? 6 : 3; }   // a multiple of kGather / 2
+constexpr int kStagesTg = 6;   // a multiple of kGather / 2
 // at least 3: a tile's slot is free once both parities are past it, and the
 // parity that waits for a tile may be two tiles ahead of the other
-__host__ __device__ constexpr int tg_slots(int KC) { return KC <= 4 ? 4 : 3; }
+constexpr int kSlotsTg = 4;
 constexpr int kTgThreads = (2 + kEpi + kGather) * 32;
 constexpr int kTgBar = 512;
 __host__ __device__ constexpr int tg_smem(int KC) {
-  return 1024 + 2 * tg_stages(KC) * KC * PQ_ROWS * 16 + tg_slots(KC) * KC * PT_ROWS * 16 + kTgBar +
-         2 * tg_stages(KC) * PQ_ROWS * 2 + 2 * kHits * kEpi * 32 * 8;
+  return 1024 + 2 * kStagesTg * KC * PQ_ROWS * 16 + kSlotsTg * KC * PT_ROWS * 16 + kTgBar +
+         2 * kStagesTg * PQ_ROWS * 2 + 2 * kHits * kEpi * 32 * 8;
 }
-static_assert(tg_smem(4) <= 232448 && tg_smem(8) <= 232448, "shared memory of the list filter");
-static_assert(tg_slots(4) >= 3 && tg_slots(8) >= 3, "tile slots");
-static_assert(tg_stages(4) % (kGather / 2) == 0 && tg_stages(8) % (kGather / 2) == 0, "a stage belongs to one gathering warp");
+static_assert(tg_smem(4) <= 232448, "shared memory of the list filter");
+static_assert(kSlotsTg >= 3, "tile slots");
+static_assert(kStagesTg % (kGather / 2) == 0, "a stage belongs to one gathering warp");
 
 // The steps of one CTA, numbered 0 .. count - 1: pieces of `len` consecutive
 // steps dealt out to the CTAs in turn, so that tiles many entries of which
@@ -652,7 +652,7 @@ template <int KC, uint32_t AB_TYPE>
 __global__ void __maxnreg__(80) k_knn_tg(TgArgs a) {
   constexpr uint32_t kATile = KC * PQ_ROWS * 16;
   constexpr uint32_t kBTile = KC * PT_ROWS * 16;
-  constexpr uint32_t kA = tg_stages(KC), kSlots = tg_slots(KC);
+  constexpr uint32_t kA = kStagesTg, kSlots = kSlotsTg;
   constexpr uint32_t kIdesc = tg_idesc(AB_TYPE);
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -1303,7 +1303,7 @@ cudaError_t run_pruned(zoom_index ix, const PrunePlan& p, const float* qfeat, co
   if (e != cudaSuccess) return e;
 #define ZOOM_PR_SORT(DD)                                                                                          \
   do {                                                                                                            \
-    constexpr int kKc = DD + 3 <= 32 ? 4 : 8;                                                                     \
+    constexpr int kKc = 4;                                                                                        \
     k_query_route<DD><<<qb, 128, 0, st>>>(qfeat, d->dpad, nq, ix->tree_basis, n1, n2, d1, d2, b.leaf, b.rank, b.hist); \
     k_leaf_scan<<<1, 1024, 0, st>>>(b.hist, leaves);                                                              \
     if (p.form == 1)                                                                                              \
@@ -1317,7 +1317,6 @@ cudaError_t run_pruned(zoom_index ix, const PrunePlan& p, const float* qfeat, co
     case 9: ZOOM_PR_SORT(9); break;
     case 25: ZOOM_PR_SORT(25); break;
     case 18: ZOOM_PR_SORT(18); break;
-    case 50: ZOOM_PR_SORT(50); break;
     default: return cudaErrorInvalidValue;
   }
 #undef ZOOM_PR_SORT
@@ -1371,8 +1370,7 @@ cudaError_t run_pruned(zoom_index ix, const PrunePlan& p, const float* qfeat, co
     a.status = ctx->d_status;
     a.wait_ns = ctx->wait_ns > 0 ? ctx->wait_ns : kWaitNs;
     a.inject = ctx->inject;
-    if (p.form == 1) e = p.kc == 4 ? run_tg<4, 1>(a, ctx->n_sm, st) : run_tg<8, 1>(a, ctx->n_sm, st);
-    else e = p.kc == 4 ? run_tg<4, 0>(a, ctx->n_sm, st) : run_tg<8, 0>(a, ctx->n_sm, st);
+    e = p.form == 1 ? run_tg<4, 1>(a, ctx->n_sm, st) : run_tg<4, 0>(a, ctx->n_sm, st);
     if (e != cudaSuccess) return e;
 #define ZOOM_PR_LIST(DD, FF)                                                                                      \
   k_rerank_list<DD, FF><<<(m + 3) / 4, 128, 0, st>>>(                                                           \
@@ -1382,11 +1380,9 @@ cudaError_t run_pruned(zoom_index ix, const PrunePlan& p, const float* qfeat, co
       case 9: ZOOM_PR_LIST(9, 2); break;
       case 25: ZOOM_PR_LIST(25, 2); break;
       case 18: ZOOM_PR_LIST(18, 2); break;
-      case 50: ZOOM_PR_LIST(50, 2); break;
       case 109: ZOOM_PR_LIST(9, 1); break;
       case 125: ZOOM_PR_LIST(25, 1); break;
-      case 118: ZOOM_PR_LIST(18, 1); break;
-      default: ZOOM_PR_LIST(50, 1); break;
+      default: ZOOM_PR_LIST(18, 1); break;
     }
 #undef ZOOM_PR_LIST
     e = cudaGetLastError();

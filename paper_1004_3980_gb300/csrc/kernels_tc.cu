@@ -1698,9 +1698,7 @@ cudaError_t launch_knn_seeds(const uint16_t* qop, const float* qn, int64_t nq, c
   return MC == 16 ? run_tw_kernel<KC, 16, T, false>(a, grid, st) : run_tw_kernel<KC, 32, T, false>(a, grid, st)
   if (MC != 16 && MC != 32) return cudaErrorInvalidValue;
   if (precision == 2 && kc == 4) ZOOM_TW(4, 0);
-  if (precision == 2 && kc == 8) ZOOM_TW(8, 0);
   if (precision == 1 && kc == 4) ZOOM_TW(4, 1);
-  if (precision == 1 && kc == 8) ZOOM_TW(8, 1);
 #undef ZOOM_TW
   return cudaErrorInvalidValue;
 }

@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(kTreeThreads) k_tree_top(const float* __restri
     load_feature<D>(feat + e * dpad, f[h]);
   }
   __syncthreads();
-  constexpr int kBlocks = (D == 18 || D == 50) ? 2 : 1;   // [g_x | g_y]
+  constexpr int kBlocks = D == 18 ? 2 : 1;   // [g_x | g_y]
   constexpr int kP2 = D / kBlocks;
 #pragma unroll
   for (int blk = 0; blk < kBlocks; ++blk) {
@@ -470,7 +470,7 @@ cudaError_t build_search_tree(zoom_index ix, void* scratch, size_t scratch_bytes
   k_tree_route<DD><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(d->feat, d->dpad, n, ix->tree_basis, node1, node2, \
                                                                 d1, d2, leaf)
 #define ZOOM_TREE_C(DD)                                                                                       \
-  k_tile_operands<DD, (DD + 3 <= 32 ? 4 : 8)><<<nt, PT_ROWS, 0, st>>>(d->feat, d->dpad, n, ix->tree_order,        \
+  k_tile_operands<DD, 4><<<nt, PT_ROWS, 0, st>>>(d->feat, d->dpad, n, ix->tree_order,        \
                                                                       ix->tree_basis, ix->tree_f1, ix->tree_bf, \
                                                                       (uint4*)ix->tree_box, ix->tree_mid, stat)
 #define ZOOM_TREE(X)                   \
@@ -478,7 +478,6 @@ cudaError_t build_search_tree(zoom_index ix, void* scratch, size_t scratch_bytes
     case 9: X(9); break;               \
     case 25: X(25); break;             \
     case 18: X(18); break;             \
-    case 50: X(50); break;             \
     default: return cudaErrorInvalidValue; \
   }
   ZOOM_TREE(ZOOM_TREE_A)

@@ -416,8 +416,9 @@ zoom_status zoom_build_index(zoom_dict d, const zoom_lsh_params* lsh, const floa
   ix->proj_dist = drawn_a.empty() ? 0 : lsh->proj_dist;
   ix->seed = drawn_a.empty() ? 0 : lsh->seed;
   ix->nd_rows = tc_rows_padded(N, true);   // whole 256-row steps for the wide-step filter
-  // the search order (a capped index walks its bins and never searches densely)
-  if (ix->cap == 0 && N >= kPruneMinEntries && N <= kPruneMaxEntries) {
+  // the search order (a capped index walks its bins and never searches
+  // densely; features of 50 values are searched densely)
+  if (ix->cap == 0 && tc_kc(d->d, 2) == 4 && N >= kPruneMinEntries && N <= kPruneMaxEntries) {
     ix->tree_tiles = (N + 255) / 256;
     tree_depths(N, &ix->tree_d1, &ix->tree_d2);
   }

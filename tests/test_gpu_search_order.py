@@ -46,3 +46,17 @@ def test_a_refused_dense_search_runs_in_two_parts(h, w, prm):
     A.limit = 1000   # no room at all
     with pytest.raises(Exception, match="OOM"):
         Z.query(ix, lr, Z.UpscaleParams(K=8, **prm))
+
+
+@pytest.mark.parametrize("feature", [1, 2])
+def test_features_of_50_values_are_searched_densely(feature):
+    import paper_1004_3980_gb300 as Z
+    ctx, ix = _build(70001, feature=feature, w=8.0)
+    lr = torch.from_numpy(S.make_image(1, 151, 163)).cuda()
+    got, sizes = [], []
+    for search in (0, 2):
+        ctx.test_allocator.sizes = []
+        got.append(Z.query(ix, lr, Z.UpscaleParams(K=8, search=search)))
+        sizes.append(ctx.test_allocator.sizes)
+    assert sizes[0] == sizes[1]
+    assert _equal(*got)
