@@ -693,6 +693,7 @@ __global__ void __maxnreg__(80) k_knn_tg(TgArgs a) {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  __syncwarp();   // the allocation is warp-collective: lane 0 comes from the initialisation
   if (warp == 0) {
     tmem_alloc(tmem_slot, 512);
     tmem_relinquish();
