@@ -199,8 +199,9 @@ struct WorkIter {
   }
 };
 
-// Where list `seg` of query q goes.
-__device__ __forceinline__ int64_t list_row(const TcArgs& a, int seg, int64_t q, float*& d, int32_t*& id) {
+// Where list `seg` of query q goes, and what is added to its values: ||q||^2,
+// or nothing in a piece's list (k_merge_parts adds it to what it keeps).
+__device__ __forceinline__ int64_t list_row(const TcArgs& a, int seg, int64_t q, float*& d, int32_t*& id, float& qn) {
   d = a.out_d;
   id = a.out_id;
   if (a.part_d) {
@@ -208,6 +209,7 @@ __device__ __forceinline__ int64_t list_row(const TcArgs& a, int seg, int64_t q,
     if (fan_out(pairs, a.nsplit, gridDim.x) > 1) {
       d = a.part_d;
       id = a.part_id;
+      qn = 0.f;
       return (int64_t)seg * pairs * (2 * TC_ROWS) + q;
     }
   }
@@ -528,13 +530,14 @@ __global__ void __maxnreg__(tc_max_regs(KC, MC)) k_knn_tc(TcArgs a) {
       if (valid) {
         float* od;
         int32_t* oi;
-        const int64_t lrow = list_row(a, split, q, od, oi);
+        float add = qn;
+        const int64_t lrow = list_row(a, split, q, od, oi, add);
         od += lrow * MC;
         oi += lrow * MC;
 #pragma unroll
         for (int j = 0; j < MC; ++j) {
           const bool real = li[j] >= 0 && (int64_t)li[j] * 32 < a.nd;
-          od[j] = real ? qn + ld[j] : FLT_MAX;
+          od[j] = real ? add + ld[j] : FLT_MAX;
           oi[j] = real ? li[j] : -1;
         }
         if (a.tail_split > 0 && t0 == 0 && t1 == a.nd_tiles) {
@@ -961,8 +964,9 @@ __global__ void __launch_bounds__(352, 1) k_knn_tw(TcArgs a) {
       if (valid) {
         float* od;
         int32_t* oi;
-        const int64_t lrow = list_row(a, split, q, od, oi);
-        L.write(qn, a.nd, od + lrow * MC, oi + lrow * MC);
+        float add = qn;
+        const int64_t lrow = list_row(a, split, q, od, oi, add);
+        L.write(add, a.nd, od + lrow * MC, oi + lrow * MC);
         if (a.tail_split > 0 && t0 == 0 && t1 == a.nd_tiles) {
           for (int s2 = 1; s2 < a.tail_split; ++s2) {
             float* od1 = a.out_d + ((int64_t)s2 * a.nq + q) * MC;
@@ -987,12 +991,14 @@ __global__ void __launch_bounds__(352, 1) k_knn_tw(TcArgs a) {
 }
 
 // The pieces' lists of a search with fan_out() > 1 joined: a warp per query
-// and list keeps the MC smallest (d~, chunk) of its pieces' lists, which is
-// the list one piece would have written (equal d~ keep the lower chunk there
-// too).
+// and list keeps the MC smallest (value, chunk) of its pieces' lists, which is
+// the list one piece would have written: the values are those it orders by
+// (d~ - ||q||^2, or the packed keys' d~; qn then nullptr), and equal ones keep
+// the lower chunk there too.  d~ itself, rounded, would make some of them equal.
 template <int MC>
 __global__ void __launch_bounds__(128) k_merge_parts(const unsigned long long* __restrict__ nq_dev, int64_t nq,
-                                                     int nsplit, int grid, const float* __restrict__ part_d,
+                                                     int nsplit, int grid, const float* __restrict__ qn,
+                                                     const float* __restrict__ part_d,
                                                      const int32_t* __restrict__ part_id, float* __restrict__ out_d,
                                                      int32_t* __restrict__ out_id) {
   const int64_t n = (int64_t)*nq_dev < nq ? (int64_t)*nq_dev : nq;
@@ -1014,7 +1020,7 @@ __global__ void __launch_bounds__(128) k_merge_parts(const unsigned long long* _
   }
   if (lane < MC) {
     const int64_t o = ((int64_t)s * nq + q) * MC + lane;
-    out_d[o] = bd;
+    out_d[o] = bi != INT_MAX && qn ? qn[q] + bd : bd;
     out_id[o] = bi == INT_MAX ? -1 : bi;
   }
 }
@@ -1558,6 +1564,22 @@ static cudaError_t knn_tc(const uint16_t* qop, const float* qn, int64_t nq, cons
                           int32_t* out_id, unsigned int* status, cudaStream_t st, const unsigned long long* nq_dev,
                           uint64_t wait_ns, int inject, const TcParts& parts);
 
+// Bits of a chunk number of nd entries.
+static int chunk_bits(int64_t nd) {
+  int b = 3;
+  while ((int64_t{1} << b) < (nd + TW_ROWS - 1) / TW_ROWS * 8) ++b;
+  return b;
+}
+
+// The BF16 form's 32-chunk lists are packed while the chunk numbers leave
+// the keys at least 15 value bits (up to 2^17 chunks, 4,194,304 entries):
+// there the merges dominate the list time (measured: 8 % off the filter
+// with 1M entries, 2 % with 4M); 16-chunk lists merge rarely and run
+// slightly faster unpacked.
+static bool packed_lists(int precision, int kc, int MC, int64_t nd) {
+  return precision == 1 && tc_wide_form(precision, kc) && MC == 32 && chunk_bits(nd) <= 17;
+}
+
 int64_t tc_part_floats(int grid, int MC) { return (int64_t)2 * grid * 2 * TC_ROWS * MC; }
 
 cudaError_t launch_knn_tc(const uint16_t* qop, const float* qn, int64_t nq, const uint16_t* dop,
@@ -1577,10 +1599,12 @@ cudaError_t launch_knn_tc(const uint16_t* qop, const float* qn, int64_t nq, cons
     const int g = (int)(grid < nsplit * pairs ? grid : nsplit * pairs);
     // fan_out() > 1 needs pairs * nsplit <= g: at most that many lists to join
     const int64_t lists = std::min<int64_t>((int64_t)g * 2 * TC_ROWS, nq * nsplit);
+    const unsigned blocks = (unsigned)((lists + 3) / 4);
+    const float* add = packed_lists(precision, kc, MC, nd) ? nullptr : qn;
     if (MC == 16)
-      k_merge_parts<16><<<(unsigned)((lists + 3) / 4), 128, 0, st>>>(nq_dev, nq, nsplit, g, part_d, part_id, out_d, out_id);
+      k_merge_parts<16><<<blocks, 128, 0, st>>>(nq_dev, nq, nsplit, g, add, part_d, part_id, out_d, out_id);
     else
-      k_merge_parts<32><<<(unsigned)((lists + 3) / 4), 128, 0, st>>>(nq_dev, nq, nsplit, g, part_d, part_id, out_d, out_id);
+      k_merge_parts<32><<<blocks, 128, 0, st>>>(nq_dev, nq, nsplit, g, add, part_d, part_id, out_d, out_id);
     return cudaGetLastError();
   }
   return knn_tc(qop, qn, nq, dop, nd, precision, kc, MC, nsplit, tail_split, grid, out_d, out_id, status, st, nq_dev,
@@ -1617,14 +1641,8 @@ static cudaError_t knn_tc(const uint16_t* qop, const float* qn, int64_t nq, cons
     const int items = tail_split > 0 ? a.nq_pairs : a.nsplit * a.nq_pairs;
     grid = grid < items ? grid : items;
     a.full_rounds = tail_split > 0 ? a.nq_pairs / grid : 0;
-    // The BF16 form's 32-chunk lists are packed while the chunk numbers leave
-    // the keys at least 15 value bits (up to 2^17 chunks, 4,194,304 entries):
-    // there the merges dominate the list time (measured: 8 % off the filter
-    // with 1M entries, 2 % with 4M); 16-chunk lists merge rarely and run
-    // slightly faster unpacked.
-    a.id_bits = 3;
-    while ((int64_t{1} << a.id_bits) < (int64_t)a.nd_tiles * 8) ++a.id_bits;
-    const bool packed = precision == 1 && MC == 32 && a.id_bits <= 17;
+    a.id_bits = chunk_bits(nd);
+    const bool packed = packed_lists(precision, kc, MC, nd);
 #define ZOOM_TW(KC, T) \
   return MC == 16 ? run_tw_kernel<KC, 16, T, false>(a, grid, st) : run_tw_kernel<KC, 32, T, false>(a, grid, st)
     if (precision == 1 && kc == 4 && packed) return run_tw_kernel<4, 32, 1, true>(a, grid, st);

@@ -60,3 +60,52 @@ def test_features_of_50_values_are_searched_densely(feature):
         sizes.append(ctx.test_allocator.sizes)
     assert sizes[0] == sizes[1]
     assert _equal(*got)
+
+
+def _ramps(n, h, w, g):
+    """n horizontal ramps of slope g (LR values, h x w) -> HR images of scale 2."""
+    x = np.arange(2 * w, dtype=np.float64) / 2 * g
+    return [np.ascontiguousarray(np.broadcast_to(x + 0.01 * i, (2 * h, 2 * w))).astype(np.float32) for i in range(n)]
+
+
+def test_pieces_of_a_list_keep_the_chunks_one_piece_would():
+    # A few queries (vertical ramps) are left to the dense filter, their lists
+    # made in pieces.  Their nearest entries are thousands of patches of
+    # horizontal ramps, equal but for the rounding of their features: hundreds
+    # of chunks whose filter values d~ - ||q||^2 = ||c||^2 differ in the last
+    # bits, and of which some are equal once ||q||^2 is added (the sum lies in
+    # the next binade: 0.014 and 0.018 to 0.022 around 1/64).  All other
+    # entries are farther (norms above 0.06).
+    import paper_1004_3980_gb300 as Z
+    from oracle import zoom_oracle as O
+    P, n_ramp = 5, 4
+    train = _ramps(n_ramp, 64, 64, (0.014 / 50) ** 0.5) + [3 * S.make_image(300 + i, 512, 512) for i in range(4)]
+    pos, ramp = [], 0
+    for m, im in enumerate(train):
+        lr = O.degrade(im, 2, 0.8)
+        f = np.lib.stride_tricks.sliding_window_view(np.asarray(lr), (P, P)).reshape(lr.shape[0] - P + 1, -1, P * P)
+        n2 = ((f - f.mean(-1, keepdims=True)) ** 2).sum(-1)
+        i, j = np.nonzero(n2 > 0.06) if m >= n_ramp else np.nonzero(n2 > 0)
+        if m < n_ramp:   # away from the clamped edges
+            keep = (j > 2) & (j < 56)
+            i, j = i[keep], j[keep]
+            ramp += len(i)
+        pos.append(np.stack([np.full(len(i), m), i, j], 1))
+    pos = np.concatenate(pos).astype(np.int32)
+    assert len(pos) >= 70000
+    ctx = Z.Context(0)
+    d = Z.Dictionary(ctx, [torch.from_numpy(x).cuda() for x in train], pos, 2, P)
+    a, b = S.lsh_draws(6, 8, 12, P * P, 4.0)
+    ix = Z.Index(d, 8, 12, 4.0, a, b)
+    img = 3 * S.make_image(1, 200, 200)
+    for k in range(100):   # 100 patches, slopes of ||q||^2 from 0.004 to 0.008
+        g = ((0.004 + 0.00004 * k) / 50) ** 0.5
+        r, c = 20 * (k // 10) + 3, 20 * (k % 10) + 3
+        img[r:r + P, c:c + P] = (0.5 + g * (np.arange(P) - 2))[:, None]
+    lr = torch.from_numpy(np.ascontiguousarray(img)).cuda()
+    got = Z.query(ix, lr, Z.UpscaleParams(K=8, precision=1, rerank_mult=2))
+    left = ctx.stats()["n_filter_fallback"]
+    ref = Z.query(ix, lr, Z.UpscaleParams(K=8, precision=1, rerank_mult=2, search=2))
+    rows = [(20 * (k // 10) + 3) * 196 + 20 * (k % 10) + 3 for k in range(100)]
+    assert int(got["nbr"][rows].max()) < ramp and left >= 100, left
+    assert _equal(got, ref)
