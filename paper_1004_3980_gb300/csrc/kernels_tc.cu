@@ -990,38 +990,77 @@ __global__ void __launch_bounds__(352, 1) k_knn_tw(TcArgs a) {
   }
 }
 
-// The pieces' lists of a search with fan_out() > 1 joined: a warp per query
-// and list keeps the MC smallest (value, chunk) of its pieces' lists, which is
-// the list one piece would have written: the values are those it orders by
-// (d~ - ||q||^2, or the packed keys' d~; qn then nullptr), and equal ones keep
-// the lower chunk there too.  d~ itself, rounded, would make some of them equal.
+// The pieces' lists of a search with fan_out() > 1 joined: of a query's and
+// list's pieces the MC smallest (value, chunk) are kept, which is the list one
+// piece would have written: the values are those it orders by (d~ - ||q||^2,
+// or the packed keys' d~; qn then nullptr), and equal ones keep the lower chunk
+// there too.  d~ itself, rounded, would make some of them equal.
+// Bound by the latency of the pieces' reads: a warp issues eight at a time and
+// merges those whose smallest value can enter, and with more than eight pieces
+// a list (few queries left) four warps share them (134 queries, 128 pieces: 136
+// us with one warp and one read in flight a list, 13 us so).  Blocks loop over
+// the lists: the count is on the device.
 template <int MC>
 __global__ void __launch_bounds__(128) k_merge_parts(const unsigned long long* __restrict__ nq_dev, int64_t nq,
                                                      int nsplit, int grid, const float* __restrict__ qn,
                                                      const float* __restrict__ part_d,
                                                      const int32_t* __restrict__ part_id, float* __restrict__ out_d,
                                                      int32_t* __restrict__ out_id) {
+  __shared__ float s_d[4][MC];
+  __shared__ int s_i[4][MC];
   const int64_t n = (int64_t)*nq_dev < nq ? (int64_t)*nq_dev : nq;
   const int pairs = (int)((n + 2 * TC_ROWS - 1) / (2 * TC_ROWS));
   const int m = fan_out(pairs, nsplit, grid);
   if (m == 1) return;
-  const int lane = threadIdx.x & 31;
-  const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t q = w / nsplit;
-  const int s = (int)(w % nsplit);
-  if (q >= n) return;   // warp-uniform
-  float bd = FLT_MAX;
-  int bi = INT_MAX;
-  for (int j = 0; j < m; ++j) {
-    const int64_t o = (((int64_t)s * m + j) * pairs * (2 * TC_ROWS) + q) * MC + lane;
-    const float v = lane < MC ? part_d[o] : FLT_MAX;
-    const int id = v < FLT_MAX ? part_id[o] : INT_MAX;
-    warp_merge_best(bd, bi, v, id, MC, lane);
-  }
-  if (lane < MC) {
-    const int64_t o = ((int64_t)s * nq + q) * MC + lane;
-    out_d[o] = bi != INT_MAX && qn ? qn[q] + bd : bd;
-    out_id[o] = bi == INT_MAX ? -1 : bi;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool shared = m > 8;   // four warps a list
+  const int64_t step = (int64_t)gridDim.x * (shared ? 1 : 4);
+  for (int64_t l = shared ? blockIdx.x : (int64_t)blockIdx.x * 4 + warp; l < n * nsplit; l += step) {
+    const int64_t q = l / nsplit;
+    const int s = (int)(l % nsplit);
+    float bd = FLT_MAX;
+    int bi = INT_MAX;
+    const int first = shared ? warp : 0, stride = shared ? 4 : 1;
+    for (int j0 = first; j0 < m; j0 += 8 * stride) {
+      float v[8];
+      int id[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int j = j0 + u * stride;
+        const int64_t o = (((int64_t)s * m + j) * pairs * (2 * TC_ROWS) + q) * MC + lane;
+        const bool has = j < m && lane < MC;
+        v[u] = has ? part_d[o] : FLT_MAX;
+        id[u] = has ? part_id[o] : INT_MAX;
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        if (!(v[u] < FLT_MAX)) {
+          v[u] = FLT_MAX;
+          id[u] = INT_MAX;
+        }
+        const float last = __shfl_sync(kFull, bd, MC - 1);
+        const int last_id = __shfl_sync(kFull, bi, MC - 1);
+        // (ascending lists: the piece's first entry is its smallest)
+        if (__any_sync(kFull, lane == 0 && lex_less(v[u], id[u], last, last_id)))
+          warp_merge_best(bd, bi, v[u], id[u], MC, lane);
+      }
+    }
+    if (shared) {
+      if (lane < MC) {
+        s_d[warp][lane] = bd;
+        s_i[warp][lane] = bi;
+      }
+      __syncthreads();
+      if (warp == 0)
+        for (int w = 1; w < 4; ++w)
+          warp_merge_best(bd, bi, lane < MC ? s_d[w][lane] : FLT_MAX, lane < MC ? s_i[w][lane] : INT_MAX, MC, lane);
+      __syncthreads();   // the lists have been read
+    }
+    if (lane < MC && (!shared || warp == 0)) {
+      const int64_t o = ((int64_t)s * nq + q) * MC + lane;
+      out_d[o] = bi != INT_MAX && qn ? qn[q] + bd : bd;
+      out_id[o] = bi == INT_MAX ? -1 : bi;
+    }
   }
 }
 
@@ -1599,7 +1638,7 @@ cudaError_t launch_knn_tc(const uint16_t* qop, const float* qn, int64_t nq, cons
     const int g = (int)(grid < nsplit * pairs ? grid : nsplit * pairs);
     // fan_out() > 1 needs pairs * nsplit <= g: at most that many lists to join
     const int64_t lists = std::min<int64_t>((int64_t)g * 2 * TC_ROWS, nq * nsplit);
-    const unsigned blocks = (unsigned)((lists + 3) / 4);
+    const unsigned blocks = (unsigned)std::min<int64_t>((lists + 3) / 4, 8 * (int64_t)grid);
     const float* add = packed_lists(precision, kc, MC, nd) ? nullptr : qn;
     if (MC == 16)
       k_merge_parts<16><<<blocks, 128, 0, st>>>(nq_dev, nq, nsplit, g, add, part_d, part_id, out_d, out_id);
