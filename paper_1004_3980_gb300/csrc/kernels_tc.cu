@@ -1468,7 +1468,9 @@ __global__ __launch_bounds__(rerank_warps(D) * 32, D > 32 ? 8 : 7) void k_rerank
     buf ^= 1;
   }
   cp_async_wait<0>();   // no copy may still target this warp's buffers
-  const bool flagged = members < K || (exact && !(T - delta > dK));
+  // (a K-th distance that is not finite leaves empty places among the K best:
+  // features whose squares overflow FP32)
+  const bool flagged = members < K || !(dK < FLT_MAX) || (exact && !(T - delta > dK));
   if (flagged) {
     if (lane == 0) {
       const unsigned long long slot = atomicAdd(fb_count, 1ull);
