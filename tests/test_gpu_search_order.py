@@ -109,3 +109,75 @@ def test_pieces_of_a_list_keep_the_chunks_one_piece_would():
     rows = [(20 * (k // 10) + 3) * 196 + 20 * (k % 10) + 3 for k in range(100)]
     assert int(got["nbr"][rows].max()) < ramp and left >= 100, left
     assert _equal(got, ref)
+
+
+def _index_on(ctx, n_pairs, n_train=10, L=8, k=12, **kw):
+    import paper_1004_3980_gb300 as Z
+    train = [S.make_image(300 + i, 256, 256) for i in range(n_train)]
+    pos = S.sample_positions(5, n_train, 128, 128, 5, n_pairs)
+    a, b = S.lsh_draws(6, L, k, 25, 4.0)
+    dic = Z.Dictionary(ctx, [torch.from_numpy(x).cuda() for x in train], pos, 2, 5)
+    return Z.Index(dic, L, k, 4.0, a, b, **kw)
+
+
+@pytest.mark.parametrize("memory", ["ordinary", "random bytes"])
+@pytest.mark.parametrize("prec", [0, 1])
+def test_waits_that_run_out_in_the_list_filter(prec, memory):
+    # Every filter of the call withholds its accumulators' releases, so its
+    # waits run out after 20 ms: reported, nothing followed outside the
+    # dictionary (with random bytes in place of what was never written), and
+    # the next call is the ordinary one's again.
+    import paper_1004_3980_gb300 as Z
+    from paper_1004_3980_gb300.capi import ZoomError
+    from tests.test_gpu_faults import GarbageAllocator
+    n = 65536
+    ctx = Z.Context(0, allocator=GarbageAllocator()) if memory == "random bytes" else Z.Context(0)
+    ix = _index_on(ctx, n)
+    lr = torch.from_numpy(S.make_image(1, 150, 152)).cuda()
+    p = Z.UpscaleParams(K=8, precision=prec)
+    ref = Z.query(ix, lr, Z.UpscaleParams(K=8, precision=prec, search=2))
+    ctx.sync_status()
+    ctx.set_fault_injection(1, 20_000_000)
+    try:
+        r = Z.query(ix, lr, p)
+        with pytest.raises(ZoomError, match="TIMEOUT"):
+            ctx.sync_status()
+    finally:
+        ctx.set_fault_injection(0, 0)
+    ctx.sync_status()
+    assert int(r["nbr"].min()) >= 0 and int(r["nbr"].max()) < n
+    assert _equal(Z.query(ix, lr, p), ref)
+    ctx.sync_status()
+
+
+@pytest.mark.parametrize("n_pairs,L,hits", [(150001, 16, 1), (300007, 12, 3)])
+@pytest.mark.parametrize("prec", [0, 1])
+def test_many_super_tiles(n_pairs, L, hits, prec):
+    # more than 32 super tiles (131,072 entries): the visits' parts, the
+    # seeds' second key a lane, ragged last tiles of both kinds
+    import paper_1004_3980_gb300 as Z
+    ctx = Z.Context(0)
+    ix = _index_on(ctx, n_pairs, n_train=21, L=L, k=14, min_table_hits=hits)
+    lr = torch.from_numpy(S.make_image(7, 260, 271)).cuda()
+    a = Z.query(ix, lr, Z.UpscaleParams(K=7, precision=prec))
+    b = Z.query(ix, lr, Z.UpscaleParams(K=7, precision=prec, search=2 if prec else 1))
+    ctx.sync_status()
+    assert _equal(a, b)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_pixels_that_are_no_numbers(prec):
+    # NaN, infinite and very large pixels: their queries find what the scan
+    # finds, and the others beside them too
+    import paper_1004_3980_gb300 as Z
+    ctx = Z.Context(0)
+    ix = _index_on(ctx, 70001)
+    img = S.make_image(1, 180, 170)
+    img[20, 30], img[21, 90], img[100, 5], img[150, 150] = np.nan, np.inf, -np.inf, 1e30
+    img[60, 60], img[120:124, 40:44] = 300.0, 1e6
+    lr = torch.from_numpy(img).cuda()
+    a = Z.query(ix, lr, Z.UpscaleParams(K=8, precision=prec))
+    b = Z.query(ix, lr, Z.UpscaleParams(K=8, precision=prec, search=2 if prec else 1))
+    ctx.sync_status()
+    assert torch.equal(a["nbr"], b["nbr"])
+    assert torch.equal(a["dist"].view(torch.int32), b["dist"].view(torch.int32))
