@@ -19,6 +19,11 @@
 // K-th member found lies within T, the K nearest members are proven; every
 // other query (too few members within T, or more candidates than the list
 // holds) goes to the dense filters and the scan.
+//
+// Where the boxes exclude little (features that do not cluster: noise, a
+// dictionary unlike the image) a round of queries is given up once its lists
+// are longer than the list filter is worth, and its queries go to the dense
+// filters too (PrunePlan::give_up).
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <float.h>
@@ -358,14 +363,16 @@ __global__ void k_radius(const float* __restrict__ ld, int MC, int r, const floa
 // FP16 operations of about 32 instructions a pair); with a query per lane and
 // the boxes broadcast it took 45 and waited for every box.  A lane ends up
 // with the mask of the queries that need its tile: one round of atomics gives
-// the 32 masks their places in the tiles' lists.  2.06M queries on 4M entries:
+// the 32 masks their places in the tiles' lists, and one more counts the
+// pairs of the round: past `give_up` the warps stop.  2.06M queries on 4M entries:
 // 20.8 ms in 32 rounds; 258,064 on 1M: 1.21 ms.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_visit(const uint4* __restrict__ qz, const float* __restrict__ vis,
                                                int nslab, const uint4* __restrict__ box, int nt,
                                                const uint4* __restrict__ sbox, int ns, int parts,
                                                uint16_t* __restrict__ list, uint32_t stride,
-                                               uint32_t* __restrict__ tcnt) {
+                                               uint32_t* __restrict__ tcnt, unsigned long long give_up,
+                                               unsigned long long* __restrict__ pairs) {
   __shared__ uint4 s_z[8][32][2];
   __shared__ float s_T[8][32];
   __shared__ int s_queue[8][64];
@@ -428,6 +435,7 @@ __global__ void __launch_bounds__(256) k_visit(const uint4* __restrict__ qz, con
   };
   int* queue = s_queue[wib];
   int qd = 0;   // tiles queued
+  bool stop = false;
   auto test = [&](int m) {   // the first m (at most 32) queued tiles
     const int t = lane < m ? queue[lane] : -1;
     unsigned mk = 0;
@@ -444,7 +452,10 @@ __global__ void __launch_bounds__(256) k_visit(const uint4* __restrict__ qz, con
       }
     }
     mk = t < 0 ? 0u : mk & act;
+    const uint32_t sum = __reduce_add_sync(kFull, (uint32_t)__popc(mk));
+    const unsigned long long before = lane == 0 && sum ? atomicAdd(pairs, (unsigned long long)sum) : 0ull;
     const uint32_t p = mk ? atomicAdd(tcnt + t, (uint32_t)__popc(mk)) : 0u;
+    stop = __any_sync(kFull, before > give_up);
     for (unsigned any = __ballot_sync(kFull, mk != 0); any; any &= any - 1) {
       const int j = __ffs(any) - 1;
       const int tj = __shfl_sync(kFull, t, j);
@@ -458,12 +469,12 @@ __global__ void __launch_bounds__(256) k_visit(const uint4* __restrict__ qz, con
     __syncwarp();
     qd = rest;
   };
-  for (int s0 = part * 32; s0 < ns; s0 += parts * 32) {
+  for (int s0 = part * 32; s0 < ns && !stop; s0 += parts * 32) {
     const int s = s0 + lane;
     bool keep = false;
     if (s < ns) keep = !(group_bound(sbox + (size_t)s * 4) > Tg);
     unsigned ms = __ballot_sync(kFull, keep);
-    while (ms) {
+    while (ms && !stop) {
       // the tiles of two super tiles at a time, one per lane
       const int b0 = __ffs(ms) - 1;
       ms &= ms - 1;
@@ -480,7 +491,7 @@ __global__ void __launch_bounds__(256) k_visit(const uint4* __restrict__ qz, con
       if (qd >= 32) test(32);
     }
   }
-  if (qd > 0) test(qd);
+  if (qd > 0 && !stop) test(qd);
 }
 
 // ---------------------------------------------------------------------------
@@ -488,9 +499,12 @@ __global__ void __launch_bounds__(256) k_visit(const uint4* __restrict__ qz, con
 // ---------------------------------------------------------------------------
 
 // One block: per tile the number of steps before it (off) and of non-empty
-// tiles before it (ord); off[nt] is the total.
+// tiles before it (ord); off[nt] is the total, or 0 where the round is given
+// up, and off[nt + 1] says so.
 __global__ void __launch_bounds__(1024) k_step_scan(const uint32_t* __restrict__ tcnt, int nt,
-                                                    uint32_t* __restrict__ off, uint32_t* __restrict__ ord) {
+                                                    uint32_t* __restrict__ off, uint32_t* __restrict__ ord,
+                                                    unsigned long long give_up,
+                                                    const unsigned long long* __restrict__ pairs) {
   __shared__ unsigned long long s_w[32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int per = (nt + 1023) / 1024, b0 = threadIdx.x * per;
@@ -526,7 +540,12 @@ __global__ void __launch_bounds__(1024) k_step_scan(const uint32_t* __restrict__
       ord[b0 + i] = (uint32_t)(ex >> 32);
       ex += (unsigned long long)((c + PQ_ROWS - 1) / PQ_ROWS) | ((unsigned long long)(c ? 1u : 0u) << 32);
     }
-  if (threadIdx.x == 1023) off[nt] = (uint32_t)s_w[31];
+  if (threadIdx.x == 1023) {
+    const uint32_t steps = (uint32_t)s_w[31];
+    const bool up = *pairs > give_up || (unsigned long long)steps * PQ_ROWS > give_up + (unsigned long long)nt * PQ_ROWS;
+    off[nt] = up ? 0u : steps;
+    off[nt + 1] = up ? 1u : 0u;
+  }
 }
 
 // A step: x the tile, y its first list entry, z the number of queries, w the
@@ -998,7 +1017,7 @@ __global__ void __launch_bounds__(128) k_rerank_list(
     const uint2* __restrict__ cand, uint32_t cap, const int32_t* __restrict__ order, int64_t nd,
     const float* __restrict__ qfeat, int dpad, const uint64_t* __restrict__ qkeys, const float* __restrict__ dfeat,
     const uint64_t* __restrict__ dkeys, int L, int tmin, int K, FilterError fe, int chunks, float trunc,
-    int64_t tail_q0, int32_t* __restrict__ nbr, float* __restrict__ dist, int32_t* __restrict__ fb_list,
+    int64_t tail_q0, const uint32_t* __restrict__ given_up, int32_t* __restrict__ nbr, float* __restrict__ dist, int32_t* __restrict__ fb_list,
     unsigned long long* __restrict__ fb_count, int32_t* __restrict__ tail_list,
     unsigned long long* __restrict__ tail_count) {
   constexpr int kRow4 = (D + 3) / 4;
@@ -1017,7 +1036,7 @@ __global__ void __launch_bounds__(128) k_rerank_list(
   const int64_t oq = perm[q];
   const float T = rad[q];
   const uint32_t n = qcnt[q];
-  bool flagged = !(T >= 0.f) || n > cap;
+  bool flagged = !(T >= 0.f) || n > cap || *given_up != 0;
   if (!flagged) {
     if (lane < L) s_qk[wib][lane] = qkeys[oq * L + lane];
     if (lane < kRow4) s_q4[wib][lane] = reinterpret_cast<const float4*>(qfeat + oq * dpad)[lane];
@@ -1243,6 +1262,7 @@ struct PruneBufs {
   uint32_t* hist;
   uint16_t *leaf, *qrow, *qop, *list;
   uint32_t *rank, *tcnt, *qcnt, *off, *ord;
+  unsigned long long* pairs;
   uint2* cand;
   float *qn, *ld, *rad, *vis;
   uint4* qz;
@@ -1266,9 +1286,11 @@ size_t carve(zoom_index ix, const PrunePlan& p, int64_t nq, void* ws, PruneBufs*
   b->li = w.take<int32_t>((size_t)nq * p.mc);
   b->rad = w.take<float>(nq);
   b->vis = w.take<float>(nq);
-  b->tcnt = w.take<uint32_t>(nt + p.slab);   // tile counts, then candidate counts: one memset
+  b->tcnt = w.take<uint32_t>(2 + nt + p.slab);   // pairs (64 bits), tile counts, candidate counts: one memset
+  b->pairs = (unsigned long long*)b->tcnt;
+  b->tcnt = b->tcnt ? b->tcnt + 2 : nullptr;
   b->qcnt = b->tcnt ? b->tcnt + nt : nullptr;
-  b->off = w.take<uint32_t>(nt + 1);
+  b->off = w.take<uint32_t>(nt + 2);
   b->ord = w.take<uint32_t>(nt);
   b->tile_of = w.take<int32_t>(nt);
   b->steps = w.take<int4>((size_t)nt + (size_t)nt * p.slab / PQ_ROWS);
@@ -1347,12 +1369,13 @@ cudaError_t run_pruned(zoom_index ix, const PrunePlan& p, const float* qfeat, co
   const int tmin = ix->t;
   for (int64_t q0 = 0; q0 < nq; q0 += p.slab) {
     const int m = (int)(nq - q0 < p.slab ? nq - q0 : p.slab);
-    e = cudaMemsetAsync(b.tcnt, 0, (size_t)(nt + p.slab) * 4, st);
+    e = cudaMemsetAsync(b.pairs, 0, (size_t)(2 + nt + p.slab) * 4, st);
     if (e != cudaSuccess) return e;
     const int warps = (m + 31) / 32 * parts;
+    const unsigned long long give_up = (unsigned long long)m * nt / p.give_up;
     k_visit<<<(warps + 7) / 8, 256, 0, st>>>(b.qz + 2 * q0, b.vis + q0, m, box, nt, sbox, ns, parts, b.list,
-                                             (uint32_t)p.slab, b.tcnt);
-    k_step_scan<<<1, 1024, 0, st>>>(b.tcnt, nt, b.off, b.ord);
+                                             (uint32_t)p.slab, b.tcnt, give_up, b.pairs);
+    k_step_scan<<<1, 1024, 0, st>>>(b.tcnt, nt, b.off, b.ord, give_up, b.pairs);
     k_steps<<<(nt * 8 + 255) / 256, 256, 0, st>>>(b.tcnt, nt, b.off, b.ord, b.steps, b.tile_of);
     TgArgs a;
     a.qrow = b.qrow + (size_t)q0 * p.kc * 8;
@@ -1376,7 +1399,7 @@ cudaError_t run_pruned(zoom_index ix, const PrunePlan& p, const float* qfeat, co
 #define ZOOM_PR_LIST(DD, FF)                                                                                      \
   k_rerank_list<DD, FF><<<(m + 3) / 4, 128, 0, st>>>(                                                           \
       b.perm + q0, b.rad + q0, m, b.qcnt, b.cand, p.cap, ix->tree_order, d->n, qfeat, d->dpad, qkeys, d->feat,  \
-      ix->dkeys, ix->L, tmin, K, fe, p.chunks, p.trunc, p.tail_q0, nbr, dist, fb, fb_count, fb_tail, tail_count)
+      ix->dkeys, ix->L, tmin, K, fe, p.chunks, p.trunc, p.tail_q0, b.off + nt + 1, nbr, dist, fb, fb_count, fb_tail, tail_count)
     switch (d->d + (p.form == 1 ? 100 : 0)) {
       case 9: ZOOM_PR_LIST(9, 2); break;
       case 25: ZOOM_PR_LIST(25, 2); break;

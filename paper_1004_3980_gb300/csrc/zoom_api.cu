@@ -563,8 +563,12 @@ struct SearchPlan {
   int MC2 = 16, nsplit2 = 1;
   // search over the dictionary's search order; the queries it cannot prove
   // go through the split filter: the first cap2 of them over nsplit2
-  // dictionary parts, the rest as one part, then the scan
-  bool pruned = false;
+  // dictionary parts, the rest as one part, then the scan.  With `many` those
+  // past cap2 go through the single-term filter first (nsplit lists of MC), and
+  // what that leaves joins the others, so that data the order does not suit
+  // cost little more than the dense search.
+  bool pruned = false, many = false;
+  int64_t cap_split() const { return many ? 2 * cap2 : cap2; }   // queries of the split filter's first stage
   PrunePlan pp;
   size_t tail_off = 0;   // workspace offset shared by the pruned search and the large split stage
   size_t bytes = 0;
@@ -620,6 +624,7 @@ SearchPlan plan_search(zoom_index ix, const zoom_upscale_params* prm, int64_t nq
     const SearchPlan dense = plan_search(ix, prm, nq, 0, 0, false);
     if (prune_plan(ix, 1, prm->K, nq, &p.pp)) {
       p.pruned = true;
+      p.pp.give_up = nq * d->n >= kPruneGiveUpPairs ? 3 : 1;
       p.pp.chunks = p.MC;
       // packed list keys keep 6 mantissa bits at least
       p.pp.trunc = p.MC == 32 ? 1.05f / 64.f : 0.f;
@@ -628,7 +633,7 @@ SearchPlan plan_search(zoom_index ix, const zoom_upscale_params* prm, int64_t nq
       const int64_t pairs = (nq + 255) / 256, grid = d->ctx->n_sm;
       p.pp.tail_q0 = dense.tail_split > 0 ? std::min<int64_t>(nq, pairs / grid * grid * 256) : 0;
       Carver c(nullptr);
-      c.take<unsigned long long>(4);
+      c.take<unsigned long long>(5);
       c.take<int32_t>(nq);
       c.take<int32_t>(nq);
       c.take<int32_t>(nq);
@@ -646,15 +651,25 @@ SearchPlan plan_search(zoom_index ix, const zoom_upscale_params* prm, int64_t nq
     p.MC2 = tc_list_size(0, prm->K, prm->rerank_mult);
     p.nsplit2 = (int)std::min<int64_t>(8, ix->nd_rows / 128);
     Carver c(nullptr);
-    c.take<unsigned long long>(4);
+    c.take<unsigned long long>(5);
     c.take<int32_t>(nq);
     c.take<int32_t>(nq);
     c.take<int32_t>(nq);
-    take_split(c, ix, p.cap2, p.nsplit2, p.MC2);
+    // (five more launches that mostly find nothing to do, about 15 us: for
+    // calls whose dense search takes a millisecond or more)
+    p.many = nq * d->n >= kPruneManyPairs;
+    if (p.many) c.take<int32_t>(nq);
+    take_split(c, ix, p.cap_split(), p.nsplit2, p.MC2);
     p.tail_off = (c.off + 255) & ~(size_t)255;
-    Carver t(nullptr);
+    Carver t(nullptr), t2(nullptr);
     take_split(t, ix, nq, 1, p.MC2);
-    p.bytes = p.tail_off + std::max(prune_ws_bytes(ix, p.pp, nq), t.off) + 256;
+    if (p.many) {
+      const SearchPlan dense = plan_search(ix, prm, nq, 0, 0, false);
+      p.nsplit = dense.tail_split > 0 ? 1 : dense.nsplit;
+      p.pp.give_up = 3;
+      take_split(t2, ix, nq, p.nsplit, p.MC, 2);
+    }
+    p.bytes = p.tail_off + std::max(prune_ws_bytes(ix, p.pp, nq), std::max(t.off, t2.off)) + 256;
     return p;
   }
   // the narrow forms step through the dictionary 256 rows at a time
@@ -742,10 +757,23 @@ __global__ void k_add_fallback_counts(const unsigned long long* __restrict__ cnt
   counters[CNT_FALLBACK2] += cnt[1];
 }
 
-// The split filter (prec 0) or the precision form's filter (1) on the queries
-// listed in idx[0 .. *cnt) (at most cap of them; the rest are appended to
-// over / *over_cnt), over nsplit dictionary parts; what its rerank leaves
-// joins left / *left_cnt.
+// The queries of a list from `keep` on move to another list; the lists' counts.
+__global__ void k_move_tail(const int32_t* __restrict__ list, const unsigned long long* __restrict__ count,
+                            int64_t keep, int32_t* __restrict__ moved, unsigned long long* __restrict__ n_moved,
+                            unsigned long long* __restrict__ n_kept) {
+  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t n = (int64_t)*count;
+  if (j == 0) {
+    *n_moved = n > keep ? n - keep : 0;
+    *n_kept = n > keep ? keep : n;
+  }
+  if (j >= keep && j < n) moved[j - keep] = list[j];
+}
+
+// The split filter (prec 0), the precision form's (1) or the single-term one
+// (2) on the queries listed in idx[0 .. *cnt) (at most cap of them; the rest
+// are appended to over / *over_cnt), over nsplit dictionary parts; what its
+// rerank leaves joins left / *left_cnt.
 cudaError_t run_split_stage(zoom_index ix, const QueryBufs& q, int prec, int64_t nq, int K, int64_t cap, int nsplit, int MC,
                             const SplitBufs& b, const int32_t* idx, const unsigned long long* cnt, int32_t* over,
                             unsigned long long* over_cnt, int32_t* left, unsigned long long* left_cnt,
@@ -757,11 +785,12 @@ cudaError_t run_split_stage(zoom_index ix, const QueryBufs& q, int prec, int64_t
   if (e == cudaSuccess)
     e = launch_operand(b.feat, d->dpad, d->d, cap, tc_rows_padded(cap, true), 0, prec, b.qop, b.qn, st, cnt);
   if (e == cudaSuccess)
-    e = launch_knn_tc(b.qop, b.qn, cap, prec == 1 ? ix->dopbf : ix->dop16, d->n, prec, tc_kc(d->d, prec), MC, nsplit, 0,
-                      ctx->n_sm, b.ld, b.li, ctx->d_status, st, cnt, ctx->wait_ns, ctx->inject, b.pd, b.pi);
+    e = launch_knn_tc(b.qop, b.qn, cap, prec == 0 ? ix->dop16 : prec == 1 ? ix->dopbf : ix->dopf1, d->n, prec,
+                      tc_kc(d->d, prec), MC, nsplit, 0, ctx->n_sm, b.ld, b.li, ctx->d_status, st, cnt, ctx->wait_ns,
+                      ctx->inject, b.pd, b.pi);
   if (e == cudaSuccess)
     e = launch_rerank(d->d, MC, K, b.feat, d->dpad, b.qn, b.keys, cap, d->feat, ix->dkeys, d->n, ix->L, ix->t, b.ld,
-                      b.li, nsplit, prec == 1 ? 0 : 1, q.nbr, q.dist, left, left_cnt, st, idx, cnt);
+                      b.li, nsplit, prec == 0 ? 1 : prec == 1 ? 0 : 2, q.nbr, q.dist, left, left_cnt, st, idx, cnt);
   return e;
 }
 
@@ -779,9 +808,11 @@ cudaError_t run_search_ws(zoom_index ix, const zoom_upscale_params* prm, const Q
     return launch_knn_exact(ix, b.feat, b.keys, nq, K, b.nbr, b.dist, ctx->d_counters, nullptr,
                             nullptr, st);
   Carver s2(ws);
-  // [0] first list, [1] second (pruned: [0] unproven, [1] left to the scan, [2] past cap2)
-  unsigned long long* cnt = s2.take<unsigned long long>(pl.pruned ? 4 : 2);
-  cudaError_t e = cudaMemsetAsync(cnt, 0, (pl.pruned ? 4 : 2) * sizeof(unsigned long long), st);
+  // [0] first list, [1] second (pruned: [0] unproven, [1] left to the scan,
+  // [2] past the split filter's first stage; many: [4] for the single-term
+  // filter, [3] then for the split filter)
+  unsigned long long* cnt = s2.take<unsigned long long>(pl.pruned ? 5 : 2);
+  cudaError_t e = cudaMemsetAsync(cnt, 0, (pl.pruned ? 5 : 2) * sizeof(unsigned long long), st);
   if (e != cudaSuccess) return e;
   if (pl.pruned) {
     int32_t* fb = s2.take<int32_t>(nq);
@@ -813,12 +844,22 @@ cudaError_t run_search_ws(zoom_index ix, const zoom_upscale_params* prm, const Q
       }
       return e;
     }
-    const SplitBufs sa = take_split(s2, ix, pl.cap2, pl.nsplit2, pl.MC2);
+    // (the pruned search's buffers are free now)
+    int32_t* far = pl.many ? s2.take<int32_t>(nq) : nullptr;
+    const SplitBufs sa = take_split(s2, ix, pl.cap_split(), pl.nsplit2, pl.MC2);
+    const unsigned long long* n_first = cnt;
+    if (e == cudaSuccess && pl.many) {
+      k_move_tail<<<(unsigned)((nq + 255) / 256), 256, 0, st>>>(fb, cnt, pl.cap2, far, cnt + 4, cnt + 3);
+      Carver t(tail);
+      const SplitBufs sb = take_split(t, ix, nq, pl.nsplit, pl.MC, 2);
+      e = run_split_stage(ix, b, 2, nq, K, nq, pl.nsplit, pl.MC, sb, far, cnt + 4, nullptr, nullptr, fb, cnt + 3, st);
+      n_first = cnt + 3;
+    }
     if (e == cudaSuccess)
-      e = run_split_stage(ix, b, 0, nq, K, pl.cap2, pl.nsplit2, pl.MC2, sa, fb, cnt, more, cnt + 2, fb2, cnt + 1, st);
-    // the pruned search's buffers are free now: the queries past cap2, as
-    // one dictionary part each
-    if (e == cudaSuccess && pl.cap2 < nq) {
+      e = run_split_stage(ix, b, 0, nq, K, pl.cap_split(), pl.nsplit2, pl.MC2, sa, fb, n_first, more, cnt + 2, fb2, cnt + 1,
+                          st);
+    // the queries past that, as one dictionary part each
+    if (e == cudaSuccess && pl.cap_split() < nq) {
       Carver t(tail);
       const SplitBufs sb = take_split(t, ix, nq, 1, pl.MC2);
       e = run_split_stage(ix, b, 0, nq, K, nq, 1, pl.MC2, sb, more, cnt + 2, nullptr, nullptr, fb2, cnt + 1, st);

@@ -236,6 +236,8 @@ constexpr int64_t kPruneMaxEntries = int64_t{2048} * 16 * 256;
 // 593 / 652 with 300,000; 4,224 queries 535 / 500 with 300,000.
 constexpr int64_t kPruneMinQueries = 20000;        // ... or
 constexpr int64_t kPruneMinPairs = 2500000000;     // queries x entries
+constexpr int64_t kPruneManyPairs = 15000000000;   // from here on: SearchPlan::many
+constexpr int64_t kPruneGiveUpPairs = 5000000000;  // BF16: rounds may be given up
 struct PrunePlan {
   int form = 2, kc = 4, mc = 16, r = 12;
   int64_t slab = 0;      // queries per round of visits and filter steps
@@ -245,6 +247,15 @@ struct PrunePlan {
   int chunks = 16;
   float trunc = 0.f;
   int64_t tail_q0 = 0;
+  // a round is given up past 1 / give_up of its (query, tile) pairs (1: never).
+  // A pair costs the list filter 2.2 times what it costs the dense one (1,080
+  // cycles a 128 x 256 step against 985 a 256 x 256 one), and the seeds and
+  // visits come on top: 3 where a dense filter of the same form takes over and
+  // is not done soon anyway.  Pixels of noise, ms given up / not / by the dense
+  // search: 512 x 512 with 1M entries exact 17.8 / 34.3 / 15.0, BF16 16.8 /
+  // 36.9 / 14.8; 280 x 280 with 300,000 2.94 / 3.96 / 2.19 and 2.86 / 4.27 /
+  // 2.09; 160 x 160 with 65,536 in BF16 0.83 / 0.73 / 0.54.
+  int give_up = 1;
 };
 bool prune_plan(zoom_index ix, int form, int K, int64_t nq, PrunePlan* p);
 size_t prune_ws_bytes(zoom_index ix, const PrunePlan& p, int64_t nq);

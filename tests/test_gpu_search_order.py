@@ -181,3 +181,25 @@ def test_pixels_that_are_no_numbers(prec):
     ctx.sync_status()
     assert torch.equal(a["nbr"], b["nbr"])
     assert torch.equal(a["dist"].view(torch.int32), b["dist"].view(torch.int32))
+
+
+@pytest.mark.parametrize("prec,n_pairs,h,w", [(0, 200_003, 280, 281), (1, 120_001, 260, 281)])
+def test_noise_is_given_up_for_the_dense_filters(prec, n_pairs, h, w):
+    # Uniform noise: a query's radius reaches nearly every tile's box.  Every
+    # round is given up (all its queries counted as left), and the dense
+    # filters find the scan's and the dense search's neighbours.
+    import paper_1004_3980_gb300 as Z
+    g = np.random.default_rng(8)
+    n_train = n_pairs // 15000 + 1
+    train = [torch.from_numpy(g.random((256, 256), dtype=np.float32)).cuda() for _ in range(n_train)]
+    ctx = Z.Context(0)
+    dic = Z.Dictionary(ctx, train, S.sample_positions(5, n_train, 128, 128, 5, n_pairs), 2, 5)
+    a, b = S.lsh_draws(6, 8, 12, 25, 64.0)
+    ix = Z.Index(dic, 8, 12, 64.0, a, b)
+    lr = torch.from_numpy(g.random((h, w), dtype=np.float32)).cuda()
+    got = Z.query(ix, lr, Z.UpscaleParams(K=8, precision=prec))
+    st = ctx.stats()
+    ref = Z.query(ix, lr, Z.UpscaleParams(K=8, precision=prec, search=2 if prec else 1))
+    ctx.sync_status()
+    assert st["n_filter_fallback"] == st["n_queries"] == (h - 4) * (w - 4)
+    assert _equal(got, ref)
