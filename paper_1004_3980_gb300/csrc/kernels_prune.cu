@@ -1225,9 +1225,16 @@ cudaError_t run_tg(const TgArgs& a, int grid, cudaStream_t st) {
 // host side
 // ---------------------------------------------------------------------------
 
-bool prune_plan(zoom_index ix, int form, int K, int64_t nq, PrunePlan* p) {
-  if (ix->tree_tiles == 0 || K > 16) return false;
-  if (nq < kPruneMinQueries && nq * ix->dict->n < kPruneMinPairs) return false;
+// Where the search order is the faster search (zoom_internal.h has both sides).
+static bool takes_search_order(int64_t n, int form, int K, int chunks, int64_t nq) {
+  const bool bf16 = form == 1, few = bf16 && chunks < 2 * K;
+  if (few && K > 12) return false;
+  if (nq >= kPruneMinQueries) return !(bf16 && K < 6 && n < 131072 && nq < 4 * kPruneMinQueries);
+  return nq * n >= kPruneMinPairs[bf16] && nq >= kPruneFewQueries[few ? 2 : bf16];
+}
+
+bool prune_plan(zoom_index ix, int form, int K, int chunks, int64_t nq, PrunePlan* p) {
+  if (ix->tree_tiles == 0 || K > 16 || !takes_search_order(ix->dict->n, form, K, chunks, nq)) return false;
   p->form = form;
   p->kc = tc_kc(ix->dict->d, form);
   // the seeds' list must hold the r-th chunk minimum: two more than K, so

@@ -622,7 +622,7 @@ SearchPlan plan_search(zoom_index ix, const zoom_upscale_params* prm, int64_t nq
   if (may_prune && p.prec == 1) {
     // the precision form's dense plan says what its lists are
     const SearchPlan dense = plan_search(ix, prm, nq, 0, 0, false);
-    if (prune_plan(ix, 1, prm->K, nq, &p.pp)) {
+    if (prune_plan(ix, 1, prm->K, p.MC, nq, &p.pp)) {
       p.pruned = true;
       p.pp.give_up = nq * d->n >= kPruneGiveUpPairs ? 3 : 1;
       p.pp.chunks = p.MC;
@@ -645,7 +645,7 @@ SearchPlan plan_search(zoom_index ix, const zoom_upscale_params* prm, int64_t nq
       return p;
     }
   }
-  if (may_prune && p.prec == 2 && prune_plan(ix, 2, prm->K, nq, &p.pp)) {
+  if (may_prune && p.prec == 2 && prune_plan(ix, 2, prm->K, p.MC, nq, &p.pp)) {
     p.pruned = true;
     p.cap2 = std::min<int64_t>(nq, std::max<int64_t>(8192, nq / 64));
     p.MC2 = tc_list_size(0, prm->K, prm->rerank_mult);

@@ -229,13 +229,25 @@ FilterError tc_filter_error(int d, int precision);
 // search over the dictionary's search order (kernels_prune.cu)
 constexpr int64_t kPruneMinEntries = 65536;   // dictionaries that get a search order
 constexpr int64_t kPruneMaxEntries = int64_t{2048} * 16 * 256;
-// The searches that use it.  The stages before the filter cost about 300 us
-// whatever the size.  Against the dense search (L = 8..16, K = 8, one
-// image's queries; auto / dense us): 24,382 queries 468 / 596 with 70,000
-// entries and 733 / 993 with 200,000; 9,312 queries 567 / 394 with 200,000,
-// 593 / 652 with 300,000; 4,224 queries 535 / 500 with 300,000.
-constexpr int64_t kPruneMinQueries = 20000;        // ... or
-constexpr int64_t kPruneMinPairs = 2500000000;     // queries x entries
+// The searches that use it (takes_search_order): those where it was the faster
+// one over both pixel features and first-order 3 x 3 gradients (dense time /
+// its time, queries in thousands):
+//   20 and more queries: exact, K = 3: 0.95 to 1.13 with 65,536 to 131,072
+//   entries, 1.29 to 3.5 from 262,144 on; K = 8 to 16: 1.2 to 3.4.  BF16: K = 8
+//   1.02 to 1.23 and 1.24 to 2.2, but K = 3 0.89 to 1.05 below 131,072 entries
+//   (1.0 to 1.2 from 80 queries on).
+//   fewer, exact: 1.0 to 2.6 from 7e9 query-entry pairs on with 5 or more (1M
+//   entries, 7.4: 1.10, 1.00, 1.62 for K = 3, 8, 12; 2M, 3.6: 0.80 to 1.63);
+//   before that 0.57 to 1.46, the lower ones where no query needs the dense
+//   search's second filter.
+//   fewer, BF16: 1.08 to 2.2 from 1.2e10 pairs on with 6 or more (2M, 7.4: 1.09;
+//   2M, 3.6: 0.80; 1M, 7.4: 0.98).
+//   BF16 whose lists hold fewer than 2 K chunks leaves more queries to the dense
+//   filter: K = 12 and 16 chunks 0.72 to 1.07 with 7.4, 1.03 and more from 15
+//   on; K = 16 and 16 chunks 0.5 to 1.0 nearly everywhere.
+constexpr int64_t kPruneMinQueries = 20000;
+constexpr int64_t kPruneMinPairs[2] = {7000000000, 12000000000};      // exact, BF16; and at least
+constexpr int64_t kPruneFewQueries[3] = {5000, 6000, 15000};          // exact, BF16, BF16 with short lists
 constexpr int64_t kPruneManyPairs = 15000000000;   // from here on: SearchPlan::many
 constexpr int64_t kPruneGiveUpPairs = 5000000000;  // BF16: rounds may be given up
 struct PrunePlan {
@@ -257,7 +269,8 @@ struct PrunePlan {
   // 2.09; 160 x 160 with 65,536 in BF16 0.83 / 0.73 / 0.54.
   int give_up = 1;
 };
-bool prune_plan(zoom_index ix, int form, int K, int64_t nq, PrunePlan* p);
+// chunks: the chunks a query the dense filter of the form lists
+bool prune_plan(zoom_index ix, int form, int K, int chunks, int64_t nq, PrunePlan* p);
 size_t prune_ws_bytes(zoom_index ix, const PrunePlan& p, int64_t nq);
 // Neighbours of nq queries into nbr / dist; those it cannot prove are
 // appended to fb (count *fb_count, zeroed by the caller); in the precision
