@@ -399,12 +399,14 @@ def order_launches(nq: int, n_pairs: int, precision: int) -> int:
     sorted (3), seeds (2) and radii; per round of queries the visits, the
     steps (2), the list filter and the rerank; the queries left over through
     the dense filter in two parts (gather, operand, filter, lists joined,
-    rerank each), the SIMT re-run and the fallback count."""
-    if not 65_536 <= n_pairs <= 2048 * 16 * 256 or (nq < 20_000 and nq * n_pairs < 2_500_000_000):
+    rerank each; large exact searches have a third, and a list moved), the
+    SIMT re-run and the fallback count.  For this file's workloads (K = 8)."""
+    if not 65_536 <= n_pairs <= 2048 * 16 * 256 or nq < 20_000:
         return 0
     tiles = -(-n_pairs // 256)
     per_round = min(2**31 // (2 * tiles) // 256 * 256, 65_280, -(-nq // 256) * 256)
-    return 6 + 5 * -(-nq // per_round) + 10 + 2 - (9 if precision == 0 else 5)
+    third = 6 if precision == 0 and nq * n_pairs >= 15_000_000_000 else 0
+    return 6 + 5 * -(-nq // per_round) + 10 + third + 2 - (9 if precision == 0 else 5)
 
 
 def max_over_ranks(ms: float, world: int, device: str) -> float:

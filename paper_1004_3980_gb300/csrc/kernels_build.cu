@@ -797,46 +797,6 @@ size_t csr_scratch_bytes(int64_t n) {
   return (size_t)(2 * n * 8 + 2 * n * 4 + hist * 4 + 2 * n * 4 + nseg * 4 + 1024);
 }
 
-size_t sort_rank16_scratch_bytes(int64_t n) {
-  const int64_t ntiles = (n + RS_TILE - 1) / RS_TILE;
-  const int64_t hist = 256 * ntiles;
-  return (size_t)n * 2 + 256 + (size_t)n * 2 + 256 + (size_t)n * 4 + 256 + (size_t)hist * 4 + 256 +
-         (size_t)((hist + SCAN_SEG - 1) / SCAN_SEG) * 4 + 256;
-}
-
-// Stable sort of 0..n-1 by a 16-bit rank below 2^bits (ids[n]; the ranks
-// are kept): one or two passes of the tables' radix kernels.
-cudaError_t sort_rank16(const uint16_t* rank, int64_t n, int bits, int32_t* ids, void* scratch,
-                        size_t scratch_bytes, cudaStream_t st) {
-  if (scratch_bytes < sort_rank16_scratch_bytes(n) || n >= (int64_t{1} << 31)) return cudaErrorInvalidValue;
-  const int ntiles = (int)((n + RS_TILE - 1) / RS_TILE);
-  char* p = (char*)scratch;
-  auto take = [&](size_t bytes) {
-    char* r = p;
-    p += (bytes + 255) & ~(size_t)255;
-    return r;
-  };
-  uint16_t* ra = (uint16_t*)take((size_t)n * 2);
-  uint16_t* rb = (uint16_t*)take((size_t)n * 2);
-  int32_t* va = (int32_t*)take((size_t)n * 4);
-  int32_t* hist = (int32_t*)take((size_t)256 * ntiles * 4);
-  int32_t* part = (int32_t*)p;
-  const int passes = bits <= 8 ? 1 : 2;
-  const uint16_t* rin = rank;
-  const int32_t* iin = nullptr;
-  for (int ps = 0; ps < passes; ++ps) {
-    int32_t* iout = ps == passes - 1 ? ids : va;
-    uint16_t* rout = ps == 0 ? ra : rb;
-    k_rank_hist_b<<<dim3(ntiles, 1), RS_THREADS, 0, st>>>(rin, n, 8 * ps, hist, ntiles);
-    cudaError_t e = exclusive_scan(hist, hist, (int64_t)256 * ntiles, part, st);
-    if (e != cudaSuccess) return e;
-    k_rank_scatter_b<<<dim3(ntiles, 1), RS_THREADS, 0, st>>>(rin, iin, rout, iout, n, 8 * ps, hist, ntiles);
-    rin = rout;
-    iin = iout;
-  }
-  return cudaGetLastError();
-}
-
 size_t csr_build_scratch_bytes(int64_t n, int L) {
   // the radix sort's buffers, then the key sets, the slot ranks, the per-table
   // flags, the 16-bit ranks of every entry in every table (twice) and their

@@ -60,6 +60,7 @@ __global__ void __launch_bounds__(128) k_query_route(const float* __restrict__ f
   for (int t = threadIdx.x; t < D * PZ; t += 128) s_b[t] = basis[t];
   __syncthreads();
   const int64_t q = (int64_t)blockIdx.x * 128 + threadIdx.x;
+  const unsigned active = __ballot_sync(kFull, q < nq);
   if (q >= nq) return;
   float f[D], z[PZ];
   load_feature<D>(feat + q * dpad, f);
@@ -68,42 +69,7 @@ __global__ void __launch_bounds__(128) k_query_route(const float* __restrict__ f
   for (int c = 0; c < PZ; ++c) s_z[c][threadIdx.x] = z[c];
   const int lf = tree_leaf(node1, node2, d1, d2, [&](int c) { return s_z[c][threadIdx.x]; });
   leaf[q] = (uint16_t)lf;
-  rank[q] = atomicAdd(hist + lf, 1u);
-}
-
-// One block: hist[n] -> exclusive prefix sums in place.
-__global__ void __launch_bounds__(1024) k_leaf_scan(uint32_t* __restrict__ hist, int n) {
-  __shared__ uint32_t s_w[32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int per = (n + 1023) / 1024, b0 = threadIdx.x * per;
-  uint32_t acc = 0;
-  for (int i = 0; i < per; ++i)
-    if (b0 + i < n) acc += hist[b0 + i];
-  uint32_t x = acc;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_up_sync(kFull, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) s_w[warp] = x;
-  __syncthreads();
-  if (warp == 0) {
-    uint32_t w = s_w[lane];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(kFull, w, o);
-      if (lane >= o) w += y;
-    }
-    s_w[lane] = w;
-  }
-  __syncthreads();
-  uint32_t ex = x - acc + (warp ? s_w[warp - 1] : 0u);
-  for (int i = 0; i < per; ++i)
-    if (b0 + i < n) {
-      const uint32_t t = hist[b0 + i];
-      hist[b0 + i] = ex;
-      ex += t;
-    }
+  rank[q] = leaf_arrival(hist, lf, active);
 }
 
 // Writes every query's operand row (row-major, and in the tile layout of the

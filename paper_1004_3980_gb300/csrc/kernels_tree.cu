@@ -6,10 +6,12 @@
 //
 // The tree splits each node at its sample median in the bound coordinate of
 // largest variance.  Two levels of sampling keep it to a few launches: one
-// block builds the first d1 levels from 2048 entries in shared memory; up to
-// 1536 further samples per leaf are routed there, and one block per leaf
+// block builds the first d1 levels from up to 2048 entries in shared memory; up
+// to 1536 further samples per leaf are routed there, and one block per leaf
 // builds d2 more levels.  Every entry is then routed (a lookup per level) and
-// the entries are sorted stably by leaf with the index's 16-bit radix passes.
+// numbered by arrival at its leaf; the leaves' counts summed give its place
+// (two 8-bit radix passes instead took ten launches, 90 us with 65,536 entries,
+// 15 us so).
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <float.h>
@@ -33,7 +35,7 @@ __device__ __forceinline__ uint32_t order_key(float f) {
 
 struct TreeSmem {
   float z[PZ][PT_TOP];
-  uint64_t key[PT_TOP];
+  uint32_t key[PT_TOP];
   uint16_t perm[PT_TOP];
   float var[128 * PZ];
   int dim[128];
@@ -77,25 +79,32 @@ __device__ void kd_build(TreeSmem& s, int n, int depth, TreeNode* __restrict__ o
     __syncthreads();
     for (int t = tid; t < n; t += kTreeThreads) {
       const uint16_t p = s.perm[t];
-      s.key[t] = ((uint64_t)order_key(s.z[s.dim[t / m]][p]) << 16) | p;
+      // (the value's upper 21 bits: what they round only moves a split a little)
+      s.key[t] = (order_key(s.z[s.dim[t / m]][p]) & ~(uint32_t)(PT_TOP - 1)) | p;
     }
     __syncthreads();
-    // bitonic sort of every node's m keys, all nodes ascending
+    // bitonic sort of every node's m keys, all nodes ascending; a thread has
+    // one pair a stage, so that a warp's pairs at distances up to 32 lie in 64
+    // keys of its own and only the longer distances need the block's barrier
+    static_assert(PT_TOP <= 2 * kTreeThreads && (PT_TOP & (PT_TOP - 1)) == 0, "one pair a thread");
     for (int k = 2; k <= m; k <<= 1) {
+      if (k > 64) __syncthreads();
       for (int j = k >> 1; j > 0; j >>= 1) {
-        for (int i = tid; i < n / 2; i += kTreeThreads) {
-          const int a = ((i & ~(j - 1)) << 1) | (i & (j - 1)), b = a | j;
+        const int a = ((tid & ~(j - 1)) << 1) | (tid & (j - 1)), b = a | j;
+        if (tid < n / 2) {
           const bool up = k == m || (a & k) == 0;
-          const uint64_t x = s.key[a], y = s.key[b];
+          const uint32_t x = s.key[a], y = s.key[b];
           if ((x > y) == up) {
             s.key[a] = y;
             s.key[b] = x;
           }
         }
-        __syncthreads();
+        if (j > 32) __syncthreads();
+        else __syncwarp();
       }
     }
-    for (int t = tid; t < n; t += kTreeThreads) s.perm[t] = (uint16_t)(s.key[t] & 0xFFFFu);
+    __syncthreads();
+    for (int t = tid; t < n; t += kTreeThreads) s.perm[t] = (uint16_t)(s.key[t] & (PT_TOP - 1));
     __syncthreads();
     for (int q = tid; q < nn; q += kTreeThreads)
       out[nn + q] = TreeNode{s.z[s.dim[q]][s.perm[q * m + m / 2 - 1]], s.dim[q]};
@@ -107,11 +116,13 @@ struct DctBasis {
   float b[25 * 25];   // [pixel][coefficient] of a P x P block
 };
 
-// One block: the variances of all D coefficients over PT_TOP entries spread
-// over the dictionary, the PZ largest as the basis, and the first d1 levels.
+// One block: the variances of all D coefficients over ns (a power of two, at
+// most PT_TOP) entries spread over the dictionary, the PZ largest as the basis,
+// and the first d1 levels.
 template <int D>
 __global__ void __launch_bounds__(kTreeThreads) k_tree_top(const float* __restrict__ feat, int dpad, int64_t n,
-                                                           DctBasis dct, int P2, int d1, float* __restrict__ basis,
+                                                           DctBasis dct, int P2, int ns, int d1,
+                                                           float* __restrict__ basis,
                                                            TreeNode* __restrict__ node1) {
   extern __shared__ __align__(16) unsigned char raw[];
   TreeSmem& s = *reinterpret_cast<TreeSmem*>(raw);
@@ -125,8 +136,10 @@ __global__ void __launch_bounds__(kTreeThreads) k_tree_top(const float* __restri
   float f[2][D];
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
-    const int64_t e = (int64_t)(tid + h * kTreeThreads) * n / PT_TOP;
-    load_feature<D>(feat + e * dpad, f[h]);
+#pragma unroll
+    for (int i = 0; i < D; ++i) f[h][i] = 0.f;
+    const int j = tid + h * kTreeThreads;
+    if (j < ns) load_feature<D>(feat + (int64_t)j * n / ns * dpad, f[h]);
   }
   __syncthreads();
   constexpr int kBlocks = D == 18 ? 2 : 1;   // [g_x | g_y]
@@ -159,16 +172,25 @@ __global__ void __launch_bounds__(kTreeThreads) k_tree_top(const float* __restri
       a += s_part[tid][0][w];
       b += s_part[tid][1][w];
     }
-    s_v[tid] = b - a * a / (float)PT_TOP;
+    s_v[tid] = b - a * a / (float)ns;
   }
   __syncthreads();
-  if (tid == 0) {
+  if (warp == 0) {
+    // the PZ largest, one after the other (equal ones: the lower number); NaN
+    // is none
+    static_assert(D <= 32, "a coefficient a lane");
+    uint64_t key =
+        lane < D && s_v[lane] > -FLT_MAX ? ((uint64_t)order_key(s_v[lane]) << 32) | (uint32_t)(64 - lane) : 0ull;
     for (int c = 0; c < PZ; ++c) {
-      int best = -1;
-      for (int i = 0; i < D; ++i)
-        if (s_v[i] > -FLT_MAX && (best < 0 || s_v[i] > s_v[best])) best = i;
-      s_pick[c] = best;   // -1: fewer coefficients than PZ (the column is zero)
-      if (best >= 0) s_v[best] = -FLT_MAX;
+      uint64_t g = key;
+#pragma unroll
+      for (int o = 16; o; o >>= 1) {
+        const uint64_t x = __shfl_xor_sync(0xffffffffu, g, o);
+        g = g > x ? g : x;
+      }
+      const int best = g ? 64 - (int)(uint32_t)g : -1;
+      if (lane == 0) s_pick[c] = best;   // -1: fewer coefficients than PZ (the column is zero)
+      if (best == lane) key = 0;
     }
   }
   __syncthreads();
@@ -187,7 +209,7 @@ __global__ void __launch_bounds__(kTreeThreads) k_tree_top(const float* __restri
     for (int c = 0; c < PZ; ++c) s.z[c][tid + h * kTreeThreads] = z[c];
   }
   __syncthreads();
-  kd_build(s, PT_TOP, d1, node1);
+  kd_build(s, ns, d1, node1);
 }
 
 // m samples spread over the dictionary, routed through the first d1 levels
@@ -233,25 +255,36 @@ __global__ void __launch_bounds__(kTreeThreads) k_tree_sub(const uint32_t* __res
   kd_build(s, n, d2, node2 + ((size_t)blockIdx.x << d2));
 }
 
-// Leaf of every entry.
+// Leaf of every entry, and its arrival number there (counts: hist).
 template <int D>
 __global__ void __launch_bounds__(128) k_tree_route(const float* __restrict__ feat, int dpad, int64_t n,
                                                     const float* __restrict__ basis,
                                                     const TreeNode* __restrict__ node1,
                                                     const TreeNode* __restrict__ node2, int d1, int d2,
-                                                    uint16_t* __restrict__ leaf) {
+                                                    uint16_t* __restrict__ leaf, uint32_t* __restrict__ rank,
+                                                    uint32_t* __restrict__ hist) {
   __shared__ __align__(16) float s_b[D * PZ];
   __shared__ float s_z[PZ][128];
   for (int t = threadIdx.x; t < D * PZ; t += 128) s_b[t] = basis[t];
   __syncthreads();
   const int64_t i = (int64_t)blockIdx.x * 128 + threadIdx.x;
+  const unsigned active = __ballot_sync(0xffffffffu, i < n);
   if (i >= n) return;
   float f[D], z[PZ];
   load_feature<D>(feat + i * dpad, f);
   bound_coords<D>(f, reinterpret_cast<const float4*>(s_b), z);
 #pragma unroll
   for (int c = 0; c < PZ; ++c) s_z[c][threadIdx.x] = z[c];
-  leaf[i] = (uint16_t)tree_leaf(node1, node2, d1, d2, [&](int c) { return s_z[c][threadIdx.x]; });
+  const int lf = tree_leaf(node1, node2, d1, d2, [&](int c) { return s_z[c][threadIdx.x]; });
+  leaf[i] = (uint16_t)lf;
+  rank[i] = leaf_arrival(hist, lf, active);
+}
+
+__global__ void __launch_bounds__(256) k_tree_place(const uint16_t* __restrict__ leaf, const uint32_t* __restrict__ rank,
+                                                    const uint32_t* __restrict__ offs, int64_t n,
+                                                    int32_t* __restrict__ order) {
+  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (i < n) order[(int64_t)offs[leaf[i]] + rank[i]] = (int32_t)i;
 }
 
 // Scaled FP16 box of [lo, hi] with the coordinates' rounding allowed for:
@@ -428,8 +461,8 @@ size_t tree_scratch_bytes(int64_t n) {
   int d1, d2;
   tree_depths(n, &d1, &d2);
   const int64_t nt = (n + PT_ROWS - 1) / PT_ROWS;
-  return ((size_t)1 << d1) * (4 + (size_t)PT_TOP * PZ * 4) + 256 + (size_t)n * 2 + 256 +
-         (size_t)nt * (3 * PZ + 1) * 4 + 256 + sort_rank16_scratch_bytes(n) + 256;
+  return ((size_t)1 << d1) * (4 + (size_t)PT_TOP * PZ * 4) + 256 + (size_t)n * (2 + 4) + 512 +
+         (size_t)nt * (3 * PZ + 1) * 4 + 256 + ((size_t)4 << (d1 + d2)) + 256;
 }
 
 // Builds the index's search order: basis, tree, order, operands, boxes.
@@ -449,10 +482,15 @@ cudaError_t build_search_tree(zoom_index ix, void* scratch, size_t scratch_bytes
   uint32_t* cnt = (uint32_t*)take(((size_t)1 << d1) * 4);
   uint16_t* leaf = (uint16_t*)take((size_t)n * 2);
   float* stat = (float*)take((size_t)nt * (3 * PZ + 1) * 4);
-  void* sort_ws = p;
-  const int64_t m = std::min<int64_t>(n, (int64_t)1536 << d1);
+  uint32_t* rank = (uint32_t*)take((size_t)n * 4);
+  uint32_t* hist = (uint32_t*)take((size_t)4 << (d1 + d2));
+  const int leaves = 1 << (d1 + d2);
+  // samples: 32 or so for every leaf of either level's tree
+  const int top = std::min(PT_TOP, 32 << d1);
+  const int64_t m = std::min<int64_t>(n, (int64_t)std::min(1536, 48 << d2) << d1);
   const DctBasis dct = dct_basis(d->P);
   cudaError_t e = cudaMemsetAsync(cnt, 0, ((size_t)1 << d1) * 4, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(hist, 0, (size_t)leaves * 4, st);
   if (e != cudaSuccess) return e;
   const int smem = (int)sizeof(TreeSmem);
   TreeNode* node1 = (TreeNode*)ix->tree_node1;
@@ -461,14 +499,14 @@ cudaError_t build_search_tree(zoom_index ix, void* scratch, size_t scratch_bytes
   do {                                                                                                         \
     e = cudaFuncSetAttribute(k_tree_top<DD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);                \
     if (e != cudaSuccess) return e;                                                                            \
-    k_tree_top<DD><<<1, kTreeThreads, smem, st>>>(d->feat, d->dpad, n, dct, d->P * d->P, d1, ix->tree_basis,     \
+    k_tree_top<DD><<<1, kTreeThreads, smem, st>>>(d->feat, d->dpad, n, dct, d->P * d->P, top, d1, ix->tree_basis, \
                                                   node1);                                                      \
     k_tree_sample<DD><<<(unsigned)((m + 127) / 128), 128, 0, st>>>(d->feat, d->dpad, n, m, ix->tree_basis, node1, \
                                                                    d1, cnt, zl);                               \
   } while (0)
 #define ZOOM_TREE_B(DD)                                                                                      \
   k_tree_route<DD><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(d->feat, d->dpad, n, ix->tree_basis, node1, node2, \
-                                                                d1, d2, leaf)
+                                                                d1, d2, leaf, rank, hist)
 #define ZOOM_TREE_C(DD)                                                                                       \
   k_tile_operands<DD, 4><<<nt, PT_ROWS, 0, st>>>(d->feat, d->dpad, n, ix->tree_order,        \
                                                                       ix->tree_basis, ix->tree_f1, ix->tree_bf, \
@@ -485,8 +523,8 @@ cudaError_t build_search_tree(zoom_index ix, void* scratch, size_t scratch_bytes
   if (e != cudaSuccess) return e;
   k_tree_sub<<<1 << d1, kTreeThreads, smem, st>>>(cnt, zl, d2, node2);
   ZOOM_TREE(ZOOM_TREE_B)
-  e = sort_rank16(leaf, n, d1 + d2, ix->tree_order, sort_ws, sort_rank16_scratch_bytes(n), st);
-  if (e != cudaSuccess) return e;
+  k_leaf_scan<<<1, 1024, 0, st>>>(hist, leaves);
+  k_tree_place<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(leaf, rank, hist, n, ix->tree_order);
   ZOOM_TREE(ZOOM_TREE_C)
   k_super_boxes<<<(ns + 3) / 4, 128, 0, st>>>(stat, n, nt, ns, (uint4*)ix->tree_sbox, ix->tree_smid);
   return cudaGetLastError();

@@ -82,6 +82,54 @@ __device__ __forceinline__ int tree_leaf(const TreeNode* __restrict__ node1, con
   return (a << d2) | tree_descend(node2 + ((size_t)a << d2), d2, zc);
 }
 
+// This lane's arrival number at leaf lf, counted in hist; one atomic per leaf
+// and warp (flat images send thousands of rows to one leaf).  active: the lanes
+// here.
+__device__ __forceinline__ uint32_t leaf_arrival(uint32_t* __restrict__ hist, int lf, unsigned active) {
+  const int lane = threadIdx.x & 31;
+  const unsigned same = __match_any_sync(active, lf);
+  const int lead = __ffs(same) - 1;
+  uint32_t base = 0;
+  if (lane == lead) base = atomicAdd(hist + lf, (uint32_t)__popc(same));
+  base = __shfl_sync(active, base, lead);
+  return base + (uint32_t)__popc(same & ((1u << lane) - 1u));
+}
+
+// One block: hist[n] -> exclusive prefix sums in place.
+__global__ void __launch_bounds__(1024) k_leaf_scan(uint32_t* __restrict__ hist, int n) {
+  __shared__ uint32_t s_w[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int per = (n + 1023) / 1024, b0 = threadIdx.x * per;
+  uint32_t acc = 0;
+  for (int i = 0; i < per; ++i)
+    if (b0 + i < n) acc += hist[b0 + i];
+  uint32_t x = acc;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) s_w[warp] = x;
+  __syncthreads();
+  if (warp == 0) {
+    uint32_t w = s_w[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, w, o);
+      if (lane >= o) w += y;
+    }
+    s_w[lane] = w;
+  }
+  __syncthreads();
+  uint32_t ex = x - acc + (warp ? s_w[warp - 1] : 0u);
+  for (int i = 0; i < per; ++i)
+    if (b0 + i < n) {
+      const uint32_t t = hist[b0 + i];
+      hist[b0 + i] = ex;
+      ex += t;
+    }
+}
+
 // A box in the scaled FP16 bound coordinates: 16 centres, 16 half widths
 // (64 bytes).
 struct alignas(16) BoxH {

@@ -141,11 +141,6 @@ size_t csr_scratch_bytes(int64_t n);
 // scratch of build_csr_tables: the radix sort's plus the key compaction's
 size_t csr_build_scratch_bytes(int64_t n, int L);
 
-// stable sort by 16-bit ranks below 2^bits
-size_t sort_rank16_scratch_bytes(int64_t n);
-cudaError_t sort_rank16(const uint16_t* rank, int64_t n, int bits, int32_t* ids, void* scratch,
-                        size_t scratch_bytes, cudaStream_t st);
-
 // search order of the dictionary (kernels_tree.cu)
 void tree_depths(int64_t n, int* d1, int* d2);
 size_t tree_scratch_bytes(int64_t n);
