@@ -117,14 +117,6 @@ struct TcArgs {
   // nq_dev != nullptr: only the first min(*nq_dev, nq) queries are searched
   // (a count written by an earlier kernel); nq stays the lists' row stride
   const unsigned long long* nq_dev;
-  // part_d / part_id (with nq_dev): room for 2 * gridDim.x parts of 256
-  // queries' lists.  Where the count is small the dictionary part of a list
-  // is cut into fan_out() equal pieces, each with lists of its own there,
-  // and k_merge_parts joins them: a few hundred queries would otherwise
-  // leave most SMs idle (124 queries, 1M entries, 8 parts: 475 us on 8 SMs,
-  // 55 us so).
-  float* part_d = nullptr;
-  int32_t* part_id = nullptr;
   // bound on every wait (ns), and the testing aid: inject == 1 makes each
   // CTA's epilogue withhold the release of its accumulators from the third
   // tile of its first item on, so the issuing threads' waits run out
@@ -133,9 +125,24 @@ struct TcArgs {
   // packed chunk lists (the BF16 form of the wide-step filter): bits of a
   // list key that hold the chunk number
   int id_bits;
-  // wide-step filter over a step list: pair qp's step t is the dictionary
-  // step step_tiles[qp * nd_tiles + t] (nullptr: step t itself); the chunk
-  // numbers written are then those of the list
+};
+
+// ... and what only searches beside the dense one need.  A struct of its own:
+// the dense wide-step filter's code is sensitive to its parameters' places (with
+// these among them the K = 64 form took 2,040 us for 689,272 entries, 1,890
+// without, and the K = 32 form up to 2 % more).
+struct TcMore : TcArgs {
+  // part_d / part_id (with nq_dev): room for 2 * gridDim.x parts of 256
+  // queries' lists.  Where the count is small the dictionary part of a list
+  // is cut into fan_out() equal pieces, each with lists of its own there,
+  // and k_merge_parts joins them: a few hundred queries would otherwise
+  // leave most SMs idle (124 queries, 1M entries, 8 parts: 475 us on 8 SMs,
+  // 55 us so).
+  float* part_d = nullptr;
+  int32_t* part_id = nullptr;
+  // wide-step filter over a step list (kTwSteps): pair qp's step t
+  // is the dictionary step step_tiles[qp * nd_tiles + t]; the chunk numbers
+  // written are then those of the list
   const int32_t* step_tiles = nullptr;
 };
 
@@ -181,27 +188,44 @@ struct WorkIter {
       }
     } else {
       const int item = c + k * G;
-      const int m = a.part_d ? fan_out(nq_pairs, a.nsplit, G) : 1;
-      if (item >= a.nsplit * m * nq_pairs) return false;
+      if (item >= a.nsplit * nq_pairs) return false;
       seg = item / nq_pairs;
       qp = item % nq_pairs;
-      const int s = seg / m, j = seg - s * m;   // piece j of list s
-      t0 = s * a.tiles_per_split;
+      t0 = seg * a.tiles_per_split;
       t1 = min(a.nd_tiles, t0 + a.tiles_per_split);
-      if (m > 1) {
-        const int n = t1 - t0;
-        t1 = t0 + (int)((int64_t)n * (j + 1) / m);
-        t0 += (int)((int64_t)n * j / m);
-      }
     }
     ++k;
     return true;
   }
 };
 
+// The same with lists in pieces.
+struct WorkIterMore {
+  int k = 0;
+  __device__ bool next(const TcMore& a, int& qp, int& seg, int& t0, int& t1) {
+    const int G = gridDim.x, c = blockIdx.x;
+    const int nq_pairs = a.nq_dev ? (int)((searched_queries(a) + 2 * TC_ROWS - 1) / (2 * TC_ROWS)) : a.nq_pairs;
+    if (!a.part_d) {
+      WorkIter it;
+      it.k = k++;
+      return it.next(a, qp, seg, t0, t1);
+    }
+    const int m = fan_out(nq_pairs, a.nsplit, G);
+    const int item = c + k++ * G;
+    if (item >= a.nsplit * m * nq_pairs) return false;
+    seg = item / nq_pairs;
+    qp = item % nq_pairs;
+    const int s = seg / m, j = seg - s * m;   // piece j of list s
+    const int p0 = s * a.tiles_per_split, n = min(a.nd_tiles, p0 + a.tiles_per_split) - p0;
+    t0 = p0 + (int)((int64_t)n * j / m);
+    t1 = p0 + (int)((int64_t)n * (j + 1) / m);
+    return true;
+  }
+};
+
 // Where list `seg` of query q goes, and what is added to its values: ||q||^2,
 // or nothing in a piece's list (k_merge_parts adds it to what it keeps).
-__device__ __forceinline__ int64_t list_row(const TcArgs& a, int seg, int64_t q, float*& d, int32_t*& id, float& qn) {
+__device__ __forceinline__ int64_t list_row(const TcMore& a, int seg, int64_t q, float*& d, int32_t*& id, float& qn) {
   d = a.out_d;
   id = a.out_id;
   if (a.part_d) {
@@ -260,7 +284,7 @@ __device__ __forceinline__ void chunk_test(float m, int chunk, float thr, float*
 }
 
 template <int KC, int MC, uint32_t AB_TYPE>
-__global__ void __maxnreg__(tc_max_regs(KC, MC)) k_knn_tc(TcArgs a) {
+__global__ void __maxnreg__(tc_max_regs(KC, MC)) k_knn_tc(TcMore a) {
   constexpr int kMma = tc_mma_warps(KC, MC);
   constexpr bool kOneRound = tc_one_round(KC, MC);
   constexpr uint32_t kTileBytes = KC * TC_ROWS * 16;  // one 128-row operand tile
@@ -323,7 +347,7 @@ __global__ void __maxnreg__(tc_max_regs(KC, MC)) k_knn_tc(TcArgs a) {
       bool first = true;
       int a_copies = 0;
       int64_t b_copies = 0;
-      WorkIter it;
+      WorkIterMore it;
       int qp, seg, t0, t1;
       while (!*abort_flag && it.next(a, qp, seg, t0, t1)) {
         if (!first) {
@@ -369,7 +393,7 @@ __global__ void __maxnreg__(tc_max_regs(KC, MC)) k_knn_tc(TcArgs a) {
       const uint64_t bd0 = smem_desc(smem_u32(sB), TC_ROWS * 16, 128);
       constexpr uint64_t kKStepAdv = (2 * TC_ROWS * 16) >> 4;
       constexpr uint64_t kTileAdv = kTileBytes >> 4;
-      WorkIter it;
+      WorkIterMore it;
       int qp, seg, t0, t1;
       while (!*abort_flag && it.next(a, qp, seg, t0, t1)) {
         if (!mbar_wait_fast(a_full, a_phase, abort_flag, a.status, a.wait_ns)) break;
@@ -426,7 +450,7 @@ __global__ void __maxnreg__(tc_max_regs(KC, MC)) k_knn_tc(TcArgs a) {
     // (two arrivals free it), which keeps that commit off the MMA threads.
     int stage = 0;
     const bool releaser = (ew & 3) == 0 && lane == 0;
-    WorkIter it;
+    WorkIterMore it;
     int qp, split, t0, t1;
     int item_no = 0;
     while (it.next(a, qp, split, t0, t1)) {
@@ -740,8 +764,15 @@ __host__ __device__ constexpr uint32_t instr_desc_wide(uint32_t ab_type) {
          ((uint32_t)(TC_ROWS >> 4) << 24);
 }
 
-template <int KC, int MC, uint32_t AB_TYPE, bool PACKED>
-__global__ void __launch_bounds__(352, 1) k_knn_tw(TcArgs a) {
+// MODE 0: the queries' number is known; 1: that, over a step list; 2: it is on
+// the device and lists may be in pieces.
+enum { kTwDense, kTwSteps, kTwCounted };
+template <int MODE>
+using TwArgs = typename std::conditional<MODE == kTwDense, TcArgs, TcMore>::type;
+template <int MODE>
+using TwIter = typename std::conditional<MODE == kTwDense, WorkIter, WorkIterMore>::type;
+template <int KC, int MC, uint32_t AB_TYPE, bool PACKED, int MODE>
+__global__ void __launch_bounds__(352, 1) k_knn_tw(TwArgs<MODE> a) {
   constexpr uint32_t kATile = KC * TC_ROWS * 16;     // one 128-row query tile
   constexpr uint32_t kStep = KC * TW_ROWS * 16;      // one 256-row dictionary step
   constexpr int kKSteps = KC / 2;
@@ -800,7 +831,7 @@ __global__ void __launch_bounds__(352, 1) k_knn_tw(TcArgs a) {
       bool first = true;
       int a_copies = 0;
       int64_t b_copies = 0;
-      WorkIter it;
+      TwIter<MODE> it;
       int qp, seg, t0, t1;
       while (!*abort_flag && it.next(a, qp, seg, t0, t1)) {
         if (!first) {
@@ -814,7 +845,8 @@ __global__ void __launch_bounds__(352, 1) k_knn_tw(TcArgs a) {
         for (int t = t0; t < t1; ++t) {
           if (!mbar_wait_fast(b_empty + stage, phase ^ 1u, abort_flag, a.status, a.wait_ns)) break;
           mbar_arrive_expect_tx(b_full + stage, kStep);
-          const size_t step = a.step_tiles ? (size_t)a.step_tiles[(size_t)qp * a.nd_tiles + t] : (size_t)t;
+          size_t step = (size_t)t;
+          if constexpr (MODE == kTwSteps) step = (size_t)a.step_tiles[(size_t)qp * a.nd_tiles + t];
           bulk_g2s(sB + stage * kStep, (const unsigned char*)a.dop + step * kStep, kStep, b_full + stage);
           ++b_copies;
           if (++stage == kStages) {
@@ -841,7 +873,7 @@ __global__ void __launch_bounds__(352, 1) k_knn_tw(TcArgs a) {
       constexpr uint64_t kBStep = (2 * TW_ROWS * 16) >> 4;
       constexpr uint64_t kStageAdv = kStep >> 4;
       const uint32_t d_addr = tmem + (uint32_t)(qt * TW_ROWS);
-      WorkIter it;
+      TwIter<MODE> it;
       int qp, seg, t0, t1;
       while (!*abort_flag && it.next(a, qp, seg, t0, t1)) {
         if (!mbar_wait_fast(a_full, a_phase, abort_flag, a.status, a.wait_ns)) break;
@@ -904,13 +936,14 @@ __global__ void __launch_bounds__(352, 1) k_knn_tw(TcArgs a) {
     const bool releaser = quad == 0 && lane == 0;   // frees each step's ring stage (one per query tile)
     int stage = 0, item_no = 0;
     uint32_t accp = 0;
-    WorkIter it;
+    TwIter<MODE> it;
     int qp, split, t0, t1;
     while (it.next(a, qp, split, t0, t1)) {
       if (__any_sync(kFull, *abort_flag != 0)) break;   // warp-uniform exit
       const bool withhold = a.inject == 1 && item_no++ == 0;   // testing aid (see TcArgs)
       const int64_t q = ((int64_t)qp * 2 + qt) * TC_ROWS + row;
-      const bool valid = q < searched_queries(a);
+      bool valid = q < a.nq;
+      if constexpr (MODE == kTwCounted) valid = q < searched_queries(a);
       const float qn = valid ? a.qn[q] : 0.f;
       if constexpr (PACKED) L.qn = qn;
       L.init();
@@ -962,11 +995,15 @@ __global__ void __launch_bounds__(352, 1) k_knn_tw(TcArgs a) {
       if (!ok) break;
       L.flush();
       if (valid) {
-        float* od;
-        int32_t* oi;
-        float add = qn;
-        const int64_t lrow = list_row(a, split, q, od, oi, add);
-        L.write(add, a.nd, od + lrow * MC, oi + lrow * MC);
+        if constexpr (MODE == kTwCounted) {
+          float* od;
+          int32_t* oi;
+          float add = qn;
+          const int64_t lrow = list_row(a, split, q, od, oi, add);
+          L.write(add, a.nd, od + lrow * MC, oi + lrow * MC);
+        } else {
+          L.write(qn, a.nd, a.out_d + ((int64_t)split * a.nq + q) * MC, a.out_id + ((int64_t)split * a.nq + q) * MC);
+        }
         if (a.tail_split > 0 && t0 == 0 && t1 == a.nd_tiles) {
           for (int s2 = 1; s2 < a.tail_split; ++s2) {
             float* od1 = a.out_d + ((int64_t)s2 * a.nq + q) * MC;
@@ -1567,9 +1604,9 @@ size_t tw_smem_bytes(int KC, int MC, bool packed) {
 
 bool tc_wide_form(int precision, int kc) { return precision != 0 && (kc == 4 || kc == 8); }
 
-template <int KC, int MC, uint32_t T, bool P>
-static cudaError_t run_tw_kernel(const TcArgs& args, int grid, cudaStream_t st) {
-  auto kern = k_knn_tw<KC, MC, T, P>;
+template <int KC, int MC, uint32_t T, bool P, int MODE>
+static cudaError_t run_tw_kernel(const TwArgs<MODE>& args, int grid, cudaStream_t st) {
+  auto kern = k_knn_tw<KC, MC, T, P, MODE>;
   const size_t smem = tw_smem_bytes(KC, MC, P);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -1582,7 +1619,7 @@ static cudaError_t run_tw_kernel(const TcArgs& args, int grid, cudaStream_t st) 
 }
 
 template <int KC, int MC, uint32_t T>
-static cudaError_t run_tc_kernel(const TcArgs& args, int grid, size_t smem, cudaStream_t st) {
+static cudaError_t run_tc_kernel(const TcMore& args, int grid, size_t smem, cudaStream_t st) {
   auto kern = k_knn_tc<KC, MC, T>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -1659,7 +1696,7 @@ static cudaError_t knn_tc(const uint16_t* qop, const float* qn, int64_t nq, cons
   if (tc_wide_form(precision, kc)) {
     // the wide-step kernel: items of 256 queries x a part of the 256-row steps
     if ((nq_dev && tail_split > 0) || (MC != 16 && MC != 32)) return cudaErrorInvalidValue;
-    TcArgs a;
+    TcMore a;
     a.part_d = parts.d;
     a.part_id = parts.id;
     a.wait_ns = wait_ns > 0 ? wait_ns : kWaitNs;
@@ -1684,18 +1721,25 @@ static cudaError_t knn_tc(const uint16_t* qop, const float* qn, int64_t nq, cons
     a.full_rounds = tail_split > 0 ? a.nq_pairs / grid : 0;
     a.id_bits = chunk_bits(nd);
     const bool packed = packed_lists(precision, kc, MC, nd);
-#define ZOOM_TW(KC, T) \
-  return MC == 16 ? run_tw_kernel<KC, 16, T, false>(a, grid, st) : run_tw_kernel<KC, 32, T, false>(a, grid, st)
-    if (precision == 1 && kc == 4 && packed) return run_tw_kernel<4, 32, 1, true>(a, grid, st);
-    if (precision == 1 && kc == 8 && packed) return run_tw_kernel<8, 32, 1, true>(a, grid, st);
-    if (precision == 2 && kc == 4) ZOOM_TW(4, 0);
-    if (precision == 2 && kc == 8) ZOOM_TW(8, 0);
-    if (precision == 1 && kc == 4) ZOOM_TW(4, 1);
-    if (precision == 1 && kc == 8) ZOOM_TW(8, 1);
+#define ZOOM_TW(KC, T, MODE)                                                     \
+  return MC == 16 ? run_tw_kernel<KC, 16, T, false, MODE>(a, grid, st)            \
+                  : run_tw_kernel<KC, 32, T, false, MODE>(a, grid, st)
+    if (nq_dev) {   // what a search over the search order leaves (narrow features)
+      if (kc != 4) return cudaErrorInvalidValue;
+      if (packed) return run_tw_kernel<4, 32, 1, true, kTwCounted>(a, grid, st);
+      if (precision == 2) ZOOM_TW(4, 0, kTwCounted);
+      ZOOM_TW(4, 1, kTwCounted);
+    }
+    if (precision == 1 && kc == 4 && packed) return run_tw_kernel<4, 32, 1, true, kTwDense>(a, grid, st);
+    if (precision == 1 && kc == 8 && packed) return run_tw_kernel<8, 32, 1, true, kTwDense>(a, grid, st);
+    if (precision == 2 && kc == 4) ZOOM_TW(4, 0, kTwDense);
+    if (precision == 2 && kc == 8) ZOOM_TW(8, 0, kTwDense);
+    if (precision == 1 && kc == 4) ZOOM_TW(4, 1, kTwDense);
+    if (precision == 1 && kc == 8) ZOOM_TW(8, 1, kTwDense);
 #undef ZOOM_TW
     return cudaErrorInvalidValue;
   }
-  TcArgs a;
+  TcMore a;
   a.part_d = parts.d;
   a.part_id = parts.id;
   a.wait_ns = wait_ns > 0 ? wait_ns : kWaitNs;
@@ -1736,7 +1780,7 @@ static cudaError_t knn_tc(const uint16_t* qop, const float* qn, int64_t nq, cons
 cudaError_t launch_knn_seeds(const uint16_t* qop, const float* qn, int64_t nq, const uint16_t* dop, int64_t nd,
                              int precision, int kc, int MC, const int32_t* seeds, int grid, float* out_d,
                              int32_t* out_id, unsigned int* status, cudaStream_t st, uint64_t wait_ns, int inject) {
-  TcArgs a{};
+  TcMore a{};
   a.wait_ns = wait_ns > 0 ? wait_ns : kWaitNs;
   a.inject = inject;
   a.qop = qop;
@@ -1754,7 +1798,8 @@ cudaError_t launch_knn_seeds(const uint16_t* qop, const float* qn, int64_t nq, c
   a.step_tiles = seeds;
   grid = grid < a.nq_pairs ? grid : a.nq_pairs;
 #define ZOOM_TW(KC, T) \
-  return MC == 16 ? run_tw_kernel<KC, 16, T, false>(a, grid, st) : run_tw_kernel<KC, 32, T, false>(a, grid, st)
+  return MC == 16 ? run_tw_kernel<KC, 16, T, false, kTwSteps>(a, grid, st) \
+                  : run_tw_kernel<KC, 32, T, false, kTwSteps>(a, grid, st)
   if (MC != 16 && MC != 32) return cudaErrorInvalidValue;
   if (precision == 2 && kc == 4) ZOOM_TW(4, 0);
   if (precision == 1 && kc == 4) ZOOM_TW(4, 1);
