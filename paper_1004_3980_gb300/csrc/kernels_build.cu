@@ -137,10 +137,12 @@ __global__ void __launch_bounds__(kGatherRows) k_dict_gather(
 // R feature rows and the block's tables (blockIdx.y: a share of the L), whose
 // alpha / beta are staged in shared memory.  Bound by the multiply-adds (L k D
 // a row) and the operations beside them:
-// - two rows a thread share each 16-byte read of the projections;
+// - two rows a thread share each 16-byte read of the projections, where the rows
+//   are many and long enough (launch_hash);
 // - floor(t / w) comes from a multiplication with 1 / w unless the product
 //   lies within its error of a whole number (or is not finite, or so small
-//   that it could have been rounded to 0), which takes the division;
+//   that it could have been rounded to 0), which takes the division (one short
+//   row a thread divides: its multiply-adds leave no room for the tests);
 // - a pair of keys leaves in one 16-byte store.
 // 1M rows, D = 25, L = k = 16: 755 us with one row a thread and a division a
 // projection, 631 us so.  Few rows split the tables over blocks instead.
@@ -208,10 +210,15 @@ __global__ void __launch_bounds__(128) k_hash(const float* __restrict__ feat, in
       for (int y = 0; y < R; ++y) {
         const float t = acc[y] + be;
         // t * rw is within 2^-23 |t / w| of t / w, the quotient within 2^-24
-        const float u = t * rw;
-        float fl = floorf(u);
-        const float off = fabsf(u - rintf(u));
-        if (!(off > 4e-7f * fabsf(u) && off > 1e-30f && fabsf(u) < 1e9f)) fl = floorf(__fdiv_rn(t, w));
+        float fl;
+        bool divide = true;
+        if constexpr (R > 1 || D >= 25) {
+          const float u = t * rw;
+          fl = floorf(u);
+          const float off = fabsf(u - rintf(u));
+          divide = !(off > 4e-7f * fabsf(u) && off > 1e-30f && fabsf(u) < 1e9f);
+        }
+        if (divide) fl = floorf(__fdiv_rn(t, w));
         x[y] = zoom_fold_step(x[y], (int)fl, j);
       }
     }
@@ -706,11 +713,14 @@ cudaError_t launch_dict_gather(const float* const* d_lr_images, const int32_t* d
 cudaError_t launch_hash(const float* feat, int dpad, int d, int64_t n, const float* alpha,
                         const float* beta, int L, int k, float w, uint64_t* keys, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
-  // two rows a thread where that leaves two blocks of 128 for each of about
-  // 150 SMs, else one, with the tables (in twos: see the stores) over blocks
-  // until there are as many (the 2x zoom of
-  // 64x64 with 3,844 queries: 189.6 us on 31 blocks, 182.9 us so)
-  const bool two = n >= 2 * 128 * 304;
+  // Two rows a thread where that was faster (L = k = 16, one / two rows, us):
+  // D = 9 never (258,064 rows 136 / 144, 1M 450 / 452), D = 18 from 800,000 rows
+  // (515,524: 307 / 311, 1M: 564 / 546), D = 25 from 100,000 (81,796: 101 / 108,
+  // 112,896: 112 / 102, 1M: 706 / 641), D = 50 from two blocks of 128 for each
+  // of about 150 SMs (81,796: 194 / 157).  With one row the tables (in twos: see
+  // the stores) go over blocks until there are as many (the 2x zoom of 64x64
+  // with 3,844 queries: 189.6 us on 31 blocks, 182.9 us so).
+  const bool two = n >= (d == 50 ? 2 * 128 * 304 : d == 25 ? 100000 : d == 18 ? 800000 : INT64_MAX);
   const int64_t rows = two ? 256 : 128, blocks = (n + rows - 1) / rows;
   int per = (L + 1) / 2 * 2;
   while (per > 2 && blocks * ((L + per - 1) / per) < 304) per = (per / 2 + 1) / 2 * 2;
