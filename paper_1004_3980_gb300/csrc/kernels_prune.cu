@@ -329,8 +329,8 @@ __global__ void k_radius(const float* __restrict__ ld, int MC, int r, const floa
 // FP16 operations of about 32 instructions a pair); with a query per lane and
 // the boxes broadcast it took 45 and waited for every box.  A lane ends up
 // with the mask of the queries that need its tile: one round of atomics gives
-// the 32 masks their places in the tiles' lists, and one more counts the
-// pairs of the round: past `give_up` the warps stop.  2.06M queries on 4M entries:
+// the 32 masks their places in the tiles' lists.  The pairs of the round are
+// counted, too: past `give_up` the warps stop.  2.06M queries on 4M entries:
 // 20.8 ms in 32 rounds; 258,064 on 1M: 1.21 ms.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_visit(const uint4* __restrict__ qz, const float* __restrict__ vis,
@@ -401,6 +401,12 @@ __global__ void __launch_bounds__(256) k_visit(const uint4* __restrict__ qz, con
   };
   int* queue = s_queue[wib];
   int qd = 0;   // tiles queued
+  // Pairs not yet in the round's count: a warp adds them an eighth of its
+  // (query, tile) pairs at a time, so that few do where the boxes exclude much
+  // (an atomic on one address per 32 tiles made 258,064 queries on 1M entries
+  // 5.34 -> 5.47 ms).  k_step_scan sees what stays uncounted in the lists.
+  const uint32_t hold = (uint32_t)(4 * nt / parts + 1);
+  uint32_t held = 0;
   bool stop = false;
   auto test = [&](int m) {   // the first m (at most 32) queued tiles
     const int t = lane < m ? queue[lane] : -1;
@@ -418,10 +424,13 @@ __global__ void __launch_bounds__(256) k_visit(const uint4* __restrict__ qz, con
       }
     }
     mk = t < 0 ? 0u : mk & act;
-    const uint32_t sum = __reduce_add_sync(kFull, (uint32_t)__popc(mk));
-    const unsigned long long before = lane == 0 && sum ? atomicAdd(pairs, (unsigned long long)sum) : 0ull;
+    held += __reduce_add_sync(kFull, (uint32_t)__popc(mk));
     const uint32_t p = mk ? atomicAdd(tcnt + t, (uint32_t)__popc(mk)) : 0u;
-    stop = __any_sync(kFull, before > give_up);
+    if (held >= hold) {
+      const unsigned long long before = lane == 0 ? atomicAdd(pairs, (unsigned long long)held) : 0ull;
+      stop = __any_sync(kFull, before > give_up);
+      held = 0;
+    }
     for (unsigned any = __ballot_sync(kFull, mk != 0); any; any &= any - 1) {
       const int j = __ffs(any) - 1;
       const int tj = __shfl_sync(kFull, t, j);
