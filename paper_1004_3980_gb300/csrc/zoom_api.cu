@@ -624,7 +624,7 @@ SearchPlan plan_search(zoom_index ix, const zoom_upscale_params* prm, int64_t nq
     const SearchPlan dense = plan_search(ix, prm, nq, 0, 0, false);
     if (prune_plan(ix, 1, prm->K, p.MC, nq, &p.pp)) {
       p.pruned = true;
-      p.pp.give_up = nq * d->n >= kPruneGiveUpPairs ? 3 : 1;
+      p.pp.give_up = nq * d->n >= kPruneGiveUpPairs ? 2 : 1;
       p.pp.chunks = p.MC;
       // packed list keys keep 6 mantissa bits at least
       p.pp.trunc = p.MC == 32 ? 1.05f / 64.f : 0.f;
@@ -666,7 +666,7 @@ SearchPlan plan_search(zoom_index ix, const zoom_upscale_params* prm, int64_t nq
     if (p.many) {
       const SearchPlan dense = plan_search(ix, prm, nq, 0, 0, false);
       p.nsplit = dense.tail_split > 0 ? 1 : dense.nsplit;
-      p.pp.give_up = 3;
+      p.pp.give_up = 2;
       take_split(t2, ix, nq, p.nsplit, p.MC, 2);
     }
     p.bytes = p.tail_off + std::max(prune_ws_bytes(ix, p.pp, nq), std::max(t.off, t2.off)) + 256;

@@ -257,11 +257,13 @@ struct PrunePlan {
   // a round is given up past 1 / give_up of its (query, tile) pairs (1: never).
   // A pair costs the list filter 2.2 times what it costs the dense one (1,080
   // cycles a 128 x 256 step against 985 a 256 x 256 one), and the seeds and
-  // visits come on top: 3 where a dense filter of the same form takes over and
-  // is not done soon anyway.  Pixels of noise, ms given up / not / by the dense
-  // search: 512 x 512 with 1M entries exact 17.8 / 34.3 / 15.0, BF16 16.8 /
-  // 36.9 / 14.8; 280 x 280 with 300,000 2.94 / 3.96 / 2.19 and 2.86 / 4.27 /
-  // 2.09; 160 x 160 with 65,536 in BF16 0.83 / 0.73 / 0.54.
+  // visits come on top: 2 where a dense filter of the same form takes over and
+  // is not done soon anyway (3 gave rounds of ordinary images up: 280 x 280
+  // with 300,000 entries 3.2 instead of 2.4 ms, sixteen images 56 instead of
+  // 52).  Pixels of noise, ms given up / not / by the dense search: 512 x 512
+  // with 1M entries exact 18.4 / 34.3 / 15.0, BF16 17.4 / 36.8 / 14.9; 280 x 280
+  // with 300,000 3.00 / 3.99 / 2.17 and 2.92 / 4.27 / 2.07; 160 x 160 with
+  // 65,536 in BF16 0.83 (at 3) / 0.71 / 0.56.
   int give_up = 1;
 };
 // chunks: the chunks a query the dense filter of the form lists
