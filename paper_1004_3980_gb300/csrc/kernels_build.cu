@@ -231,6 +231,9 @@ __global__ void __launch_bounds__(128) k_hash(const float* __restrict__ feat, in
       held[y] = x[y];
     }
   }
+  // Launched beside the kernel before it (launch_hash): that one has to be
+  // complete before this one is, for what follows both on the stream.
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // ---------------------------------------------------------------------------
@@ -711,7 +714,8 @@ cudaError_t launch_dict_gather(const float* const* d_lr_images, const int32_t* d
 }
 
 cudaError_t launch_hash(const float* feat, int dpad, int d, int64_t n, const float* alpha,
-                        const float* beta, int L, int k, float w, uint64_t* keys, cudaStream_t st) {
+                        const float* beta, int L, int k, float w, uint64_t* keys, cudaStream_t st,
+                        bool beside) {
   if (n == 0) return cudaSuccess;
   // Two rows a thread where that was faster (L = k = 16, one / two rows, us):
   // D = 9 never (258,064 rows 136 / 144, 1M 450 / 452), D = 18 from 800,000 rows
@@ -725,15 +729,24 @@ cudaError_t launch_hash(const float* feat, int dpad, int d, int64_t n, const flo
   int per = (L + 1) / 2 * 2;
   while (per > 2 && blocks * ((L + per - 1) / per) < 304) per = (per / 2 + 1) / 2 * 2;
   const size_t smem = (size_t)(per < L ? per : L) * k * ((d + 3) / 4 * 4 + 1) * sizeof(float);
-  const dim3 grid((unsigned)blocks, (unsigned)((L + per - 1) / per));
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)blocks, (unsigned)((L + per - 1) / per));
+  cfg.blockDim = dim3(128);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = beside ? 1 : 0;
+  cudaError_t e = cudaSuccess;
 #define ZOOM_HASH1(DD, RR)                                                                                  \
   do {                                                                                                      \
     if (smem > 48 * 1024) {                                                                                 \
-      const cudaError_t e =                                                                                 \
-          cudaFuncSetAttribute(k_hash<DD, RR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);     \
+      e = cudaFuncSetAttribute(k_hash<DD, RR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);     \
       if (e != cudaSuccess) return e;                                                                       \
     }                                                                                                       \
-    k_hash<DD, RR><<<grid, 128, smem, st>>>(feat, dpad, n, alpha, beta, L, per, k, w, keys);                \
+    e = cudaLaunchKernelEx(&cfg, k_hash<DD, RR>, feat, dpad, n, alpha, beta, L, per, k, w, keys);           \
   } while (0)
 #define ZOOM_HASH(DD)            \
   do {                           \
@@ -749,7 +762,7 @@ cudaError_t launch_hash(const float* feat, int dpad, int d, int64_t n, const flo
   }
 #undef ZOOM_HASH1
 #undef ZOOM_HASH
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 namespace {

@@ -26,6 +26,9 @@
 namespace {
 
 constexpr int kTreeThreads = 1024;
+// The first level's sample counts lie in cache lines of their own: 98,304
+// samples that all counted in two lines took 35 us, 15 us so.
+constexpr int kCountStride = 32;
 
 // Order-preserving 32-bit key of an FP32 value.
 __device__ __forceinline__ uint32_t order_key(float f) {
@@ -118,7 +121,10 @@ struct DctBasis {
 
 // One block: the variances of all D coefficients over ns (a power of two, at
 // most PT_TOP) entries spread over the dictionary, the PZ largest as the basis,
-// and the first d1 levels.
+// and the first d1 levels.  Bound by the barriers and shared memory of its one
+// SM (73 us with 512 entries, 108 with 2048), so the next kernel is let in at
+// once: with the hash beside it the build of 200,000 pairs takes 675 us instead
+// of 780.
 template <int D>
 __global__ void __launch_bounds__(kTreeThreads) k_tree_top(const float* __restrict__ feat, int dpad, int64_t n,
                                                            DctBasis dct, int P2, int ns, int d1,
@@ -132,6 +138,7 @@ __global__ void __launch_bounds__(kTreeThreads) k_tree_top(const float* __restri
   __shared__ int s_pick[PZ];
   __shared__ __align__(16) float s_b[D * PZ];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   for (int t = tid; t < P2 * P2; t += kTreeThreads) s_dct[t] = dct.b[t];
   float f[2][D];
 #pragma unroll
@@ -231,7 +238,7 @@ __global__ void __launch_bounds__(128) k_tree_sample(const float* __restrict__ f
 #pragma unroll
   for (int c = 0; c < PZ; ++c) s_z[c][threadIdx.x] = z[c];
   const int leaf = tree_descend(node1, d1, [&](int c) { return s_z[c][threadIdx.x]; });
-  const uint32_t slot = atomicAdd(cnt + leaf, 1u);
+  const uint32_t slot = atomicAdd(cnt + leaf * kCountStride, 1u);
   if (slot < PT_TOP) {
     float4* o = reinterpret_cast<float4*>(zl + ((size_t)leaf * PT_TOP + slot) * PZ);
 #pragma unroll
@@ -245,7 +252,7 @@ __global__ void __launch_bounds__(kTreeThreads) k_tree_sub(const uint32_t* __res
                                                            TreeNode* __restrict__ node2) {
   extern __shared__ __align__(16) unsigned char raw[];
   TreeSmem& s = *reinterpret_cast<TreeSmem*>(raw);
-  const int have = (int)min(cnt[blockIdx.x], (uint32_t)PT_TOP);
+  const int have = (int)min(cnt[blockIdx.x * kCountStride], (uint32_t)PT_TOP);
   int n = 1;
   while (2 * n <= have) n *= 2;
   if (have == 0) n = 0;
@@ -461,11 +468,35 @@ size_t tree_scratch_bytes(int64_t n) {
   int d1, d2;
   tree_depths(n, &d1, &d2);
   const int64_t nt = (n + PT_ROWS - 1) / PT_ROWS;
-  return ((size_t)1 << d1) * (4 + (size_t)PT_TOP * PZ * 4) + 256 + (size_t)n * (2 + 4) + 512 +
+  return ((size_t)1 << d1) * (kCountStride * 4 + (size_t)PT_TOP * PZ * 4) + 256 + (size_t)n * (2 + 4) + 512 +
          (size_t)nt * (3 * PZ + 1) * 4 + 256 + ((size_t)4 << (d1 + d2)) + 256;
 }
 
-// Builds the index's search order: basis, tree, order, operands, boxes.
+cudaError_t launch_tree_top(zoom_index ix, cudaStream_t st) {
+  zoom_dict d = ix->dict;
+  const int top = std::min(PT_TOP, 32 << ix->tree_d1);   // samples: 32 or so for every leaf
+  const DctBasis dct = dct_basis(d->P);
+  const int smem = (int)sizeof(TreeSmem);
+  cudaError_t e;
+#define ZOOM_TREE_TOP(DD)                                                                                        \
+  do {                                                                                                           \
+    e = cudaFuncSetAttribute(k_tree_top<DD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);                  \
+    if (e != cudaSuccess) return e;                                                                              \
+    k_tree_top<DD><<<1, kTreeThreads, smem, st>>>(d->feat, d->dpad, d->n, dct, d->P * d->P, top, ix->tree_d1,      \
+                                                  ix->tree_basis, (TreeNode*)ix->tree_node1);                    \
+  } while (0)
+  switch (d->d) {
+    case 9: ZOOM_TREE_TOP(9); break;
+    case 25: ZOOM_TREE_TOP(25); break;
+    case 18: ZOOM_TREE_TOP(18); break;
+    default: return cudaErrorInvalidValue;
+  }
+#undef ZOOM_TREE_TOP
+  return cudaGetLastError();
+}
+
+// Builds the index's search order below the first levels: tree, order,
+// operands, boxes.
 cudaError_t build_search_tree(zoom_index ix, void* scratch, size_t scratch_bytes, cudaStream_t st) {
   zoom_dict d = ix->dict;
   const int64_t n = d->n;
@@ -479,31 +510,23 @@ cudaError_t build_search_tree(zoom_index ix, void* scratch, size_t scratch_bytes
     return r;
   };
   float* zl = (float*)take(((size_t)1 << d1) * PT_TOP * PZ * 4);
-  uint32_t* cnt = (uint32_t*)take(((size_t)1 << d1) * 4);
+  uint32_t* cnt = (uint32_t*)take(((size_t)1 << d1) * kCountStride * 4);
   uint16_t* leaf = (uint16_t*)take((size_t)n * 2);
   float* stat = (float*)take((size_t)nt * (3 * PZ + 1) * 4);
   uint32_t* rank = (uint32_t*)take((size_t)n * 4);
   uint32_t* hist = (uint32_t*)take((size_t)4 << (d1 + d2));
   const int leaves = 1 << (d1 + d2);
-  // samples: 32 or so for every leaf of either level's tree
-  const int top = std::min(PT_TOP, 32 << d1);
+  // samples: 48 or so for every leaf
   const int64_t m = std::min<int64_t>(n, (int64_t)std::min(1536, 48 << d2) << d1);
-  const DctBasis dct = dct_basis(d->P);
-  cudaError_t e = cudaMemsetAsync(cnt, 0, ((size_t)1 << d1) * 4, st);
+  cudaError_t e = cudaMemsetAsync(cnt, 0, ((size_t)1 << d1) * kCountStride * 4, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(hist, 0, (size_t)leaves * 4, st);
   if (e != cudaSuccess) return e;
   const int smem = (int)sizeof(TreeSmem);
   TreeNode* node1 = (TreeNode*)ix->tree_node1;
   TreeNode* node2 = (TreeNode*)ix->tree_node2;
-#define ZOOM_TREE_A(DD)                                                                                        \
-  do {                                                                                                         \
-    e = cudaFuncSetAttribute(k_tree_top<DD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);                \
-    if (e != cudaSuccess) return e;                                                                            \
-    k_tree_top<DD><<<1, kTreeThreads, smem, st>>>(d->feat, d->dpad, n, dct, d->P * d->P, top, d1, ix->tree_basis, \
-                                                  node1);                                                      \
-    k_tree_sample<DD><<<(unsigned)((m + 127) / 128), 128, 0, st>>>(d->feat, d->dpad, n, m, ix->tree_basis, node1, \
-                                                                   d1, cnt, zl);                               \
-  } while (0)
+#define ZOOM_TREE_A(DD)                                                                                       \
+  k_tree_sample<DD><<<(unsigned)((m + 127) / 128), 128, 0, st>>>(d->feat, d->dpad, n, m, ix->tree_basis, node1, \
+                                                                 d1, cnt, zl)
 #define ZOOM_TREE_B(DD)                                                                                      \
   k_tree_route<DD><<<(unsigned)((n + 127) / 128), 128, 0, st>>>(d->feat, d->dpad, n, ix->tree_basis, node1, node2, \
                                                                 d1, d2, leaf, rank, hist)

@@ -478,8 +478,9 @@ zoom_status zoom_build_index(zoom_dict d, const zoom_lsh_params* lsh, const floa
   zoom_status rc = ZOOM_OK;
   cudaError_t e = cudaMemcpyAsync(ix->alpha, alpha, (size_t)L * k * d->d * 4, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(ix->beta, beta, (size_t)L * k * 4, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess && nt) e = launch_tree_top(ix, st);
   if (e == cudaSuccess)
-    e = launch_hash(d->feat, d->dpad, d->d, N, ix->alpha, ix->beta, L, k, ix->w, ix->dkeys, st);
+    e = launch_hash(d->feat, d->dpad, d->d, N, ix->alpha, ix->beta, L, k, ix->w, ix->dkeys, st, nt > 0);
   if (e == cudaSuccess)
     e = launch_operand(d->feat, d->dpad, d->d, N, ix->nd_rows, 1, 0, ix->dop16, nullptr, st);
   if (e == cudaSuccess)

@@ -135,7 +135,8 @@ cudaError_t launch_dict_gather(const float* const* d_lr_images, const int32_t* d
                                const int32_t* d_hr_w, const int32_t* d_pos, int64_t n, int P, int s,
                                zoom_dict d, cudaStream_t st);
 cudaError_t launch_hash(const float* feat, int dpad, int d, int64_t n, const float* alpha,
-                        const float* beta, int L, int k, float w, uint64_t* keys, cudaStream_t st);
+                        const float* beta, int L, int k, float w, uint64_t* keys, cudaStream_t st,
+                        bool beside = false);   // beside: together with the kernel before it on the stream
 cudaError_t build_csr_tables(zoom_index ix, void* scratch, size_t scratch_bytes, cudaStream_t st);
 size_t csr_scratch_bytes(int64_t n);
 // scratch of build_csr_tables: the radix sort's plus the key compaction's
@@ -144,6 +145,9 @@ size_t csr_build_scratch_bytes(int64_t n, int L);
 // search order of the dictionary (kernels_tree.cu)
 void tree_depths(int64_t n, int* d1, int* d2);
 size_t tree_scratch_bytes(int64_t n);
+// the basis and the first levels: the kernel after it may be launched beside it
+cudaError_t launch_tree_top(zoom_index ix, cudaStream_t st);
+// all the rest
 cudaError_t build_search_tree(zoom_index ix, void* scratch, size_t scratch_bytes, cudaStream_t st);
 
 // per-query steps (kernels_query.cu)

@@ -203,3 +203,13 @@ def test_noise_is_given_up_for_the_dense_filters(prec, n_pairs, h, w):
     ctx.sync_status()
     assert st["n_filter_fallback"] == st["n_queries"] == (h - 4) * (w - 4)
     assert _equal(got, ref)
+
+
+@pytest.mark.parametrize("L,k,n_pairs", [(1, 1, 65_536), (2, 3, 150_001), (16, 16, 65_537)])
+def test_a_hash_shorter_than_the_trees_first_levels(L, k, n_pairs):
+    # the index build launches the two beside each other
+    import paper_1004_3980_gb300 as Z
+    ctx, ix = _build(n_pairs, L=L, k=k)
+    lr = torch.from_numpy(S.make_image(5, 163, 151)).cuda()
+    got = [Z.query(ix, lr, Z.UpscaleParams(K=8, search=search)) for search in (0, 2)]
+    assert _equal(*got)
