@@ -126,7 +126,11 @@ typedef struct {
  * queries, then the SIMT scan for any left; 3 = the split filter alone (then
  * the SIMT scan).  All four give the same neighbours bit for bit.  Precision 1
  * knows 0 and, for 1 to 3 alike, the filter over the whole dictionary; it
- * always uses the tensor cores and needs rerank_mult * K <= 32. */
+ * always uses the tensor cores and needs rerank_mult * K <= 32.
+ * Scratch: a search over the search order takes query lists of at most 2 GiB
+ * and some 300 bytes a query and more (2.6 GB in all for 2M queries on 4M
+ * entries); where the allocator refuses it the whole dictionary is searched, and
+ * where it refuses that search's scratch, in two parts of the queries. */
 typedef struct {
   int32_t K;
   float reg_rel;
@@ -150,9 +154,13 @@ typedef struct {
   int64_t n_padded_queries; /* queries with fewer than K candidates (padded)  */
   int64_t n_fp64_solves;    /* LLE solves that ran in FP64                    */
   int64_t n_exact_match;    /* queries equal to a dictionary entry (one-hot)  */
-  int64_t n_filter_fallback;/* queries the first tensor filter's rerank could
-                              * not settle (searched again: the split filter
-                              * after the single-term one, else the SIMT scan) */
+  int64_t n_filter_fallback;/* queries the first search could not settle: the
+                              * dense search's first filter (searched again: the
+                              * split filter after the single-term one, else the
+                              * SIMT scan), or the search over the search order
+                              * (searched again: the dense filters).  The latter
+                              * count can differ a little from run to run; the
+                              * neighbours do not. */
   double ms_total;          /* device time of the last call (CUDA events)     */
   /* per-stage device milliseconds of the last call, when stage timing is on:
    * [0] features, [1] hashing, [2] bin lookup, [3] neighbour search,
@@ -255,7 +263,9 @@ zoom_status zoom_sample_positions(uint64_t seed, int32_t n_images, const int32_t
  * [L*k] offsets in [0, w).  Both NULL: the library draws them from
  * lsh->seed and lsh->proj_dist (zoom_lsh_draws).  Builds, per table, the
  * bucket key of every entry and a CSR of its bins (keys radix-sorted on the
- * device).  Errors: INVALID_ARG for parameters out of range or only one of
+ * device).  Indexes without a cap over 65,536 to 8,388,608 entries with features
+ * of at most 25 values also keep a search order for the automatic search (132
+ * bytes an entry); without room for it the index goes without.  Errors: INVALID_ARG for parameters out of range or only one of
  * alpha and beta given. */
 zoom_status zoom_build_index(zoom_dict d, const zoom_lsh_params* lsh, const float* alpha,
                              const float* beta, void* stream, zoom_index* out);

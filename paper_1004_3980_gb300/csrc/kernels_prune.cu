@@ -325,13 +325,15 @@ __global__ void k_radius(const float* __restrict__ ld, int MC, int r, const floa
 // super tiles' boxes, then against their tiles' boxes; the tiles that are
 // left queue up, and 32 of them at a time are tested against every query, one
 // tile per lane with its box in registers and the queries' coordinates
-// broadcast from shared memory.  Bound by the issue of that test (24 paired
-// FP16 operations of about 32 instructions a pair); with a query per lane and
-// the boxes broadcast it took 45 and waited for every box.  A lane ends up
+// broadcast from shared memory.  Bound by that test, half by its issue and half by
+// its latency (24 paired FP16 operations of about 32 instructions a pair; 280 x
+// 280 queries on 300,000 entries: 53 % of the issue slots, 17 % of the warps
+// that fit, no memory above 36 %); with a query per lane and the boxes
+// broadcast it took 45 and waited for every box.  A lane ends up
 // with the mask of the queries that need its tile: one round of atomics gives
 // the 32 masks their places in the tiles' lists.  The pairs of the round are
 // counted, too: past `give_up` the warps stop.  2.06M queries on 4M entries:
-// 20.8 ms in 32 rounds; 258,064 on 1M: 1.21 ms.
+// 20.4 ms in 32 rounds; 258,064 on 1M: 1.19 ms.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_visit(const uint4* __restrict__ qz, const float* __restrict__ vis,
                                                int nslab, const uint4* __restrict__ box, int nt,
@@ -560,9 +562,12 @@ __global__ void k_steps(const uint32_t* __restrict__ tcnt, int nt, const uint32_
 // epilogue cost about 350 cycles each.)  Bound by the hand-offs between the
 // roles: with two 128-column accumulators a parity, one read while the other
 // is computed, a step took 1250 cycles against 1080 here -- each hand-off costs
-// the slowest of eight warps some 400 cycles whatever it covers.  2.06M queries
-// on 4M entries (BF16): 34.4 ms where the dense filter took 394 ms; 258,064 on
-// 1M (FP16): 2.10 ms and 13.1 ms.
+// the slowest of eight warps some 400 cycles whatever it covers; the counters have
+// nothing near its limit (280 x 280 queries on 300,000 entries: tensor pipe 22 %
+// of the cycles, issue slots 55 %, L1 and shared memory 49 %, L2 and DRAM below
+// 10 %).  2.06M queries
+// on 4M entries (BF16): 34.1 ms where the dense filter took 394 ms; 258,064 on
+// 1M (FP16): 2.11 ms and 13.1 ms.
 // ---------------------------------------------------------------------------
 constexpr int kHits = PT_ROWS / 64;   // records per lane and step, at most: 128 columns
 constexpr int kEpi = 16;              // epilogue warps
